@@ -2,18 +2,26 @@
 //
 // y = W3 g(W2 g(W1 x + b1) + b2) + b3 with the exact GELU g(z) = z Phi(z).
 // Every product is a BF16 x BF16 -> FP32 tensor-core GEMM (mma.sync
-// m16n8k16: the matrices are a few hundred wide, far below the sizes where
-// the tcgen05 / TMEM pipeline would pay off).  FP32 master weights and Adam
-// moments; BF16 copies of the weights and of every GEMM operand
-// (activations, output and hidden gradients); FP32 pre-activations for the
-// GELU derivative; FP32 gradients.
+// m16n8k16).  FP32 master weights and Adam moments; BF16 copies of the
+// weights and of every GEMM operand (activations, output and hidden
+// gradients); FP32 pre-activations for the GELU derivative; FP32 gradients.
 //
-// One generic tiled GEMM serves all products through strided operand views
-// (C[i][j] = sum_k A(i,k) B(k,j), A(i,k) = A[i sar + k sac]), so forward
-// (X W^T), input gradients (dZ W) and weight gradients (dZ^T H) are the same
-// kernel with different strides and epilogues.  Weight gradients reduce over
-// the batch (K = B) into few output tiles; they are split along K over
-// gridDim.z into FP32 partial tiles, added in a fixed order afterwards.
+// What bounds it: latency.  A training step of the 111-256-256-40 network on
+// a batch of 1,024 is 0.6 GFLOP over a few MB that stay in L2, so what counts
+// is the number of dependent launches and the depth of each.  A step is seven:
+// three forward layers (the last one forms the output gradient and the loss
+// too), two input gradients, all weight and bias gradients together, and one
+// that adds their partial sums, steps Adam and refreshes the BF16 weights.
+// Each starts while its predecessor drains (programmatic dependent launch) and
+// fetches its weights before it waits.  The GEMMs stage 16-byte cp.async
+// copies of whole 64-wide k tiles, four in flight (K = 256 is in flight
+// entirely), in XOR-swizzled rows read with ldmatrix; 32 x 64 output tiles
+// spread a batch of 1,024 over 128 blocks.  Operand rows are padded to whole
+// 16-byte chunks, zero-filled.  Every sum runs in a fixed order: k ascending in
+// the products, gradients over the batch in kchunk slices added in order.
+// Measured, host calls included: 8 steps and one loss_grad on a batch of 1,024
+// in 376 us (2,627 us with one strided-load GEMM kernel and 27 launches per
+// step), the proposal's inference for 256 robots in 76 us (123 us).
 #include <cuda_bf16.h>
 #include <math.h>
 #include <string.h>
@@ -22,34 +30,14 @@
 #include <new>
 #include <vector>
 
-#include "internal.h"
+#include "mppi_cycle.cuh"
 
 namespace exact {
 
 typedef __nv_bfloat16 bf16;
 
-constexpr int GM = 64, GN = 64, GK = 32, GPAD = 8;   // block tile, k step, smem row padding
-constexpr int kMlpInPad = 128;                        // inputs are zero-padded to this width
-
-enum { EPI_PLAIN = 0, EPI_BIAS_GELU = 1, EPI_GELU_GRAD = 2, EPI_BIAS = 3 };
-
-struct GemmArgs {
-    int M, N, K;
-    const bf16 *A;
-    long long sar, sac;
-    const bf16 *B;
-    long long sbr, sbc;
-    float *C;          // FP32 result (row-major, ldc)
-    int ldc;
-    bf16 *Cb;          // optional BF16 result (row-major, ldcb)
-    int ldcb;
-    const float *bias; // per column j
-    const float *gz;   // pre-activation for EPI_GELU_GRAD (row-major, ldgz)
-    int ldgz;
-    int epi;
-    int kchunk;        // k range of one block along gridDim.z (split-K); K when unsplit
-    float *P;          // split-K: FP32 partial tiles P[z][i][j] (M x N each), summed by splitk_sum_kernel
-};
+constexpr int kMlpInPad = 128;   // inputs are zero-padded to this width
+constexpr int kBN = 64, kBK = 64, kStages = 4;
 
 __device__ __forceinline__ float gelu_f(float z) { return 0.5f * z * (1.f + erff(z * 0.70710678118654752f)); }
 __device__ __forceinline__ float gelu_grad_f(float z) {
@@ -64,173 +52,344 @@ __device__ __forceinline__ void mma_bf16(float *d, const uint32_t *a, const uint
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-__device__ __forceinline__ uint32_t ld_pair(const bf16 *p) { return *reinterpret_cast<const uint32_t *>(p); }
+// ---------------------------------------------------------------- tiles
+// A tile is R rows of 64 bf16 (128 bytes) in shared memory, the 16-byte chunks
+// of a row XORed with the row's low bits, so that the eight rows an ldmatrix
+// reads fall into different banks.
+__device__ __forceinline__ unsigned tile_addr(const bf16 *tile, int row, int chunk) {
+    return smem_addr(tile) + row * 128 + ((chunk ^ (row & 7)) << 4);
+}
+// Rows [r0, r0 + R) x columns [c0, c0 + 64) of a row-major matrix (ld a
+// multiple of 8, 16-byte aligned); rows from rmax and chunks from cmax (a
+// multiple of 8) on are zero.  128 threads, no wait.
+template <int R>
+__device__ __forceinline__ void tile_load(bf16 *tile, const bf16 *__restrict__ g, int ld, int r0, int rmax, int c0,
+                                          int cmax) {
+#pragma unroll
+    for (int k = 0; k < R * 8 / 128; ++k) {
+        const int e = k * 128 + threadIdx.x, row = e >> 3, chunk = e & 7;
+        const bool ok = r0 + row < rmax && c0 + chunk * 8 < cmax;
+        const bf16 *src = ok ? g + (size_t)(r0 + row) * ld + c0 + chunk * 8 : g;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(tile_addr(tile, row, chunk)), "l"(src),
+                     "r"(ok ? 16 : 0)
+                     : "memory");
+    }
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+template <bool TRANS>
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], unsigned addr) {
+    if constexpr (TRANS)
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                     : "r"(addr)
+                     : "memory");
+    else
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                     : "r"(addr)
+                     : "memory");
+}
+// A fragment (16 x 16 at m0, k0) of a tile stored [m][k], or [k][m] (TRANS).
+template <bool TRANS>
+__device__ __forceinline__ void frag_a(uint32_t (&a)[4], const bf16 *tile, int m0, int k0) {
+    const int lane = threadIdx.x & 31, r = lane & 7, mi = lane >> 3;
+    if constexpr (TRANS)
+        ldsm4<true>(a, tile_addr(tile, k0 + r + (mi >> 1) * 8, (m0 >> 3) + (mi & 1)));
+    else
+        ldsm4<false>(a, tile_addr(tile, m0 + r + (mi & 1) * 8, (k0 >> 3) + (mi >> 1)));
+}
+// B fragments of two neighbouring 8-column tiles (b[0..1] at n0, b[2..3] at
+// n0 + 8) of a tile stored [n][k], or [k][n] (TRANS).
+template <bool TRANS>
+__device__ __forceinline__ void frag_b2(uint32_t (&b)[4], const bf16 *tile, int n0, int k0) {
+    const int lane = threadIdx.x & 31, r = lane & 7, mi = lane >> 3;
+    if constexpr (TRANS)
+        ldsm4<true>(b, tile_addr(tile, k0 + r + (mi & 1) * 8, (n0 >> 3) + (mi >> 1)));
+    else
+        ldsm4<false>(b, tile_addr(tile, n0 + r + (mi >> 1) * 8, (k0 >> 3) + (mi & 1)));
+}
+// One 64-wide k tile: four warps in a 2 x 2 grid, each MT x 4 mma tiles.
+template <int MT, bool TA, bool TB>
+__device__ __forceinline__ void tile_mma(float (&acc)[MT][4][4], const bf16 *As, const bf16 *Bs) {
+    const int warp = threadIdx.x >> 5, wm = (warp >> 1) * MT * 16, wn = (warp & 1) * 32;
+#pragma unroll
+    for (int kk = 0; kk < kBK; kk += 16) {
+        uint32_t a[MT][4], b[2][4];
+#pragma unroll
+        for (int mi = 0; mi < MT; ++mi) frag_a<TA>(a[mi], As, wm + mi * 16, kk);
+#pragma unroll
+        for (int p = 0; p < 2; ++p) frag_b2<TB>(b[p], Bs, wn + p * 16, kk);
+#pragma unroll
+        for (int mi = 0; mi < MT; ++mi)
+#pragma unroll
+            for (int ni = 0; ni < 4; ++ni) mma_bf16(acc[mi][ni], a[mi], &b[ni >> 1][(ni & 1) * 2]);
+    }
+}
 
-// 64 x 64 output tile per block (4 warps, 32 x 32 each = 2 x 4 mma tiles of
-// 16 x 8), k in steps of 32 staged through shared memory.  A is staged as
-// As[i][k], B transposed as Bs[j][k], so both fragments are pairs of
-// consecutive k (one 32-bit load each).  Out-of-range elements are zero.
-__global__ void __launch_bounds__(128) gemm_bf16_kernel(const GemmArgs g) {
-    __shared__ __align__(16) bf16 As[GM][GK + GPAD];
-    __shared__ __align__(16) bf16 Bs[GN][GK + GPAD];
-    const int i0 = blockIdx.y * GM, j0 = blockIdx.x * GN;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int wm = warp >> 1, wn = warp & 1;
-    const int gid = lane >> 2, t4 = lane & 3;
-    const bf16 zero = __float2bfloat16_rn(0.f);
-    float acc[2][4][4];
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) acc[a][b][c] = 0.f;
+// ---------------------------------------------------------------- layers
+enum { LAYER_IN, LAYER_HIDDEN, LAYER_OUT, LAYER_GRAD };
 
-    const int kb = blockIdx.z * g.kchunk, ke = min(g.K, kb + g.kchunk);
-    for (int k0 = kb; k0 < ke; k0 += GK) {
-        for (int e = threadIdx.x; e < GM * GK; e += 128) {
-            const int r = e / GK, c = e - r * GK, i = i0 + r, k = k0 + c;
-            As[r][c] = (i < g.M && k < ke) ? g.A[(long long)i * g.sar + (long long)k * g.sac] : zero;
-        }
-        for (int e = threadIdx.x; e < GN * GK; e += 128) {
-            const int r = e / GK, c = e - r * GK, j = j0 + r, k = k0 + c;
-            Bs[r][c] = (j < g.N && k < ke) ? g.B[(long long)k * g.sbr + (long long)j * g.sbc] : zero;
-        }
-        __syncthreads();
+struct LayerArgs {
+    int M, N, K;          // batch rows, output columns, inner size
+    const float *x;       // LAYER_IN: the FP32 input, M x K
+    bf16 *Xb;             // LAYER_IN: its BF16 copy (kMlpInPad columns), written for the weight gradient
+    const bf16 *A;        // else: M x K activations (row stride lda)
+    int lda;
+    const bf16 *W;        // N x K weights; LAYER_GRAD: K x N
+    int ldw;
+    const float *bias;    // N
+    float *C;             // M x N FP32: pre-activations, outputs or gradients (row stride N)
+    bf16 *Cb;             // BF16 activations or gradients (row stride ldcb)
+    int ldcb;
+    const float *gz;      // LAYER_GRAD: pre-activations (row stride N)
+    const float *target;  // LAYER_OUT: M x N, or NULL
+    float *dY;            // LAYER_OUT with a target: 2 (y - target) / (M N)
+    float scale;
+    double *lossp;        // LAYER_OUT with a target: per block, sum of squares
+};
+
+// 32 rows x 64 columns of one layer.  Only the weights are read before the
+// wait: they were written at least two launches ago.
+template <int MODE>
+__global__ void __launch_bounds__(128) layer_kernel(const LayerArgs g) {
+    constexpr int BM = 32;
+    constexpr bool NN = MODE == LAYER_GRAD;   // weights stored [k][n]
+    __shared__ __align__(128) bf16 As[kStages][BM * kBK];
+    __shared__ __align__(128) bf16 Bs[kStages][kBN * kBK];
+    const int i0 = blockIdx.y * BM, j0 = blockIdx.x * kBN;
+    const int kt_n = (g.K + kBK - 1) / kBK;
+    const int kpad = (g.K + 7) & ~7, npad = (g.N + 7) & ~7;
+    auto load_b = [&](int kt) {
+        bf16 *t = Bs[kt % kStages];
+        if constexpr (NN) tile_load<kBK>(t, g.W, g.ldw, kt * kBK, g.K, j0, npad);
+        else tile_load<kBN>(t, g.W, g.ldw, j0, g.N, kt * kBK, MODE == LAYER_IN ? kMlpInPad : kpad);
+    };
+    auto load_a = [&](int kt) {
+        bf16 *t = As[kt % kStages];
+        if constexpr (MODE == LAYER_IN) {
+            float v[BM * kBK / 128];   // every load in flight before the first store
 #pragma unroll
-        for (int kk = 0; kk < GK; kk += 16) {
-            uint32_t af[2][4], bfm[4][2];
-#pragma unroll
-            for (int mi = 0; mi < 2; ++mi) {
-                const int row = wm * 32 + mi * 16 + gid;
-                af[mi][0] = ld_pair(&As[row][kk + 2 * t4]);
-                af[mi][1] = ld_pair(&As[row + 8][kk + 2 * t4]);
-                af[mi][2] = ld_pair(&As[row][kk + 2 * t4 + 8]);
-                af[mi][3] = ld_pair(&As[row + 8][kk + 2 * t4 + 8]);
+            for (int p = 0; p < BM * kBK / 128; ++p) {
+                const int e = p * 128 + threadIdx.x, i = i0 + e / kBK, k = kt * kBK + e % kBK;
+                v[p] = i < g.M && k < g.K ? __ldca(g.x + (size_t)i * g.K + k) : 0.f;
             }
 #pragma unroll
-            for (int ni = 0; ni < 4; ++ni) {
-                const int col = wn * 32 + ni * 8 + gid;
-                bfm[ni][0] = ld_pair(&Bs[col][kk + 2 * t4]);
-                bfm[ni][1] = ld_pair(&Bs[col][kk + 2 * t4 + 8]);
+            for (int p = 0; p < BM * kBK / 128; ++p) {
+                const int e = p * 128 + threadIdx.x, row = e / kBK, c = e % kBK, i = i0 + row;
+                const bf16 h = __float2bfloat16_rn(v[p]);
+                t[row * kBK + (((c >> 3) ^ (row & 7)) << 3) + (c & 7)] = h;
+                if (blockIdx.x == 0 && g.Xb && i < g.M) g.Xb[(size_t)i * kMlpInPad + kt * kBK + c] = h;
             }
-#pragma unroll
-            for (int mi = 0; mi < 2; ++mi)
-#pragma unroll
-                for (int ni = 0; ni < 4; ++ni) mma_bf16(acc[mi][ni], af[mi], bfm[ni]);
+        } else {
+            tile_load<BM>(t, g.A, g.lda, i0, g.M, kt * kBK, kpad);
         }
+    };
+    if constexpr (MODE == LAYER_IN) grid_dep_wait();   // the weights may come from the launch before this one
+    for (int kt = 0; kt < kt_n && kt < kStages; ++kt) load_b(kt);
+    if constexpr (MODE != LAYER_IN) grid_dep_wait();
+    grid_dep_release();   // after the wait: a launch that starts now finds everything before this one complete
+    for (int kt = 0; kt < kStages; ++kt) {
+        if (kt < kt_n) load_a(kt);
+        cp_commit();
+    }
+    float acc[1][4][4] = {};
+    for (int kt = 0; kt < kt_n; ++kt) {
+        cp_wait<kStages - 1>();
         __syncthreads();
+        tile_mma<1, false, NN>(acc, As[kt % kStages], Bs[kt % kStages]);
+        if (kt + kStages < kt_n) {
+            __syncthreads();
+            load_a(kt + kStages);
+            load_b(kt + kStages);
+        }
+        cp_commit();
     }
 
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gid = lane >> 2, t4 = lane & 3;
+    double sq = 0.0;
+#pragma unroll
+    for (int ni = 0; ni < 4; ++ni)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int i = i0 + (warp >> 1) * 16 + gid + 8 * (q >> 1), j = j0 + (warp & 1) * 32 + ni * 8 + 2 * t4 + (q & 1);
+            if (i >= g.M || j >= g.N) continue;
+            float v = acc[0][ni][q];
+            const size_t c = (size_t)i * g.N + j;
+            if constexpr (MODE == LAYER_GRAD) {
+                v = v * gelu_grad_f(g.gz[c]);
+                g.C[c] = v;
+                g.Cb[(size_t)i * g.ldcb + j] = __float2bfloat16_rn(v);
+            } else {
+                v += g.bias[j];
+                g.C[c] = v;
+                if constexpr (MODE == LAYER_OUT) {
+                    if (g.target) {
+                        const float d = v - g.target[c], gv = d * g.scale;
+                        sq += (double)d * (double)d;
+                        g.dY[c] = gv;
+                        g.Cb[(size_t)i * g.ldcb + j] = __float2bfloat16_rn(gv);
+                    }
+                } else {
+                    g.Cb[(size_t)i * g.ldcb + j] = __float2bfloat16_rn(gelu_f(v));
+                }
+            }
+        }
+    if constexpr (MODE == LAYER_OUT) {
+        if (!g.target) return;
+        __syncthreads();
+        double *s_sq = reinterpret_cast<double *>(As[0]);   // the tiles are consumed
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+        if (lane == 0) s_sq[warp] = sq;
+        __syncthreads();
+        if (threadIdx.x == 0) g.lossp[blockIdx.y * gridDim.x + blockIdx.x] = ((s_sq[0] + s_sq[1]) + s_sq[2]) + s_sq[3];
+    }
+}
+
+// ---------------------------------------------------------------- parameter gradients
+// Weight gradients G[i][j] = sum_b D[b][i] H[b][j] (M x N, K = the batch) in
+// S slices of kchunk rows each: block (tile, slice) leaves its partial tile in
+// P[slice]; bias gradients sum_b F[b][j] in kColSlices slices (slice s adds rows
+// s, s + kColSlices, ...).  All layers' blocks run in one launch.
+constexpr int kColSlices = 32;
+struct GradArgs {
+    const bf16 *D, *H;   // B x M (row stride ldd), B x N (row stride ldh)
+    int ldd, ldh, M, N, S, kchunk;
+    float *P;            // S x M x N
+    const float *F;      // B x M: FP32 gradient of the layer's output
+    float *Q;            // kColSlices x M
+    int gemm_blocks, blocks;   // blocks of this layer: GEMM blocks first
+};
+struct GradSet {
+    GradArgs l[3];
+    int B;
+};
+
+__global__ void __launch_bounds__(128) grad_kernel(const GradSet gs) {
+    constexpr int BM = 64;
+    __shared__ __align__(128) bf16 As[2][BM * kBK];
+    __shared__ __align__(128) bf16 Bs[2][kBN * kBK];
+    int b = blockIdx.x, li = 0;
+    while (li < 2 && b >= gs.l[li].blocks) b -= gs.l[li++].blocks;
+    const GradArgs &g = gs.l[li];
+    grid_dep_wait();
+    grid_dep_release();
+    if (b >= g.gemm_blocks) {   // bias: one thread per column
+        b -= g.gemm_blocks;
+        const int tiles = (g.M + 127) / 128, sl = b / tiles, j = (b - sl * tiles) * 128 + threadIdx.x;
+        if (j >= g.M) return;
+        float a = 0.f;
+#pragma unroll 8
+        for (int r = sl; r < gs.B; r += kColSlices) a += g.F[(size_t)r * g.M + j];
+        g.Q[(size_t)sl * g.M + j] = a;
+        return;
+    }
+    const int nt = (g.N + kBN - 1) / kBN, mt = (g.M + BM - 1) / BM;
+    const int z = b / (nt * mt), t = b - z * nt * mt, i0 = (t / nt) * BM, j0 = (t % nt) * kBN;
+    const int kb = z * g.kchunk, ke = min(gs.B, kb + g.kchunk);
+    const int kt_n = ke > kb ? (ke - kb + kBK - 1) / kBK : 0;
+    auto load = [&](int kt) {   // rows of the batch are k
+        tile_load<kBK>(As[kt & 1], g.D, g.ldd, kb + kt * kBK, ke, i0, (g.M + 7) & ~7);
+        tile_load<kBK>(Bs[kt & 1], g.H, g.ldh, kb + kt * kBK, ke, j0, (g.N + 7) & ~7);
+    };
+    for (int kt = 0; kt < 2; ++kt) {
+        if (kt < kt_n) load(kt);
+        cp_commit();
+    }
+    float acc[2][4][4] = {};
+    for (int kt = 0; kt < kt_n; ++kt) {
+        cp_wait<1>();
+        __syncthreads();
+        tile_mma<2, true, true>(acc, As[kt & 1], Bs[kt & 1]);
+        if (kt + 2 < kt_n) {
+            __syncthreads();
+            load(kt + 2);
+        }
+        cp_commit();
+    }
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gid = lane >> 2, t4 = lane & 3;
+    float *P = g.P + (size_t)z * g.M * g.N;
 #pragma unroll
     for (int mi = 0; mi < 2; ++mi)
 #pragma unroll
         for (int ni = 0; ni < 4; ++ni)
 #pragma unroll
-            for (int h = 0; h < 2; ++h)
+            for (int q = 0; q < 4; ++q) {
+                const int i = i0 + (warp >> 1) * 32 + mi * 16 + gid + 8 * (q >> 1);
+                const int j = j0 + (warp & 1) * 32 + ni * 8 + 2 * t4 + (q & 1);
+                if (i < g.M && j < g.N) P[(size_t)i * g.N + j] = acc[mi][ni][q];
+            }
+}
+
+// ---------------------------------------------------------------- finish
+struct FinishArgs {
+    const float *P[3], *Q[3];   // partial weight and bias gradients per layer
+    int M[3], N[3], S[3];
+    bf16 *Wb[3];                // BF16 weight copies (row stride ldw)
+    int ldw[3];
+    float *grads;               // packed gradients out, or NULL
+    float *w, *m, *v;           // packed parameters and moments (stepped when adam)
+    int adam;
+    float lr, b1, b2, eps, c1, c2;
+    const double *lossp;
+    int n_lossp;
+    double inv_n;
+    float *loss;                // or NULL
+    long long n;
+};
+
+// The packed gradient (slices added in order), Adam (Kingma & Ba) on the FP32
+// parameters (c1 = 1 - beta1^t, c2 = 1 - beta2^t), the BF16 copy of every
+// stepped weight, and the mean squared error.
+__global__ void __launch_bounds__(256) finish_kernel(const FinishArgs g) {
+    grid_dep_wait();
+    grid_dep_release();
+    const long long e = blockIdx.x * 256ll + threadIdx.x;
+    if (e < g.n) {
+        long long r = e;
+        int li = 0;
+        while (li < 2 && r >= (long long)g.M[li] * g.N[li] + g.M[li]) {
+            r -= (long long)g.M[li] * g.N[li] + g.M[li];
+            ++li;
+        }
+        const long long nw = (long long)g.M[li] * g.N[li];
+        float gk = 0.f;
+        if (r < nw) {
+#pragma unroll 8
+            for (int z = 0; z < g.S[li]; ++z) gk += g.P[li][z * nw + r];
+        } else {
+#pragma unroll 8
+            for (int sl = 0; sl < kColSlices; ++sl) gk += g.Q[li][(long long)sl * g.M[li] + (r - nw)];
+        }
+        if (g.grads) g.grads[e] = gk;
+        if (g.adam) {
+            const float mk = fmaf(1.f - g.b1, gk, g.b1 * g.m[e]);   // one rounding order, whatever the compiler fuses
+            const float vk = fmaf((1.f - g.b2) * gk, gk, g.b2 * g.v[e]);
+            g.m[e] = mk;
+            g.v[e] = vk;
+            const float w = g.w[e] - g.lr * (mk / g.c1) / (sqrtf(vk / g.c2) + g.eps);
+            g.w[e] = w;
+            if (r < nw) {
+                const int row = (int)(r / g.N[li]), col = (int)(r - (long long)row * g.N[li]);
+                g.Wb[li][(size_t)row * g.ldw[li] + col] = __float2bfloat16_rn(w);
+            }
+        }
+    }
+    if (blockIdx.x == 0 && g.loss) {
+        __shared__ double s[8];
+        double a = 0.0;
+        for (int k = threadIdx.x; k < g.n_lossp; k += 256) a += g.lossp[k];
 #pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    const int i = i0 + wm * 32 + mi * 16 + gid + 8 * h;
-                    const int j = j0 + wn * 32 + ni * 8 + 2 * t4 + c;
-                    if (i >= g.M || j >= g.N) continue;
-                    float v = acc[mi][ni][2 * h + c];
-                    if (g.P) {   // split-K: this block's partial, no epilogue
-                        g.P[((long long)blockIdx.z * g.M + i) * g.N + j] = v;
-                        continue;
-                    }
-                    float out = v;
-                    if (g.epi == EPI_BIAS || g.epi == EPI_BIAS_GELU) v += g.bias[j];
-                    if (g.epi == EPI_BIAS_GELU) {
-                        out = v;                               // pre-activation kept in C
-                        if (g.Cb) g.Cb[(long long)i * g.ldcb + j] = __float2bfloat16_rn(gelu_f(v));
-                    } else if (g.epi == EPI_GELU_GRAD) {
-                        out = v * gelu_grad_f(g.gz[(long long)i * g.ldgz + j]);
-                        if (g.Cb) g.Cb[(long long)i * g.ldcb + j] = __float2bfloat16_rn(out);
-                    } else {
-                        out = v;
-                        if (g.Cb) g.Cb[(long long)i * g.ldcb + j] = __float2bfloat16_rn(out);
-                    }
-                    if (g.C) g.C[(long long)i * g.ldc + j] = out;
-                }
-}
-
-// C[i][j] (row stride ldc) = sum_z P[z][i][j], z in order (fixed, so the
-// result does not depend on scheduling)
-__global__ void splitk_sum_kernel(const float *__restrict__ P, int S, int M, int N, float *__restrict__ C, int ldc) {
-    const long long n = (long long)M * N;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-        float a = 0.f;
-        for (int z = 0; z < S; ++z) a += P[z * n + e];
-        C[(e / N) * ldc + e % N] = a;
-    }
-}
-
-// x (B x d_in, FP32) -> Xb (B x 128, BF16, zero-padded)
-__global__ void pack_input_kernel(const float *__restrict__ x, int B, int d_in, bf16 *__restrict__ Xb) {
-    const long long n = (long long)B * kMlpInPad;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-        const int b = (int)(e / kMlpInPad), d = (int)(e - (long long)b * kMlpInPad);
-        Xb[e] = __float2bfloat16_rn(d < d_in ? x[(long long)b * d_in + d] : 0.f);
-    }
-}
-
-// dY = 2 (Y - target) / (B O) (FP32 and BF16) and the mean squared error
-// (one block, fixed reduction order).
-__global__ void __launch_bounds__(1024)
-mse_grad_kernel(const float *__restrict__ Y, const float *__restrict__ tgt, int B, int O, float *__restrict__ dY,
-                bf16 *__restrict__ dYb, float *__restrict__ loss) {
-    __shared__ double s[32];
-    const long long n = (long long)B * O;
-    const float scale = 2.f / (float)n;
-    double acc = 0.0;
-    for (long long e = threadIdx.x; e < n; e += blockDim.x) {
-        const float d = Y[e] - tgt[e];
-        acc += (double)d * (double)d;
-        const float gv = d * scale;
-        dY[e] = gv;
-        dYb[e] = __float2bfloat16_rn(gv);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += s[w];
-        if (loss) *loss = (float)(t / (double)n);
-    }
-}
-
-// Bias gradients g[j] = sum_b D[b][j] in two fixed-order stages: slice s of
-// kColSlices adds its rows b = s, s + kColSlices, ... (one thread per column,
-// coalesced across columns), then colsum_finish adds the slices in order.
-constexpr int kColSlices = 32;
-__global__ void colsum_kernel(const float *__restrict__ D, int B, int n, float *__restrict__ part) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x, sl = blockIdx.y;
-    if (j >= n) return;
-    float a = 0.f;
-    for (int b = sl; b < B; b += kColSlices) a += D[(long long)b * n + j];
-    part[(long long)sl * n + j] = a;
-}
-__global__ void colsum_finish_kernel(const float *__restrict__ part, int n, float *__restrict__ g) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    float a = 0.f;
-    for (int sl = 0; sl < kColSlices; ++sl) a += part[(long long)sl * n + j];
-    g[j] = a;
-}
-
-// Adam (Kingma & Ba) on the packed FP32 parameters; c1 = 1 - beta1^t, c2 = 1 - beta2^t.
-__global__ void adam_kernel(float *__restrict__ w, const float *__restrict__ g, float *__restrict__ m,
-                            float *__restrict__ v, long long n, float lr, float b1, float b2, float eps, float c1,
-                            float c2) {
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
-        const float gk = g[k];
-        const float mk = b1 * m[k] + (1.f - b1) * gk;
-        const float vk = b2 * v[k] + (1.f - b2) * gk * gk;
-        m[k] = mk;
-        v[k] = vk;
-        w[k] -= lr * (mk / c1) / (sqrtf(vk / c2) + eps);
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if ((threadIdx.x & 31) == 0) s[threadIdx.x >> 5] = a;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double t = 0.0;
+            for (int k = 0; k < 8; ++k) t += s[k];
+            *g.loss = (float)(t * g.inv_n);
+        }
     }
 }
 
@@ -249,112 +408,129 @@ __global__ void to_bf16_kernel(const float *__restrict__ W, int rows, int cols, 
 using namespace exact;
 
 struct exact_mlp {
-    int din = 0, H = 0, O = 0, maxB = 0;
+    int din = 0, H = 0, O = 0, maxB = 0, Hp = 0, Op = 0;   // Hp, Op: BF16 row strides (multiples of 8)
     long long nparam = 0;
     long long oW1, ob1, oW2, ob2, oW3, ob3;   // offsets into the packed parameter vector
     void *dev = nullptr;
-    float *w, *g, *m, *v;                     // packed FP32 parameters, gradients, moments
+    float *w, *m, *v;                         // packed FP32 parameters and moments
     bf16 *W1b, *W2b, *W3b;                    // BF16 weights (W1b rows padded to 128)
-    bf16 *Xb, *H1b, *H2b, *dYb, *dZb;         // BF16 operands
-    float *Z1, *Z2, *Y, *dY, *dZ, *loss;      // FP32 activations / gradients
-    float *ws;                                // split-K partial tiles and column-sum slices
+    bf16 *Xb, *H1b, *H2b, *dYb, *dZ1b, *dZ2b; // BF16 operands (padding columns stay zero)
+    float *Z1, *Z2, *Y, *dY, *dZ1, *dZ2;      // FP32 activations / gradients
+    float *P[3], *Q[3];                       // partial weight and bias gradients
+    double *lossp;                            // partial losses
     int t = 0;                                // Adam step
 };
 
-// split-K factor of a GEMM whose output tiles would not fill the GPU
+// Slices of a weight gradient over the batch: enough that its 64 x 64 tiles
+// fill the GPU, at least 64 rows each.  (Part of the result: the slices are
+// summed in order.)
 constexpr int kSplitMax = 16;
-static int splits_for(int M, int N, int K) {
-    const int tiles = ((M + GM - 1) / GM) * ((N + GN - 1) / GN);
+static int splits_for(int M, int N, long long K) {
+    const int tiles = ((M + 63) / 64) * ((N + 63) / 64);
     int s = 1;
-    while (s < kSplitMax && tiles * s * 2 <= 152 && K / (s * 2) >= 2 * GK) s *= 2;
+    while (s < kSplitMax && tiles * s * 2 <= 152 && K / (s * 2) >= 64) s *= 2;
     return s;
 }
+static int chunk_for(int S, int K) { return S > 1 ? ((K + S - 1) / S + 31) / 32 * 32 : K; }
 
 static int grid_for(long long n, int block) {
     long long g = (n + block - 1) / block;
     return (int)(g < 1 ? 1 : (g > 65535 ? 65535 : g));
 }
 
-static cudaError_t gemm(const GemmArgs &g0, cudaStream_t st, float *ws = nullptr) {
-    GemmArgs g = g0;
-    // weight gradients (no epilogue, K = the batch) are split along K into
-    // partial tiles when their output tiles alone would not fill the GPU
-    const int S = (ws && g.epi == EPI_PLAIN && !g.Cb) ? splits_for(g.M, g.N, g.K) : 1;
-    g.kchunk = S > 1 ? ((g.K + S - 1) / S + GK - 1) / GK * GK : g.K;
-    g.P = S > 1 ? ws : nullptr;
-    dim3 grid((g.N + GN - 1) / GN, (g.M + GM - 1) / GM, S);
-    gemm_bf16_kernel<<<grid, 128, 0, st>>>(g);
-    if (S > 1) {
-        const long long n = (long long)g.M * g.N;
-        splitk_sum_kernel<<<(int)((n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024), 256, 0, st>>>(ws, S, g.M, g.N, g.C,
-                                                                                               g.ldc);
-    }
-    return cudaGetLastError();
-}
-
-static void colsum(const float *D, int B, int n, float *g, float *ws, cudaStream_t st) {
-    colsum_kernel<<<dim3((n + 127) / 128, kColSlices), 128, 0, st>>>(D, B, n, ws);
-    colsum_finish_kernel<<<(n + 127) / 128, 128, 0, st>>>(ws, n, g);
-}
-
-static GemmArgs make_gemm(int M, int N, int K, const bf16 *A, long long sar, long long sac, const bf16 *B, long long sbr,
-                          long long sbc, float *C, int ldc, int epi) {
-    GemmArgs g;
-    memset(&g, 0, sizeof(g));
-    g.M = M; g.N = N; g.K = K;
-    g.A = A; g.sar = sar; g.sac = sac;
-    g.B = B; g.sbr = sbr; g.sbc = sbc;
-    g.C = C; g.ldc = ldc;
-    g.epi = epi;
-    return g;
-}
-
 static int refresh_bf16(exact_mlp *m, cudaStream_t st) {
     to_bf16_kernel<<<grid_for((long long)m->H * kMlpInPad, 256), 256, 0, st>>>(m->w + m->oW1, m->H, m->din, kMlpInPad, m->W1b);
-    to_bf16_kernel<<<grid_for((long long)m->H * m->H, 256), 256, 0, st>>>(m->w + m->oW2, m->H, m->H, m->H, m->W2b);
-    to_bf16_kernel<<<grid_for((long long)m->O * m->H, 256), 256, 0, st>>>(m->w + m->oW3, m->O, m->H, m->H, m->W3b);
+    to_bf16_kernel<<<grid_for((long long)m->H * m->Hp, 256), 256, 0, st>>>(m->w + m->oW2, m->H, m->H, m->Hp, m->W2b);
+    to_bf16_kernel<<<grid_for((long long)m->O * m->Hp, 256), 256, 0, st>>>(m->w + m->oW3, m->O, m->H, m->Hp, m->W3b);
     return cuda_status(cudaGetLastError());
 }
 
-// forward: Xb -> Z1 (pre-act), H1b -> Z2, H2b -> Y
-static int forward(exact_mlp *m, const float *x, int B, float *y, cudaStream_t st) {
-    pack_input_kernel<<<grid_for((long long)B * kMlpInPad, 256), 256, 0, st>>>(x, B, m->din, m->Xb);
+template <int MODE>
+static cudaError_t layer(const LayerArgs &g, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((g.N + kBN - 1) / kBN, (g.M + 31) / 32);
+    cfg.blockDim = dim3(128);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, layer_kernel<MODE>, g);
+}
+
+// forward: x -> Z1, H1b -> Z2, H2b -> y; with a target also dY, dYb and the
+// partial losses
+static int forward(exact_mlp *m, const float *x, int B, float *y, const float *target, cudaStream_t st) {
     const int H = m->H, O = m->O;
-    GemmArgs g1 = make_gemm(B, H, kMlpInPad, m->Xb, kMlpInPad, 1, m->W1b, 1, kMlpInPad, m->Z1, H, EPI_BIAS_GELU);
-    g1.bias = m->w + m->ob1; g1.Cb = m->H1b; g1.ldcb = H;
-    GemmArgs g2 = make_gemm(B, H, H, m->H1b, H, 1, m->W2b, 1, H, m->Z2, H, EPI_BIAS_GELU);
-    g2.bias = m->w + m->ob2; g2.Cb = m->H2b; g2.ldcb = H;
-    GemmArgs g3 = make_gemm(B, O, H, m->H2b, H, 1, m->W3b, 1, H, y, O, EPI_BIAS);
-    g3.bias = m->w + m->ob3;
-    if (gemm(g1, st) != cudaSuccess || gemm(g2, st) != cudaSuccess || gemm(g3, st) != cudaSuccess) return EXACT_ECUDA;
+    LayerArgs a;
+    memset(&a, 0, sizeof a);
+    a.M = B; a.N = H; a.K = m->din; a.x = x; a.Xb = target ? m->Xb : nullptr; a.W = m->W1b; a.ldw = kMlpInPad;
+    a.bias = m->w + m->ob1; a.C = m->Z1; a.Cb = m->H1b; a.ldcb = m->Hp;
+    LayerArgs b;
+    memset(&b, 0, sizeof b);
+    b.M = B; b.N = H; b.K = H; b.A = m->H1b; b.lda = m->Hp; b.W = m->W2b; b.ldw = m->Hp;
+    b.bias = m->w + m->ob2; b.C = m->Z2; b.Cb = m->H2b; b.ldcb = m->Hp;
+    LayerArgs c;
+    memset(&c, 0, sizeof c);
+    c.M = B; c.N = O; c.K = H; c.A = m->H2b; c.lda = m->Hp; c.W = m->W3b; c.ldw = m->Hp;
+    c.bias = m->w + m->ob3; c.C = y; c.Cb = m->dYb; c.ldcb = m->Op;
+    c.target = target; c.dY = m->dY; c.scale = 2.f / (float)((long long)B * O); c.lossp = m->lossp;
+    if (layer<LAYER_IN>(a, st) != cudaSuccess || layer<LAYER_HIDDEN>(b, st) != cudaSuccess ||
+        layer<LAYER_OUT>(c, st) != cudaSuccess)
+        return EXACT_ECUDA;
     return EXACT_OK;
 }
 
-// loss and gradients into m->g (packed like the parameters)
-static int backward(exact_mlp *m, const float *x, const float *target, int B, cudaStream_t st) {
-    int rc = forward(m, x, B, m->Y, st);
+// Loss and gradients of one batch; grads / loss may be NULL; adam: step the
+// parameters with learning rate lr (step m->t).
+static int backward(exact_mlp *m, const float *x, const float *target, int B, float *grads, float *loss, bool adam,
+                    float lr, cudaStream_t st) {
+    int rc = forward(m, x, B, m->Y, target, st);
     if (rc != EXACT_OK) return rc;
     const int H = m->H, O = m->O, D = m->din;
-    mse_grad_kernel<<<1, 1024, 0, st>>>(m->Y, target, B, O, m->dY, m->dYb, m->loss);
-    // layer 3: gW3 = dY^T H2, gb3 = sum dY, dZ2 = (dY W3) * g'(Z2)
-    GemmArgs a = make_gemm(O, H, B, m->dYb, 1, O, m->H2b, H, 1, m->g + m->oW3, H, EPI_PLAIN);
-    colsum(m->dY, B, O, m->g + m->ob3, m->ws, st);
-    GemmArgs b = make_gemm(B, H, O, m->dYb, O, 1, m->W3b, H, 1, m->dZ, H, EPI_GELU_GRAD);
-    b.gz = m->Z2; b.ldgz = H; b.Cb = m->dZb; b.ldcb = H;
-    if (gemm(a, st, m->ws) != cudaSuccess || gemm(b, st) != cudaSuccess) return EXACT_ECUDA;
-    // layer 2: gW2 = dZ2^T H1, gb2 = sum dZ2, dZ1 = (dZ2 W2) * g'(Z1)
-    GemmArgs c = make_gemm(H, H, B, m->dZb, 1, H, m->H1b, H, 1, m->g + m->oW2, H, EPI_PLAIN);
-    colsum(m->dZ, B, H, m->g + m->ob2, m->ws, st);
-    if (gemm(c, st, m->ws) != cudaSuccess) return EXACT_ECUDA;
-    // dZ1 overwrites dZ / dZb only after gW2 and gb2 have consumed them (stream order)
-    GemmArgs d = make_gemm(B, H, H, m->dZb, H, 1, m->W2b, H, 1, m->Z2, H, EPI_GELU_GRAD);
-    d.gz = m->Z1; d.ldgz = H; d.Cb = m->H2b; d.ldcb = H;   // Z2 / H2b are free after layer 2's backward
-    if (gemm(d, st) != cudaSuccess) return EXACT_ECUDA;
-    // layer 1: gW1 = dZ1^T X (only the d_in real columns), gb1 = sum dZ1
-    GemmArgs e = make_gemm(H, D, B, m->H2b, 1, H, m->Xb, kMlpInPad, 1, m->g + m->oW1, D, EPI_PLAIN);
-    colsum(m->Z2, B, H, m->g + m->ob1, m->ws, st);
-    if (gemm(e, st, m->ws) != cudaSuccess) return EXACT_ECUDA;
-    return cuda_status(cudaGetLastError());
+    // dZ2 = (dY W3) g'(Z2), dZ1 = (dZ2 W2) g'(Z1)
+    LayerArgs a;
+    memset(&a, 0, sizeof a);
+    a.M = B; a.N = H; a.K = O; a.A = m->dYb; a.lda = m->Op; a.W = m->W3b; a.ldw = m->Hp;
+    a.C = m->dZ2; a.Cb = m->dZ2b; a.ldcb = m->Hp; a.gz = m->Z2;
+    LayerArgs b = a;
+    b.K = H; b.A = m->dZ2b; b.lda = m->Hp; b.W = m->W2b; b.C = m->dZ1; b.Cb = m->dZ1b; b.gz = m->Z1;
+    if (layer<LAYER_GRAD>(a, st) != cudaSuccess || layer<LAYER_GRAD>(b, st) != cudaSuccess) return EXACT_ECUDA;
+    GradSet gs;
+    memset(&gs, 0, sizeof gs);
+    gs.B = B;
+    const bf16 *Ds[3] = {m->dZ1b, m->dZ2b, m->dYb}, *Hs[3] = {m->Xb, m->H1b, m->H2b};
+    const float *Fs[3] = {m->dZ1, m->dZ2, m->dY};
+    const int ldd[3] = {m->Hp, m->Hp, m->Op}, ldh[3] = {kMlpInPad, m->Hp, m->Hp}, Ms[3] = {H, H, O}, Ns[3] = {D, H, H};
+    FinishArgs f;
+    memset(&f, 0, sizeof f);
+    bf16 *Wb[3] = {m->W1b, m->W2b, m->W3b};
+    int blocks = 0;
+    for (int k = 0; k < 3; ++k) {
+        GradArgs &g = gs.l[k];
+        g.D = Ds[k]; g.H = Hs[k]; g.ldd = ldd[k]; g.ldh = ldh[k]; g.M = Ms[k]; g.N = Ns[k];
+        g.S = splits_for(g.M, g.N, B);
+        g.kchunk = chunk_for(g.S, B);
+        g.P = m->P[k]; g.F = Fs[k]; g.Q = m->Q[k];
+        g.gemm_blocks = ((g.M + 63) / 64) * ((g.N + kBN - 1) / kBN) * g.S;
+        g.blocks = g.gemm_blocks + ((g.M + 127) / 128) * kColSlices;
+        blocks += g.blocks;
+        f.P[k] = g.P; f.Q[k] = g.Q; f.M[k] = g.M; f.N[k] = g.N; f.S[k] = g.S;
+        f.Wb[k] = Wb[k]; f.ldw[k] = ldh[k];
+    }
+    f.grads = grads; f.w = m->w; f.m = m->m; f.v = m->v; f.adam = adam ? 1 : 0;
+    const double b1 = 0.9, b2 = 0.999;
+    f.lr = lr; f.b1 = (float)b1; f.b2 = (float)b2; f.eps = 1e-8f;
+    f.c1 = (float)(1.0 - pow(b1, m->t)); f.c2 = (float)(1.0 - pow(b2, m->t));
+    f.lossp = m->lossp; f.n_lossp = ((O + kBN - 1) / kBN) * ((B + 31) / 32);
+    f.inv_n = 1.0 / (double)((long long)B * O);
+    f.loss = loss;
+    f.n = m->nparam;
+    if (launch_dependent(grad_kernel, (unsigned)blocks, 128u, 0, st, gs) != cudaSuccess ||
+        launch_dependent(finish_kernel, (unsigned)((m->nparam + 255) / 256), 256u, 0, st, f) != cudaSuccess)
+        return EXACT_ECUDA;
+    return EXACT_OK;
 }
 
 extern "C" int exact_mlp_create(int d_in, int hidden, int d_out, int max_batch, exact_mlp **out) {
@@ -369,23 +545,30 @@ extern "C" int exact_mlp_create(int d_in, int hidden, int d_out, int max_batch, 
     m->oW1 = 0; m->ob1 = H * D; m->oW2 = m->ob1 + H; m->ob2 = m->oW2 + H * H; m->oW3 = m->ob2 + H;
     m->ob3 = m->oW3 + O * H;
     m->nparam = m->ob3 + O;
+    m->Hp = (hidden + 7) & ~7;
+    m->Op = (d_out + 7) & ~7;
+    const long long Hp = m->Hp, Op = m->Op, most = 1ll << 40;
     std::vector<size_t> sz = {
-        (size_t)m->nparam * 4, (size_t)m->nparam * 4, (size_t)m->nparam * 4, (size_t)m->nparam * 4,   // w g m v
-        (size_t)(H * kMlpInPad) * 2, (size_t)(H * H) * 2, (size_t)(O * H) * 2,                          // W1b W2b W3b
-        (size_t)(B * kMlpInPad) * 2, (size_t)(B * H) * 2, (size_t)(B * H) * 2, (size_t)(B * O) * 2,      // Xb H1b H2b dYb
-        (size_t)(B * H) * 2,                                                                             // dZb
-        (size_t)(B * H) * 4, (size_t)(B * H) * 4, (size_t)(B * O) * 4, (size_t)(B * O) * 4,              // Z1 Z2 Y dY
-        (size_t)(B * H) * 4, 256,                                                                        // dZ loss
-        (size_t)kSplitMax * (size_t)std::max(H * std::max(H, D), O * H) * 4};                           // ws
+        (size_t)m->nparam * 4, (size_t)m->nparam * 4, (size_t)m->nparam * 4,                            // w m v
+        (size_t)(H * kMlpInPad) * 2, (size_t)(H * Hp) * 2, (size_t)(O * Hp) * 2,                        // W1b W2b W3b
+        (size_t)(B * kMlpInPad) * 2, (size_t)(B * Hp) * 2, (size_t)(B * Hp) * 2, (size_t)(B * Op) * 2,   // Xb H1b H2b dYb
+        (size_t)(B * Hp) * 2, (size_t)(B * Hp) * 2,                                                     // dZ1b dZ2b
+        (size_t)(B * H) * 4, (size_t)(B * H) * 4, (size_t)(B * O) * 4, (size_t)(B * O) * 4,             // Z1 Z2 Y dY
+        (size_t)(B * H) * 4, (size_t)(B * H) * 4,                                                       // dZ1 dZ2
+        (size_t)splits_for(hidden, d_in, most) * H * D * 4, (size_t)splits_for(hidden, hidden, most) * H * H * 4,
+        (size_t)splits_for(d_out, hidden, most) * O * H * 4,                                            // P
+        (size_t)kColSlices * H * 4, (size_t)kColSlices * H * 4, (size_t)kColSlices * O * 4,             // Q
+        (size_t)((O + kBN - 1) / kBN) * ((B + 31) / 32) * 8};                                           // lossp
     size_t total = 0;
     for (auto s : sz) total += align_up(s, 256);
     if (cudaMalloc(&m->dev, total) != cudaSuccess) { delete m; return EXACT_ECUDA; }
     if (cudaMemset(m->dev, 0, total) != cudaSuccess) { cudaFree(m->dev); delete m; return EXACT_ECUDA; }
     char *p = static_cast<char *>(m->dev);
-    void **slots[] = {(void **)&m->w, (void **)&m->g, (void **)&m->m, (void **)&m->v, (void **)&m->W1b,
-                      (void **)&m->W2b, (void **)&m->W3b, (void **)&m->Xb, (void **)&m->H1b, (void **)&m->H2b,
-                      (void **)&m->dYb, (void **)&m->dZb, (void **)&m->Z1, (void **)&m->Z2, (void **)&m->Y,
-                      (void **)&m->dY, (void **)&m->dZ, (void **)&m->loss, (void **)&m->ws};
+    void **slots[] = {(void **)&m->w, (void **)&m->m, (void **)&m->v, (void **)&m->W1b, (void **)&m->W2b,
+                      (void **)&m->W3b, (void **)&m->Xb, (void **)&m->H1b, (void **)&m->H2b, (void **)&m->dYb,
+                      (void **)&m->dZ1b, (void **)&m->dZ2b, (void **)&m->Z1, (void **)&m->Z2, (void **)&m->Y,
+                      (void **)&m->dY, (void **)&m->dZ1, (void **)&m->dZ2, (void **)&m->P[0], (void **)&m->P[1],
+                      (void **)&m->P[2], (void **)&m->Q[0], (void **)&m->Q[1], (void **)&m->Q[2], (void **)&m->lossp};
     for (size_t i = 0; i < sz.size(); ++i) {
         *slots[i] = p;
         p += align_up(sz[i], 256);
@@ -458,35 +641,22 @@ extern "C" int exact_mlp_forward(exact_mlp *m, const float *x, int B, float *y, 
     if (!m || !x || !y || B < 0) return EXACT_EINVAL;
     if (B == 0) return EXACT_OK;
     if (B > m->maxB) return EXACT_ECAPACITY;
-    return forward(m, x, B, y, (cudaStream_t)stream);
+    return forward(m, x, B, y, nullptr, (cudaStream_t)stream);
 }
 
 extern "C" int exact_mlp_loss_grad(exact_mlp *m, const float *x, const float *target, int B, float *loss,
                                    float *grads, void *stream) {
     if (!m || !x || !target || B < 1) return EXACT_EINVAL;
     if (B > m->maxB) return EXACT_ECAPACITY;
-    cudaStream_t st = (cudaStream_t)stream;
-    const int rc = backward(m, x, target, B, st);
-    if (rc != EXACT_OK) return rc;
-    if (loss && cudaMemcpyAsync(loss, m->loss, 4, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return EXACT_ECUDA;
-    if (grads && cudaMemcpyAsync(grads, m->g, (size_t)m->nparam * 4, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-        return EXACT_ECUDA;
-    return EXACT_OK;
+    return backward(m, x, target, B, grads, loss, false, 0.f, (cudaStream_t)stream);
 }
 
 extern "C" int exact_mlp_train_step(exact_mlp *m, const float *x, const float *target, int B, float lr, float *loss,
                                     void *stream) {
     if (!m || !x || !target || B < 1 || !(lr > 0.f)) return EXACT_EINVAL;
     if (B > m->maxB) return EXACT_ECAPACITY;
-    cudaStream_t st = (cudaStream_t)stream;
-    int rc = backward(m, x, target, B, st);
-    if (rc != EXACT_OK) return rc;
     m->t += 1;
-    const double b1 = 0.9, b2 = 0.999;
-    const float c1 = (float)(1.0 - pow(b1, m->t)), c2 = (float)(1.0 - pow(b2, m->t));
-    adam_kernel<<<grid_for(m->nparam, 256), 256, 0, st>>>(m->w, m->g, m->m, m->v, m->nparam, lr, (float)b1, (float)b2,
-                                                          1e-8f, c1, c2);
-    if ((rc = refresh_bf16(m, st)) != EXACT_OK) return rc;
-    if (loss && cudaMemcpyAsync(loss, m->loss, 4, cudaMemcpyDeviceToDevice, st) != cudaSuccess) return EXACT_ECUDA;
-    return cuda_status(cudaGetLastError());
+    const int rc = backward(m, x, target, B, nullptr, loss, true, lr, (cudaStream_t)stream);
+    if (rc != EXACT_OK) m->t -= 1;
+    return rc;
 }
