@@ -91,10 +91,12 @@ void exact_ctx_destroy(exact_ctx *ctx);
  * of up to max_K samples and max_T steps exists (synchronous). */
 int exact_ctx_reserve(exact_ctx *ctx, int max_poses, int max_K, int max_T);
 /* The same, also for clouds of up to max_points points: an MPPI step without
- * a d_min output keeps a spatially ordered copy of clouds of 1,024 points or
- * more in the context (it makes the pruning of far points effective whatever
- * the input order), so a step with a larger cloud than any before may
- * allocate -- reserve ahead of stream capture. */
+ * a d_min output sorts clouds of 1,024 points or more into a cell grid kept in
+ * the context (so that each sample looks only at the points near its
+ * footprint, whatever the input order), and exact_sdf_batch keeps a spatially
+ * sorted copy for many poses, so a call with a larger cloud than any before
+ * may allocate -- reserve ahead of stream capture.  (A capturing
+ * exact_sdf_batch without that scratch takes its general path.) */
 int exact_ctx_reserve_cloud(exact_ctx *ctx, int max_poses, int max_K, int max_T, int max_points);
 /* Device-side error word of the context (an exact_status, 0 = none): the
  * first error a kernel launched with this context recorded.  Kernels record
@@ -186,10 +188,9 @@ typedef struct {
  *   U_upd     device, T x n_u, or NULL: the updated nominal before shift/reset
  *   dmin      device, K x T, or NULL: d_min of every scored rollout state.
  *             Without it the sample phase skips the points that provably
- *             cannot come within d_safe of the footprint at a step (bounding
- *             circles of point sub-chunks, then the footprint's bounding box
- *             for the points or 16-point fine sub-chunks of the kept ones;
- *             below 1,024 points, bounding circles per point): every cost
+ *             cannot come within d_safe of the footprint at a step, or cannot
+ *             lower its minimum (a cell grid over the cloud and bounds on each
+ *             point's distance; below 1,024 points, bounding circles): every cost
  *             term and the validation test are the same for any d >= d_safe,
  *             so costs, weights and U are identical either way
  * Limits: 1 <= K <= 65536, 1 <= T <= 128, n_points >= 0, n_wp >= 1,
@@ -288,10 +289,10 @@ int exact_proposal_select(const float *costs_prop, const float *costs_plain, int
  * same output bits) without a context: its scratch is a file-scope device
  * array of EXACT_NOALLOC_ARENA_BYTES that every GPU loading the library
  * holds until the process exits.  One difference in cost, not in results:
- * without a d_min output and with 1,024 points or more, mppi_step prunes far
- * point chunks on a spatially ordered copy of the cloud kept in its context,
- * while this call prunes on the cloud in the order given, which skips fewer
- * chunks (and so runs slower) when consecutive points are not close together.  It allocates nothing (no cudaMalloc,
+ * without a d_min output and with 1,024 points or more, mppi_step walks a cell
+ * grid of the cloud kept in its context, while this call skips far chunks of
+ * the cloud in the order given, which looks at more points (and so runs
+ * slower).  It allocates nothing (no cudaMalloc,
  * cudaFree or allocating library call); it clears the parts of the array
  * that must start at zero with stream-ordered memsets on `stream`.
  *  - The first call on a device looks the array's device address up (once,
@@ -358,10 +359,8 @@ int mppi_step_batched(exact_batch *batch, void *stream);
 
 /* Tile autotuner: times the batch's sample phase (which writes only batch
  * scratch, never the scenes' U or outputs) for each candidate tile shape
- * (threads per block x point pairs per lane: the sample phase cuts the
- * staged cloud into sub-chunks of 64 x pairs_per_lane points, the unit it
- * skips when a sub-chunk cannot come within d_safe of the footprint at a
- * step; scenes without a d_min output only), `iters` runs
+ * (threads per block x point pairs per lane; the scenes without a d_min
+ * output, which walk a cell grid, only use the threads), `iters` runs
  * each, keeps the fastest for later steps and, when json_out is non-NULL,
  * writes the timings as JSON text (at most json_cap bytes, NUL-terminated).
  * Synchronises `stream`. */

@@ -3,17 +3,21 @@
 //
 // Plan (exact_batch_create, host, once): a device scene table (parameters,
 // pointers, footprint constants, scratch addresses), the work-item list of
-// the sample phase -- one item per (scene, sample), or per (scene, two
-// consecutive samples) when the batch holds at least four samples per SM and
-// the scene's horizon fits two in a block's step slots; scenes ordered by
+// the sample phase -- per scene without a d_min output one item per group of
+// samples (cloud_grid.cuh); per other scene one per (scene, sample), or per
+// (scene, two consecutive samples) when the batch holds at least four samples
+// per SM and the scene's horizon fits two in a block's step slots; scenes ordered by
 // per-sample cost T * N * edges, heaviest first (longest-processing-time
 // order) -- and the block tables of the update and validation phases.
 //
 // Step (mppi_step_batched, capturable): a memset of the per-scene control
-// words and the queue head, then
+// words and the queue heads, then
+//   batched_cloud_grid_kernel, batched_grid_sample_kernel
+//                           one block per cloud sorts it into a cell grid;
+//                           persistent blocks take groups of samples
 //   batched_sample_kernel   persistent: SMs x resident blocks; each block
 //                           pulls items from an atomic queue and runs
-//                           sample_body with the scene's footprint constants
+//                           (scenes with a d_min output) sample_body with the scene's footprint constants
 //                           in shared memory (reloaded only when the scene
 //                           changes; so are the staged points when the cloud
 //                           fits the stage);
@@ -54,25 +58,49 @@ batched_sample_kernel(const SceneDev *__restrict__ scenes, const int2 *__restric
         const int2 it = items[item];
         const SceneDev &D = scenes[it.x];
         if (it.x != fp_scene) {
-            load_fp(s_fp, D);
+            load_table(s_fp, D.fp);
             __syncthreads();
             fp_scene = it.x;
         }
-        const SmemEval ev{s_fp, D.kind, D.nfp, D.bc, D.bh};
-        sample_body(D.V, ev, item_sample(it), 0, sm, s_pts, it.x == pts_scene, pairs_per_lane, D.circ,
-                    item_second(it));
+        const SmemEval ev = table_eval(D.fp, s_fp);
+        sample_body(D.V, ev, item_sample(it), 0, sm, s_pts, it.x == pts_scene, pairs_per_lane, item_second(it));
         pts_scene = D.V.N <= kStage ? it.x : -1;
     }
 }
 
-// Spatially ordered cloud copies of the scenes that prune (one block each).
-__global__ void __launch_bounds__(kSortThreads)
-batched_sort_kernel(const SceneDev *__restrict__ scenes, const int *__restrict__ list) {
-    __shared__ SortSmem sm;
+// The scenes without a d_min output: persistent blocks take grid items from
+// the queue, a scene's footprint terms and distance field in shared memory.
+__global__ void __launch_bounds__(768)   // at most 512 are launched: 80 registers, three blocks of 256 per SM
+batched_grid_sample_kernel(const SceneDev *__restrict__ scenes, const int2 *__restrict__ items, int n_items,
+                           int group, unsigned *queue) {
+    extern __shared__ float4 dyn[];
+    __shared__ float4 s_fp[kFpSlots];
+    __shared__ int s_item, s_next;
+    int fp_scene = -1;   // block-uniform
+    for (;;) {
+        if (threadIdx.x == 0) s_item = (int)atomicAdd(queue, 1u);
+        __syncthreads();   // also: the previous item's costs are formed
+        const int item = s_item;
+        if (item >= n_items) break;
+        const int2 it = items[item];
+        const SceneDev &D = scenes[it.x];
+        const bool fresh = it.x != fp_scene;
+        if (fresh) {
+            load_table(s_fp, D.fp);
+            __syncthreads();
+            fp_scene = it.x;
+        }
+        grid_samples<false>(D.V, D.grid, GridStride{0, 0}, table_eval(D.fp, s_fp), it.y, min(group, D.V.P.K - it.y),
+                            reinterpret_cast<char *>(dyn), fresh, &s_next);
+    }
+}
+
+// Cell grids of the scenes without a d_min output (one block each).
+__global__ void __launch_bounds__(kGridThreads)
+batched_cloud_grid_kernel(const SceneDev *__restrict__ scenes, const int *__restrict__ list) {
+    __shared__ GridSmem sm;
     const SceneDev &D = scenes[list[blockIdx.x]];
-    sort_cloud_block<false>(D.src_pts, nullptr, D.src_mask, D.V.N, const_cast<float2 *>(D.V.pts), nullptr, sm);
-    __syncthreads();
-    cloud_circles<false>(D.V.pts, nullptr, D.V.N, const_cast<float4 *>(D.circ));
+    build_grid<false>(D.src_pts, nullptr, D.src_mask, D.V.N, const_cast<float2 *>(D.V.pts), nullptr, D.grid, sm);
 }
 
 __global__ void __launch_bounds__(kUpdBlock)
@@ -88,10 +116,10 @@ batched_validate_kernel(const SceneDev *__restrict__ scenes, const int2 *__restr
     __shared__ ValidateSmem sm;
     const int2 t = table[blockIdx.x];
     const SceneDev &D = scenes[t.x];
-    load_fp(s_fp, D);
+    load_table(s_fp, D.fp);
     __syncthreads();
-    const SmemEval ev{s_fp, D.kind, D.nfp, D.bc, D.bh};
-    validate_body(D.V, ev, t.y / D.V.val_chunks, t.y % D.V.val_chunks, sm, D.circ);
+    const SmemEval ev = table_eval(D.fp, s_fp);
+    validate_body(D.V, ev, t.y / D.V.val_chunks, t.y % D.V.val_chunks, sm, D.grid);
 }
 
 int check_params(const exact_mppi_params *p);
@@ -114,8 +142,19 @@ static int batch_grid(exact_batch *b) {
         return EXACT_ECUDA;
     if (per_sm < 1) return EXACT_EINVAL;
     b->grid = b->sms * per_sm;
+    if (b->n_gitems == 0) return EXACT_OK;
+    if (cudaFuncSetAttribute(batched_grid_sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)grid_smem(b)) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batched_grid_sample_kernel, b->threads, grid_smem(b)) !=
+            cudaSuccess)
+        return EXACT_ECUDA;
+    if (per_sm < 1) return EXACT_EINVAL;
+    b->ggrid = b->sms * per_sm;
     return EXACT_OK;
 }
+
+// Scenes without a d_min output walk a cell grid (cloud_grid.cuh).
+static bool uses_grid(const exact_scene &S) { return !S.dmin && S.n_points <= kGridMaxPoints; }
 
 extern "C" int exact_batch_create(int n_scenes, const exact_scene *scenes, exact_batch **out) {
     if (!out || !scenes || n_scenes < 1) return EXACT_EINVAL;
@@ -134,14 +173,15 @@ extern "C" int exact_batch_create(int n_scenes, const exact_scene *scenes, exact
         if (S.n_points > 0 && (!S.cloud || ((uintptr_t)S.cloud & 7u) != 0)) return EXACT_EINVAL;
         scratch_off[s] = scratch_total;
         scratch_total += align_up(scene_scratch_bytes(S.params.K, S.params.T, 1), 256);
-        // scenes that prune (no d_min output, large cloud) get a spatially ordered cloud copy
-        if (!S.dmin && S.n_points >= kPruneMin)
-            scratch_total += align_up((size_t)S.n_points * sizeof(float2), 256) + circle_bytes(S.n_points);
-        max_stage = std::max(max_stage, std::min(S.n_points, kStage));
+        // scenes without a d_min output get a grid and a copy of their cloud in cell order
+        if (uses_grid(S))
+            scratch_total += grid_copy_bytes(S.n_points, false);
+        else
+            max_stage = std::max(max_stage, std::min(S.n_points, kStage));
     }
     std::vector<int> sort_list;
     for (int s = 0; s < n_scenes; ++s)
-        if (!scenes[s].dmin && scenes[s].n_points >= kPruneMin) sort_list.push_back(s);
+        if (uses_grid(scenes[s])) sort_list.push_back(s);
     const size_t table_bytes = align_up(sizeof(SceneDev) * n_scenes, 256);
     // items and block tables
     std::vector<int> order(n_scenes);
@@ -151,12 +191,24 @@ extern "C" int exact_batch_create(int n_scenes, const exact_scene *scenes, exact
         return (double)S.params.T * std::max(S.n_points, 1) * (double)S.fp->n_pad;
     };
     std::stable_sort(order.begin(), order.end(), [&](int a, int c) { return cost(a) > cost(c); });
-    std::vector<int2> items, upd, val;
-    long long total_k = 0;
-    for (int s = 0; s < n_scenes; ++s) total_k += scenes[s].params.K;
+    std::vector<int2> items, gitems, upd, val;
+    long long total_k = 0, grid_k = 0;
+    int grid_T = 1;
+    for (int s = 0; s < n_scenes; ++s) {
+        total_k += scenes[s].params.K;
+        if (uses_grid(scenes[s])) {
+            grid_k += scenes[s].params.K;
+            grid_T = std::max(grid_T, scenes[s].params.T);
+        }
+    }
     const int sms_now = current_sm_count();
+    const int group = grid_group(grid_k, sms_now);
     for (int s : order) {
         const exact_mppi_params &p = scenes[s].params;
+        if (uses_grid(scenes[s])) {
+            for (int r = 0; r < p.K; r += group) gitems.push_back(make_int2(s, r));
+            continue;
+        }
         // pairs of samples per item when the whole batch has enough samples
         // to fill the GPU at half the items (and this scene's horizon fits)
         const bool two = pair_samples((int)std::min<long long>(total_k, 1 << 29), p.T, 1, sms_now);
@@ -166,16 +218,17 @@ extern "C" int exact_batch_create(int n_scenes, const exact_scene *scenes, exact
     for (int s = 0; s < n_scenes; ++s) {
         const exact_mppi_params &p = scenes[s].params;
         for (int q = 0; q < upd_blocks_for(p.K, p.T, p.n_u); ++q) upd.push_back(make_int2(s, q));
-        for (int q = 0; q < p.T * val_chunks_for(scenes[s].n_points); ++q) val.push_back(make_int2(s, q));
+        for (int q = 0; q < p.T * val_chunks_for(scenes[s].n_points, uses_grid(scenes[s])); ++q) val.push_back(make_int2(s, q));
     }
-    const size_t items_bytes = align_up(items.size() * sizeof(int2), 256);
+    const size_t items_bytes = align_up(items.size() * sizeof(int2) + 1, 256);
+    const size_t gitems_bytes = align_up(gitems.size() * sizeof(int2) + 1, 256);
     const size_t upd_bytes = align_up(upd.size() * sizeof(int2), 256);
     const size_t val_bytes = align_up(val.size() * sizeof(int2), 256);
-    const size_t ctrl_bytes = align_up(kHdrStride * n_scenes + sizeof(unsigned), 256);
+    const size_t ctrl_bytes = align_up(kHdrStride * n_scenes + 2 * sizeof(unsigned), 256);
     const size_t sort_bytes = align_up(sort_list.size() * sizeof(int) + 1, 256);
     const size_t err_bytes = 256;
     const size_t total =
-        2 * table_bytes + items_bytes + upd_bytes + val_bytes + ctrl_bytes + sort_bytes + err_bytes + scratch_total;
+        2 * table_bytes + items_bytes + gitems_bytes + upd_bytes + val_bytes + ctrl_bytes + sort_bytes + err_bytes + scratch_total;
 
     exact_batch *b = new (std::nothrow) exact_batch();
     if (!b) return EXACT_EINVAL;
@@ -184,6 +237,7 @@ extern "C" int exact_batch_create(int n_scenes, const exact_scene *scenes, exact
     b->d_scenes = reinterpret_cast<SceneDev *>(p); p += table_bytes;
     b->d_tune = reinterpret_cast<SceneDev *>(p); p += table_bytes;
     b->d_items = reinterpret_cast<int2 *>(p); p += items_bytes;
+    b->d_gitems = reinterpret_cast<int2 *>(p); p += gitems_bytes;
     b->d_upd = reinterpret_cast<int2 *>(p); p += upd_bytes;
     b->d_val = reinterpret_cast<int2 *>(p); p += val_bytes;
     b->d_ctrl = p; p += ctrl_bytes;
@@ -195,6 +249,9 @@ extern "C" int exact_batch_create(int n_scenes, const exact_scene *scenes, exact
     b->d_queue = reinterpret_cast<unsigned *>(b->d_ctrl + kHdrStride * n_scenes);
     b->n = n_scenes;
     b->n_items = (int)items.size();
+    b->n_gitems = (int)gitems.size();
+    b->grid_group = group;
+    b->grid_T = grid_T;
     b->n_upd = (int)upd.size();
     b->n_val = (int)val.size();
     b->smem = kFpSlots * sizeof(float4) + (size_t)max_stage * sizeof(float2);
@@ -225,40 +282,27 @@ extern "C" int exact_batch_create(int n_scenes, const exact_scene *scenes, exact
         carve_scene(V, scratch + scratch_off[s], S.params.K, S.params.T, 1);
         D.src_pts = V.pts;
         D.src_mask = V.mask;
-        if (!S.dmin && S.n_points >= kPruneMin) {   // the sort kernel fills the copy before each step
+        if (uses_grid(S)) {   // filled before each step's sample phase
             char *q = scratch + scratch_off[s] + align_up(scene_scratch_bytes(S.params.K, S.params.T, 1), 256);
-            V.pts = reinterpret_cast<const float2 *>(q);
-            D.circ = reinterpret_cast<const float4 *>(q + align_up((size_t)S.n_points * sizeof(float2), 256));
+            D.grid = reinterpret_cast<CloudGrid *>(q);
+            V.pts = reinterpret_cast<const float2 *>(q + kGridBytes);
             V.mask = nullptr;
         }
         V.upd_chunk = upd_chunk_for(S.params.K, S.params.T, S.params.n_u);
         V.upd_blocks = upd_blocks_for(S.params.K, S.params.T, S.params.n_u);
-        V.val_chunks = val_chunks_for(S.n_points);
+        V.val_chunks = val_chunks_for(S.n_points, uses_grid(S));
         const exact_footprint *fp = S.fp;
-        D.kind = fp->kind;
-        D.nfp = fp->n_pad;
-        D.bc = make_float3(fp->bcx, fp->bcy, fp->brad);
-        D.bh = make_float2(fp->bhx, fp->bhy);
-        if (fp->kind == EXACT_FP_POLYGON) {
-            const int E = fp->n_pad;
-            float *eyn = reinterpret_cast<float *>(D.fpc + 3 * E + 1);
-            for (int e = 0; e < E; ++e) {
-                D.fpc[3 * e] = make_float4(-fp->vx[e], -fp->vx[e], -fp->vy[e], -fp->vy[e]);
-                D.fpc[3 * e + 1] = make_float4(fp->exn[e], fp->exn[e], -fp->kx[e], -fp->kx[e]);
-                D.fpc[3 * e + 2] = make_float4(-fp->ex[e], -fp->ex[e], -fp->ey[e], -fp->ey[e]);
-                eyn[e] = fp->eyn[e];
-            }
-            D.fpc[3 * E] = D.fpc[0];
-        } else {
-            for (int j = 0; j < fp->n_pad; ++j) D.fpc[j] = make_float4(fp->cx[j], fp->cy[j], fp->sx[j], fp->sy[j]);
-        }
+        D.fp = make_table(fp);
     }
     std::vector<SceneDev> tune = host;
     for (auto &D : tune) D.V.dmin = nullptr;
     int rc = EXACT_OK;
     if (cudaMemcpy(b->d_scenes, host.data(), sizeof(SceneDev) * n_scenes, cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(b->d_tune, tune.data(), sizeof(SceneDev) * n_scenes, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(b->d_items, items.data(), items.size() * sizeof(int2), cudaMemcpyHostToDevice) != cudaSuccess ||
+        (b->n_items &&
+         cudaMemcpy(b->d_items, items.data(), items.size() * sizeof(int2), cudaMemcpyHostToDevice) != cudaSuccess) ||
+        (b->n_gitems && cudaMemcpy(b->d_gitems, gitems.data(), gitems.size() * sizeof(int2), cudaMemcpyHostToDevice) !=
+                            cudaSuccess) ||
         cudaMemcpy(b->d_upd, upd.data(), upd.size() * sizeof(int2), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemcpy(b->d_val, val.data(), val.size() * sizeof(int2), cudaMemcpyHostToDevice) != cudaSuccess ||
         (b->n_sort && cudaMemcpy(b->d_sort, sort_list.data(), sort_list.size() * sizeof(int), cudaMemcpyHostToDevice) !=
@@ -283,24 +327,31 @@ extern "C" void exact_batch_destroy(exact_batch *b) {
     delete b;
 }
 
+static int launch_uniform(exact_batch *b, const SceneDev *table, cudaStream_t st, BatchPhase phase) {
+    return b->fp.kind == EXACT_FP_POLYGON && b->fp.n_pad > 16 ? launch_uniform_large(b, table, st, phase)
+                                                               : launch_uniform_small(b, table, st, phase);
+}
+
 static int launch_sample(exact_batch *b, const SceneDev *table, cudaStream_t st) {
     if (cudaMemsetAsync(b->d_ctrl, 0, b->ctrl_bytes, st) != cudaSuccess) return EXACT_ECUDA;
-    if (b->n_sort > 0) {
-        batched_sort_kernel<<<b->n_sort, kSortThreads, 0, st>>>(table, b->d_sort);
-        if (cudaGetLastError() != cudaSuccess) return EXACT_ECUDA;
+    if (b->n_items > 0) {   // scenes with a d_min output
+        if (!b->uniform) {
+            batched_sample_kernel<<<b->grid, b->threads, b->smem, st>>>(table, b->d_items, b->n_items, b->d_queue,
+                                                                         b->pairs);
+            if (cudaGetLastError() != cudaSuccess) return EXACT_ECUDA;
+        } else {
+            const int rc = launch_uniform(b, table, st, kPhaseSample);
+            if (rc != EXACT_OK) return rc;
+        }
     }
-    if (!b->uniform) {
-        // behind the cloud-ordering kernel the persistent blocks start early
-        // (rollouts first; sample_body waits before it reads a cloud)
-        if (b->n_sort > 0)
-            return cuda_status(launch_dependent(batched_sample_kernel, (unsigned)b->grid, (unsigned)b->threads, b->smem,
-                                                st, table, (const int2 *)b->d_items, b->n_items, b->d_queue, b->pairs));
-        batched_sample_kernel<<<b->grid, b->threads, b->smem, st>>>(table, b->d_items, b->n_items, b->d_queue,
-                                                                     b->pairs);
-        return cuda_status(cudaGetLastError());
-    }
-    return b->fp.kind == EXACT_FP_POLYGON && b->fp.n_pad > 16 ? launch_uniform_large(b, table, st, false)
-                                                               : launch_uniform_small(b, table, st, false);
+    if (b->n_gitems == 0) return EXACT_OK;
+    batched_cloud_grid_kernel<<<b->n_sort, kGridThreads, 0, st>>>(table, b->d_sort);
+    if (cudaGetLastError() != cudaSuccess) return EXACT_ECUDA;
+    // the persistent warps start early (rollouts first; grid_sample waits
+    // before it reads a grid)
+    return cuda_status(launch_dependent(batched_grid_sample_kernel, (unsigned)b->ggrid, (unsigned)b->threads,
+                                        grid_smem(b), st, table, (const int2 *)b->d_gitems, b->n_gitems, b->grid_group,
+                                        b->d_queue + 1));
 }
 
 extern "C" int mppi_step_batched(exact_batch *b, void *stream) {
@@ -317,8 +368,7 @@ extern "C" int mppi_step_batched(exact_batch *b, void *stream) {
     if (!b->uniform)
         return cuda_status(launch_dependent(batched_validate_kernel, (unsigned)b->n_val, (unsigned)kBlock, 0, st,
                                             (const SceneDev *)b->d_scenes, (const int2 *)b->d_val));
-    return b->fp.kind == EXACT_FP_POLYGON && b->fp.n_pad > 16 ? launch_uniform_large(b, b->d_scenes, st, true)
-                                                               : launch_uniform_small(b, b->d_scenes, st, true);
+    return launch_uniform(b, b->d_scenes, st, kPhaseValidate);
 }
 
 extern "C" int exact_batch_get_error(exact_batch *b, void *stream) {

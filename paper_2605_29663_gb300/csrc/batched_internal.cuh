@@ -3,34 +3,27 @@
 // table entry and the batch plan.
 #pragma once
 
-#include "mppi_cycle.cuh"
+#include "cloud_grid.cuh"
 
 namespace exact {
 
-constexpr int kFpSlots = poly_slot_count(EXACT_MAX_POLY_VERTICES);   // float4 footprint slots
 constexpr size_t kHdrStride = 64;                            // bytes between scene headers
 
 struct SceneDev {
     SceneView V;
-    const float2 *src_pts;      // the caller's cloud (V.pts may be its spatially ordered copy)
+    const float2 *src_pts;      // the caller's cloud (V.pts may be its copy in cell order)
     const uint8_t *src_mask;
-    const float4 *circ;         // sub-chunk circles of the ordered copy, or NULL
-    int kind, nfp;
-    float3 bc;    // footprint bounding circle
-    float2 bh;    // half extents of the footprint's bounding box about the circle's centre
-    float4 fpc[kFpSlots];
+    CloudGrid *grid;            // cell grid of the ordered copy, or NULL
+    FpTable fp;
 };
 
-// A sample item is (scene, r); bit 30 of r marks an item that also takes
-// sample r + 1 of the same scene (see sample_body).
+// A sample item of a scene with a d_min output is (scene, r); bit 30 of r
+// marks an item that also takes sample r + 1 of the same scene (see
+// sample_body).  A grid item is (scene, r): grid_group consecutive samples
+// from r on (see grid_samples).
 constexpr int kItemPair = 1 << 30;
 __device__ __forceinline__ int item_sample(int2 it) { return it.y & (kItemPair - 1); }
 __device__ __forceinline__ int item_second(int2 it) { return (it.y & kItemPair) ? (it.y & (kItemPair - 1)) + 1 : -1; }
-
-__device__ __forceinline__ void load_fp(float4 *dst, const SceneDev &D) {
-    const int nf = D.kind == EXACT_FP_POLYGON ? poly_slot_count(D.nfp) : D.nfp;
-    for (int i = threadIdx.x; i < nf; i += blockDim.x) dst[i] = D.fpc[i];
-}
 
 }  // namespace exact
 
@@ -39,15 +32,17 @@ struct exact_batch {
     void *dev = nullptr;
     exact::SceneDev *d_scenes = nullptr;      // for steps
     exact::SceneDev *d_tune = nullptr;        // same, without the dmin outputs (autotuning)
-    int2 *d_items = nullptr, *d_upd = nullptr, *d_val = nullptr;
-    int n_items = 0, n_upd = 0, n_val = 0;
+    int2 *d_items = nullptr, *d_gitems = nullptr, *d_upd = nullptr, *d_val = nullptr;
+    int n_items = 0, n_gitems = 0, n_upd = 0, n_val = 0;
+    int grid_group = 1, grid_T = 1;      // samples per grid item, longest horizon of a grid scene
     char *d_ctrl = nullptr;            // n headers (kHdrStride apart) + queue head
     size_t ctrl_bytes = 0;
-    unsigned *d_queue = nullptr;
-    int *d_sort = nullptr;             // scenes whose cloud gets a spatially ordered copy
+    unsigned *d_queue = nullptr;       // queue heads: items, grid items
+    int *d_sort = nullptr;             // scenes whose cloud gets a grid
     int n_sort = 0;
     size_t smem = 0;
     int threads = exact::kBlock, pairs = 1, sms = 0, grid = 0;
+    int ggrid = 0;                     // persistent grid of the grid kernel
     bool uniform = false;              // every scene has the same footprint constants
     exact_footprint fp;                // their copy (uniform batches)
     int grid_c = 0;                    // persistent grid of the constant-footprint kernel (0 = not yet known)
@@ -55,10 +50,12 @@ struct exact_batch {
 };
 
 namespace exact {
-// Sample (validate = false) or validation launch of a batch whose scenes
-// share one footprint, footprint constants as kernel parameters
-// (batched_uniform.cuh): rectangle covers and polygons of up to 16 edges,
-// and larger polygons.
-int launch_uniform_small(exact_batch *b, const SceneDev *table, cudaStream_t st, bool validate);
-int launch_uniform_large(exact_batch *b, const SceneDev *table, cudaStream_t st, bool validate);
+// Sample or validation launch of a batch whose scenes share one footprint,
+// footprint constants as kernel parameters (batched_uniform.cuh): rectangle
+// covers and polygons of up to 16 edges, and larger polygons.
+enum BatchPhase { kPhaseSample, kPhaseValidate };
+int launch_uniform_small(exact_batch *b, const SceneDev *table, cudaStream_t st, BatchPhase phase);
+int launch_uniform_large(exact_batch *b, const SceneDev *table, cudaStream_t st, BatchPhase phase);
+
+inline size_t grid_smem(const exact_batch *b) { return grid_smem_bytes(b->grid_T, b->grid_group, b->threads / 32); }
 }  // namespace exact

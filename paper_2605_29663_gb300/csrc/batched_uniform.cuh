@@ -28,8 +28,7 @@ batched_sample_kernel_c(const SceneDev *__restrict__ scenes, const int2 *__restr
         if (item >= n_items) break;
         const int2 it = items[item];
         const SceneDev &D = scenes[it.x];
-        sample_body(D.V, ev, item_sample(it), 0, sm, s_pts, it.x == pts_scene, pairs_per_lane, D.circ,
-                    item_second(it));
+        sample_body(D.V, ev, item_sample(it), 0, sm, s_pts, it.x == pts_scene, pairs_per_lane, item_second(it));
         pts_scene = D.V.N <= kStage ? it.x : -1;
     }
 }
@@ -41,7 +40,7 @@ batched_validate_kernel_c(const SceneDev *__restrict__ scenes, const int2 *__res
     __shared__ ValidateSmem sm;
     const int2 t = table[blockIdx.x];
     const SceneDev &D = scenes[t.x];
-    validate_body(D.V, ev, t.y / D.V.val_chunks, t.y % D.V.val_chunks, sm, D.circ);
+    validate_body(D.V, ev, t.y / D.V.val_chunks, t.y % D.V.val_chunks, sm, D.grid);
 }
 
 template <class FPC>
@@ -56,10 +55,6 @@ int launch_uniform_sample_t(exact_batch *b, const SceneDev *table, cudaStream_t 
             return EXACT_ECUDA;
         b->grid_c = b->sms * per_sm;
     }
-    if (b->n_sort > 0)   // behind the cloud-ordering kernel: start early (see batched.cu)
-        return cuda_status(launch_dependent(k, (unsigned)b->grid_c, (unsigned)b->threads, b->smem, st, table,
-                                            (const int2 *)b->d_items, b->n_items, b->d_queue, b->pairs,
-                                            ConstEval<FPC>{fpc}));
     k<<<b->grid_c, b->threads, b->smem, st>>>(table, b->d_items, b->n_items, b->d_queue, b->pairs,
                                               ConstEval<FPC>{fpc});
     return cuda_status(cudaGetLastError());
@@ -71,8 +66,10 @@ int launch_uniform_validate_t(exact_batch *b, cudaStream_t st, const FPC &fpc) {
                                         (const SceneDev *)b->d_scenes, (const int2 *)b->d_val, ConstEval<FPC>{fpc}));
 }
 
-// Per size class (returns EXACT_EINVAL for a footprint of the other class).
-int launch_uniform_small(exact_batch *b, const SceneDev *table, cudaStream_t st, bool validate);
-int launch_uniform_large(exact_batch *b, const SceneDev *table, cudaStream_t st, bool validate);
+// The launch of one phase.
+template <class FPC>
+int launch_uniform_t(exact_batch *b, const SceneDev *table, cudaStream_t st, BatchPhase phase, const FPC &fpc) {
+    return phase == kPhaseValidate ? launch_uniform_validate_t(b, st, fpc) : launch_uniform_sample_t(b, table, st, fpc);
+}
 
 }  // namespace exact

@@ -3,11 +3,9 @@
 
 namespace exact {
 
-int launch_uniform_small(exact_batch *b, const SceneDev *table, cudaStream_t st, bool validate) {
+int launch_uniform_small(exact_batch *b, const SceneDev *table, cudaStream_t st, BatchPhase phase) {
     const exact_footprint *fp = &b->fp;
-    auto go = [&](auto fpc) -> int {
-        return validate ? launch_uniform_validate_t(b, st, fpc) : launch_uniform_sample_t(b, table, st, fpc);
-    };
+    auto go = [&](auto fpc) -> int { return launch_uniform_t(b, table, st, phase, fpc); };
     if (fp->kind == EXACT_FP_POLYGON) {
         switch (fp->n_pad) {
         case 4: return go(make_poly<4>(fp));

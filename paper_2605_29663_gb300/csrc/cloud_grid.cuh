@@ -1,0 +1,492 @@
+// cloud_grid.cuh -- the cell grid over an obstacle cloud and the sample phase
+// that walks it.
+//
+// A cycle without a d_min output needs, per (sample, step), only the points
+// within d_safe of the footprint: every cost term and the validation test
+// are the same for any d >= d_safe.  So one block per cloud sorts the points
+// into the cells of a uniform grid (row-major, so consecutive cells of a row
+// hold consecutive points), and the sample phase walks, per (sample, step),
+// the grid rows that the footprint's bounding box (grown by d_safe and a
+// slack far above rounding) crosses: each row contributes one contiguous run
+// of points, found with two reads of the cell-start table.  A distance field
+// of the footprint bounds each of those points' distances from both sides
+// (fill_field), and only the points that can be a step's minimum are evaluated.
+// No output changes by a bit: a point in no walked cell is farther than
+// d_safe, and a point not evaluated is farther than one that is.
+//
+// What bounds it: instruction issue (41 to 68 % of the cycles issue) where
+// many points lie inside the footprints, else the latency of one sample's
+// rollout, walk and evaluation.  Measured against sub-chunk circles over a
+// Morton-ordered copy (cycle times, the nominal driven to where the samples
+// touch obstacles): forklift K = 2,048, T = 40, N = 4,096 127 -> 87 us;
+// hybrid 3 x K = 1,024, N = 2,048 70 -> 43 us; 64 scenes of up to 20,000
+// points 6.29 -> 1.60 ms; predicted K = 1,024, N = 2,048 49 -> 29 us.  One warp
+// per sample was slower than a block's warps sharing eight samples (the
+// forklift's near points range from 0 to 4,700 per sample).
+#pragma once
+
+#include "mppi_cycle.cuh"
+
+namespace exact {
+
+constexpr int kGridThreads = 1024;
+constexpr int kGridRegs = 4;          // points per thread kept in registers (clouds of up to 4,096)
+
+struct GridSmem {
+    int cnt[kCells + 1];
+    float red[5][kGridThreads / 32];
+    float box[5];
+    int part[kGridThreads / 32];
+};
+
+// One block sorts the cloud's valid points (unmasked, finite position and
+// velocity) into cells: opts / ovel in cell order, grid header and cell
+// starts.  The order inside a cell follows the scatter's atomics; nothing
+// computed from the cloud depends on it (minima are exact in any order).
+// PREDICT: the points are taken where they are at time th.
+template <bool MOVING, bool PREDICT = false>
+__device__ __forceinline__ void build_grid(const float2 *__restrict__ pts, const float2 *__restrict__ vel,
+                                           const uint8_t *__restrict__ mask, int N, float2 *__restrict__ opts,
+                                           float2 *__restrict__ ovel, CloudGrid *__restrict__ grid, GridSmem &sm,
+                                           float th = 0.f) {
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
+    grid_dep_release();   // the sample kernel may start its rollouts meanwhile
+    auto fetch = [&](int i, float2 &p, float2 &v) {
+        p = pts[i];
+        v = MOVING || PREDICT ? vel[i] : make_float2(0.f, 0.f);
+        if (PREDICT) p = make_float2(fmaf(th, v.x, p.x), fmaf(th, v.y, p.y));
+        return (!mask || mask[i]) && isfinite(p.x) && isfinite(p.y) && (!MOVING || (isfinite(v.x) && isfinite(v.y)));
+    };
+    // clouds of up to kGridRegs points per thread are read once and kept in
+    // registers (point tid + k nt in slot k); larger ones are re-read per pass
+    const bool inreg = N <= kGridRegs * nt;
+    float2 rp[kGridRegs], rv[kGridRegs];
+    bool ok[kGridRegs];
+    float lx = finf(), ly = finf(), hx = -finf(), hy = -finf(), vm = 0.f;
+    auto grow = [&](float2 p, float2 v) {
+        lx = fminf(lx, p.x); hx = fmaxf(hx, p.x); ly = fminf(ly, p.y); hy = fmaxf(hy, p.y);
+        if (MOVING) vm = fmaxf(vm, fabsf(v.x) + fabsf(v.y));
+    };
+    if (inreg) {
+#pragma unroll
+        for (int k = 0; k < kGridRegs; ++k) {
+            const int i = tid + k * nt;
+            ok[k] = i < N && fetch(i, rp[k], rv[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < kGridRegs; ++k)
+            if (ok[k]) grow(rp[k], rv[k]);
+    } else {
+#pragma unroll 4
+        for (int i = tid; i < N; i += nt) {
+            float2 p, v;
+            if (fetch(i, p, v)) grow(p, v);
+        }
+    }
+    for (int c = tid; c <= kCells; c += nt) sm.cnt[c] = 0;
+    lx = warp_min_f(lx); ly = warp_min_f(ly); hx = -warp_min_f(-hx); hy = -warp_min_f(-hy);
+    if (MOVING) vm = -warp_min_f(-vm);
+    if (lane == 0) {
+        sm.red[0][warp] = lx; sm.red[1][warp] = ly; sm.red[2][warp] = hx; sm.red[3][warp] = hy;
+        sm.red[4][warp] = vm;
+    }
+    __syncthreads();
+    {   // every warp reduces the warps' boxes itself: one barrier less
+        const bool w = lane < nw;
+        lx = warp_min_f(w ? sm.red[0][lane] : finf());
+        ly = warp_min_f(w ? sm.red[1][lane] : finf());
+        hx = -warp_min_f(w ? -sm.red[2][lane] : finf());
+        hy = -warp_min_f(w ? -sm.red[3][lane] : finf());
+        if (MOVING) vm = -warp_min_f(w ? -sm.red[4][lane] : 0.f);
+    }
+    // square cells over the box; a cloud without a valid point gets one cell
+    const bool any = lx <= hx;
+    if (!any) lx = ly = hx = hy = 0.f;
+    const float w = hx - lx, h = hy - ly, wide = fmaxf(w, h);
+    const float cell = fmaxf(fmaxf(sqrtf(w * (h / kCellTarget)), wide / (float)(kGridDim - 1)), 1e-6f);
+    const float inv = 1.f / cell;
+    const int nx = min(kGridDim, (int)(w * inv) + 1), ny = min(kGridDim, (int)(h * inv) + 1);
+    const int ncell = min(kCells, nx * ny);
+    auto cell_of = [&](float2 p) { return cell_axis(p.y, ly, inv, ny) * nx + cell_axis(p.x, lx, inv, nx); };
+    int rc[kGridRegs], rank[kGridRegs];   // cell, place among its points
+    if (inreg) {
+#pragma unroll
+        for (int k = 0; k < kGridRegs; ++k)
+            if (ok[k]) {
+                rc[k] = min(ncell - 1, cell_of(rp[k]));
+                rank[k] = atomicAdd(&sm.cnt[rc[k]], 1);
+            }
+    } else {
+#pragma unroll 4
+        for (int i = tid; i < N; i += nt) {
+            float2 p, v;
+            if (fetch(i, p, v)) atomicAdd(&sm.cnt[min(ncell - 1, cell_of(p))], 1);
+        }
+    }
+    __syncthreads();
+    // exclusive prefix over the counts: contiguous segments per thread
+    const int per = ((ncell + nt) / nt) | 1, c0 = tid * per, c1 = min(ncell + 1, c0 + per);   // odd: no bank conflicts
+    int s = 0;
+    for (int c = c0; c < c1; ++c) s += sm.cnt[c];
+    int inc = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += t;
+    }
+    if (lane == 31) sm.part[warp] = inc;
+    __syncthreads();
+    {   // the totals of the warps below, again by every warp itself
+        int v = lane < warp ? sm.part[lane] : 0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        int run = v + inc - s;
+        for (int c = c0; c < c1; ++c) {
+            const int n = sm.cnt[c];
+            sm.cnt[c] = run;   // cell ncell holds no point: the number of valid points
+            run += n;
+        }
+    }
+    if (tid == 0) {
+        grid->head = GridHead{lx, ly, inv, cell, fmaxf(fmaxf(fabsf(lx), fabsf(hx)), fmaxf(fabsf(ly), fabsf(hy))),
+                              MOVING ? vm * 1.0001f : 0.f, nx, ny};
+    }
+    __syncthreads();
+    for (int c = tid; c <= ncell; c += nt) grid->start[c] = sm.cnt[c];
+    if (inreg) {
+#pragma unroll
+        for (int k = 0; k < kGridRegs; ++k)
+            if (ok[k]) {
+                const int pos = sm.cnt[rc[k]] + rank[k];
+                opts[pos] = rp[k];
+                if (MOVING) ovel[pos] = rv[k];
+            }
+    } else {
+        __syncthreads();   // the starts are written: the counts may move
+#pragma unroll 4
+        for (int i = tid; i < N; i += nt) {
+            float2 p, v;
+            if (fetch(i, p, v)) {
+                const int pos = atomicAdd(&sm.cnt[min(ncell - 1, cell_of(p))], 1);
+                opts[pos] = p;
+                if (MOVING) ovel[pos] = v;
+            }
+        }
+    }
+}
+
+// ---------------------------------------------------------------- sample phase
+// One block takes up to kGroup samples of a scene at a time: one warp each
+// rolls them out, then all warps share out the (sample, step) slots, a few
+// steps at a time from a shared counter (a sample that drives through a wall
+// has thousands of near points, its neighbour none), then one warp each forms
+// the J~.
+constexpr int kGroup = 8;
+constexpr int kRuns = 64;     // a warp's queued runs: 32 are handled at a time, at most 31 stay
+constexpr int kEvals = 128;   // a warp's queued points: 64 are evaluated at a time, at most 63 stay
+constexpr int kLongRun = 40;  // points from which a run is taken by itself
+constexpr int kField = 32;    // cells of the footprint's distance field along one axis
+__host__ __device__ constexpr int grid_T_pad(int T) { return (T + 3) / 4 * 4; }
+__host__ __device__ constexpr size_t grid_smem_bytes(int T, int samples, int warps) {
+    return kField * kField * 4 + (size_t)grid_T_pad(T) * 32 * samples + kGroup * 4 + (size_t)warps * (kRuns * 12 + kEvals * 8);
+}
+
+// Samples per block: as few as keep the blocks to the three per SM that are
+// resident at once, so that a small sample count still spreads over the GPU.
+inline int grid_group(long long samples, int sms) {
+    const long long slots = 3LL * (sms > 0 ? sms : 148), g = (samples + slots - 1) / slots;
+    return (int)(g < 1 ? 1 : g > kGroup ? kGroup : g);
+}
+
+// The footprint's signed distance at the centres of kField x kField cells over
+// its bounding box grown by d_safe (and the slack): for a point in a cell the
+// distance is within rd (half the cell's diagonal, and a slack far above
+// rounding) of the centre's, because every signed distance is 1-Lipschitz.
+// So one shared-memory read bounds a point's distance from both sides: the
+// smallest upper bound of a step's points replaces d_safe as what still
+// matters, and only the points whose lower bound is below it are evaluated
+// (a few per step, whatever the number of points inside the footprint).
+struct Field {
+    float x0, y0, ix, iy, rd;
+};
+template <class EV>
+__device__ __forceinline__ Field make_field(const EV &ev, float cap) {
+    const float4 fb = ev.box();
+    const float hx = fb.z + cap + 2.f * kPruneSlack, hy = fb.w + cap + 2.f * kPruneSlack;
+    const float cx = 2.f * hx / kField, cy = 2.f * hy / kField;
+    return Field{fb.x - hx, fb.y - hy, 1.f / cx, 1.f / cy, fmaf(0.50001f, sqrtf(fmaf(cx, cx, cy * cy)), 0.1f * kPruneSlack)};
+}
+template <class EV>
+__device__ __forceinline__ void fill_field(const EV &ev, const Field &f, float *field) {
+    const float cx = 1.f / f.ix, cy = 1.f / f.iy;
+    for (int i = 2 * threadIdx.x; i < kField * kField; i += 2 * blockDim.x) {
+        const float x = fmaf((float)(i % kField) + 0.5f, cx, f.x0), y = fmaf((float)(i / kField) + 0.5f, cy, f.y0);
+        float k0, k1;
+        ev.eval2(x, y, x + cx, y, k0, k1);
+        *reinterpret_cast<float2 *>(field + i) = make_float2(ev.dist(k0), ev.dist(k1));
+    }
+}
+
+// Samples [r0, r0 + ns) of a scene, ns <= kGroup; every thread of the block
+// calls.  mem holds grid_smem_bytes(V.P.T, ns, warps) bytes, first the
+// footprint's distance field (filled here when fill is set), and next is a
+// shared counter.  The keys are the same bits whatever warp takes a slot.
+template <bool MOVING, class EV>
+__device__ __forceinline__ void grid_samples(const SceneView &V, const CloudGrid *grid, GridStride gst, const EV &ev,
+                                             int r0, int ns, char *mem, bool fill, int *next) {
+    const MppiP &P = V.P;
+    const int T = P.T, nu = P.nu, Tp = grid_T_pad(T), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nwarps = blockDim.x >> 5;
+    const unsigned full = 0xffffffffu;
+    // per slot (sample s, step h) = s Tp + h
+    float *field = reinterpret_cast<float *>(mem);
+    float4 *pose = reinterpret_cast<float4 *>(field + kField * kField);
+    unsigned *key = reinterpret_cast<unsigned *>(pose + ns * Tp);   // minimum order key
+    unsigned *lim = key + ns * Tp;                                  // f2ord of the distance that still matters
+    float *stage = reinterpret_cast<float *>(lim + ns * Tp);                                   // stage cost without the obstacle term
+    float *time = stage + ns * Tp;                                  // time of the scored state
+    float *term = time + ns * Tp;                                   // per sample: terminal cost
+    // this warp's queues: points to evaluate (slot, point); runs of points (slot, first, count)
+    char *own = reinterpret_cast<char *>(term + kGroup) + warp * (kRuns * 12 + kEvals * 8);
+    int2 *eval = reinterpret_cast<int2 *>(own);
+    int *run_p = reinterpret_cast<int *>(eval + kEvals), *run_n = run_p + kRuns, *run_s = run_n + kRuns;
+    const float cap = fmaxf(P.d_safe, 0.f);
+    const Field fd = make_field(ev, cap);
+    if (fill) fill_field(ev, fd, field);
+    for (int s = warp; s < ns; s += nwarps) {
+        const int r = r0 + s, off = s * Tp;
+        if (r == 0 && lane == 0 && !(isfinite(V.state[0]) && isfinite(V.state[1]) && isfinite(V.state[2])))
+            report_error(V.err, EXACT_EINVAL);   // a start state the host could not see is not finite
+        const float *U = V.U;
+        const float *eps = V.noise + (size_t)r * T * nu;
+        LaneRollout R;
+        warp_rollout(P, V.state[0], V.state[1], V.state[2],
+                     [&](int h, int j) { return clamp_u(P, j, U[h * nu + j] + eps[h * nu + j]); }, R);
+#pragma unroll
+        for (int e = 0; e < kMaxPerLane; ++e) {
+            const int h = lane * R.per + e;
+            if (e < R.per && h < T) {
+                float sn, cs;
+                sincosf(R.th[e], &sn, &cs);
+                pose[off + h] = make_float4(R.x[e], R.y[e], cs, sn);
+                key[off + h] = f2ord(finf());
+                lim[off + h] = f2ord(cap);
+                time[off + h] = (float)(h + P.state_offset) * P.dt;
+                const float u2 = fmaf(R.u[e][0], R.u[e][0], fmaf(R.u[e][1], R.u[e][1], R.u[e][2] * R.u[e][2]));
+                stage[off + h] = fmaf(P.w_goal, guidance_dist(R.x[e], R.y[e], V.wp, V.W), P.w_ctrl * u2);
+            }
+        }
+        if (lane == 0) term[s] = P.w_term * guidance_dist(R.qTx, R.qTy, V.wp, V.W);
+    }
+    if (threadIdx.x == 0) *next = 0;
+    grid_dep_wait();   // launched early behind the kernel that builds the grid
+    __syncthreads();
+    {
+        const float4 fb = ev.box();
+        int nruns = 0, nev = 0;   // queued runs and points (warp-uniform)
+
+        auto point_at = [&](int i, int slot) -> float2 {
+            float2 o = __ldca(V.pts + i);
+            if constexpr (MOVING) {
+                const float th = time[slot];
+                const float2 v = __ldca(V.vel + i);
+                o = make_float2(fmaf(th, v.x, o.x), fmaf(th, v.y, o.y));
+            }
+            return o;
+        };
+        auto evaluate = [&](int cnt) {   // queued points [0, cnt), cnt <= 64: two per lane
+            __syncwarp();
+            const int a = 2 * lane;
+            if (a < cnt) {
+                const bool two = a + 1 < cnt;
+                const int2 ea = eval[a], eb = two ? eval[a + 1] : ea;
+                const float2 oa = point_at(ea.y, ea.x), ob = point_at(eb.y, eb.x);
+                const float4 pa = pose[ea.x], pb = pose[eb.x];
+                float pxa, pya, pxb, pyb;
+                body_frame(oa.x, oa.y, pa.x, pa.y, pa.z, pa.w, pxa, pya);
+                body_frame(ob.x, ob.y, pb.x, pb.y, pb.z, pb.w, pxb, pyb);
+                float ka, kb;
+                ev.eval2(pxa, pya, pxb, pyb, ka, kb);
+                const unsigned oa2 = f2ord(ka), ob2 = f2ord(kb);
+                if (oa2 < key[ea.x]) atomicMin(key + ea.x, oa2);
+                if (ob2 < key[eb.x]) atomicMin(key + eb.x, ob2);
+            }
+            __syncwarp();
+        };
+        // the points of queued runs [0, n), n <= 32, 64 at a time: those whose
+        // lower bound is below their slot's limit go to the evaluation queue.
+        // A long run is taken by itself, the short ones' points are dealt out
+        // (each lane searches its run in the prefix sums of their lengths)
+        auto walk_runs = [&](int n) {
+            __syncwarp();
+            int cnt = lane < n ? run_n[lane] : 0;
+            const int first = lane < n ? run_p[lane] : 0, rs = lane < n ? run_s[lane] : 0;
+            unsigned longs = __ballot_sync(full, cnt >= kLongRun);
+            const int len = cnt;
+            if (cnt >= kLongRun) cnt = 0;
+            int incl = cnt;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_up_sync(full, incl, o);
+                if (lane >= o) incl += t;
+            }
+            const int off = first - (incl - cnt);   // the run's first point as an offset from the dealt index
+            const int total = __shfl_sync(full, incl, 31);
+            int b = 0, long_p = 0, long_n = 0, long_s = 0;   // dealt points; the long run being taken
+            for (;;) {
+                float lb[2], ub[2], now[2];   // bounds of the distance; the slot's limit
+                int i[2], sl[2];
+                bool in[2], lower = false;
+                if (long_n <= 0 && longs) {
+                    const int l = __ffs(longs) - 1;
+                    longs &= longs - 1u;
+                    long_p = __shfl_sync(full, first, l);
+                    long_n = __shfl_sync(full, len, l);
+                    long_s = __shfl_sync(full, rs, l);
+                }
+                if (long_n > 0) {
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        i[q] = long_p + 32 * q + lane;
+                        sl[q] = long_s;
+                        in[q] = 32 * q + lane < long_n;
+                    }
+                    long_p += 64;
+                    long_n -= 64;
+                } else if (b < total) {
+                    int k[2] = {0, 0};   // the number of runs that end at or before an index
+#pragma unroll
+                    for (int st = 16; st > 0; st >>= 1)
+#pragma unroll
+                        for (int q = 0; q < 2; ++q)
+                            if (__shfl_sync(full, incl, k[q] + st - 1) <= b + 32 * q + lane) k[q] += st;
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) {
+                        i[q] = b + 32 * q + lane + __shfl_sync(full, off, k[q]);
+                        sl[q] = __shfl_sync(full, rs, k[q]);
+                        in[q] = b + 32 * q + lane < total;
+                    }
+                    b += 64;
+                } else {
+                    break;
+                }
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    lb[q] = ub[q] = finf();
+                    now[q] = ord2f(lim[sl[q]]);
+                    if (in[q]) {
+                        const float4 p = pose[sl[q]];
+                        const float2 o = point_at(i[q], sl[q]);
+                        float px, py;
+                        body_frame(o.x, o.y, p.x, p.y, p.z, p.w, px, py);
+                        // cell of the field; a point outside it is farther than d_safe
+                        const float u = (px - fd.x0) * fd.ix, v = (py - fd.y0) * fd.iy;
+                        if (u >= 0.f && u < (float)kField && v >= 0.f && v < (float)kField) {
+                            const float f = field[(int)v * kField + (int)u];
+                            lb[q] = f - fd.rd;
+                            ub[q] = f + fd.rd;
+                        }
+                    }
+                    lower |= ub[q] < now[q];
+                }
+                if (__any_sync(full, lower)) {   // some point's distance is below the limit: it falls
+#pragma unroll
+                    for (int q = 0; q < 2; ++q)
+                        if (ub[q] < now[q]) atomicMin(lim + sl[q], f2ord(ub[q]));
+                    __syncwarp();
+#pragma unroll
+                    for (int q = 0; q < 2; ++q) now[q] = ord2f(*(volatile unsigned *)(lim + sl[q]));
+                }
+                const bool keep[2] = {lb[0] <= now[0], lb[1] <= now[1]};
+                const unsigned b0 = __ballot_sync(full, keep[0]), b1 = __ballot_sync(full, keep[1]);
+                if (b0 | b1) {
+                    const unsigned below = (1u << lane) - 1u;
+                    if (keep[0]) eval[nev + __popc(b0 & below)] = make_int2(sl[0], i[0]);
+                    nev += __popc(b0);
+                    if (keep[1]) eval[nev + __popc(b1 & below)] = make_int2(sl[1], i[1]);
+                    nev += __popc(b1);
+                    if (nev >= 64) {
+                        evaluate(64);
+                        int2 m0 = make_int2(0, 0), m1 = m0;
+                        if (lane < nev - 64) m0 = eval[64 + lane];
+                        if (lane + 32 < nev - 64) m1 = eval[96 + lane];
+                        __syncwarp();
+                        if (lane < nev - 64) eval[lane] = m0;
+                        if (lane + 32 < nev - 64) eval[32 + lane] = m1;
+                        nev -= 64;
+                    }
+                }
+            }
+        };
+
+        // slots in groups of `per` steps of one sample from the shared counter:
+        // about three groups per warp, 4 to 8 steps; 32 / per' lanes share a
+        // step's rows (per' = per rounded up to a power of two)
+        const int per = max(4, min(8, ns * T / (3 * nwarps)));
+        const int groups = (T + per - 1) / per, items = ns * groups;
+        int lg = 5;
+        while ((32 >> lg) < per) --lg;
+        const int lanes = 1 << lg, phase = lane & (lanes - 1);
+        for (;;) {
+            int item = 0;
+            if (lane == 0) item = atomicAdd(next, 1);
+            item = __shfl_sync(full, item, 0);
+            if (item >= items) break;
+            const int sm = item / groups, q = lane >> lg, h = (item - sm * groups) * per + q, slot = sm * Tp + h;
+            RowWalk w;
+            GridHead g;
+            const CloudGrid *gh = grid + h * gst.grids;
+            const int base = h * gst.points;
+            int rows = 0;
+            float reach = kPruneSlack;   // a predicted point may have moved by t_h vmax
+            if (q < per && h < T) {
+                g = load_head(gh);
+                if (MOVING) reach = fmaf(time[slot], g.vmax, reach);
+                w = row_walk(g, pose[slot], fb, cap + reach);
+                rows = walk_rows(w);
+            }
+            for (int k = phase; __any_sync(full, k < rows); k += lanes) {
+                int p0 = 0, p1 = 0;
+                if (k < rows) row_run(g, gh->start, w, walk_row(w, k), ord2f(lim[slot]) + reach, p0, p1);
+                const bool some = p1 > p0;
+                const unsigned b = __ballot_sync(full, some);
+                if (b) {
+                    if (some) {
+                        const int at = nruns + __popc(b & ((1u << lane) - 1u));
+                        run_p[at] = base + p0;
+                        run_n[at] = p1 - p0;
+                        run_s[at] = slot;
+                    }
+                    nruns += __popc(b);
+                    if (nruns >= 32) {
+                        walk_runs(32);
+                        int a = 0, n = 0, c = 0;
+                        if (lane < nruns - 32) { a = run_p[32 + lane]; n = run_n[32 + lane]; c = run_s[32 + lane]; }
+                        __syncwarp();
+                        if (lane < nruns - 32) { run_p[lane] = a; run_n[lane] = n; run_s[lane] = c; }
+                        nruns -= 32;
+                    }
+                }
+            }
+        }
+        if (nruns > 0) walk_runs(nruns);
+        if (nev > 0) evaluate(nev);
+    }
+    __syncthreads();
+    for (int s = warp; s < ns; s += nwarps) {
+        const int off = s * Tp;
+        ff acc{0.f, 0.f};
+        bool unsafe = false;
+        for (int h = lane; h < T; h += 32) {
+            const float kh = ord2f(key[off + h]);
+            const float d = kh == finf() ? finf() : ev.dist(kh);
+            acc = add_phi_obs(P, d, ff_add(acc, stage[off + h]));
+            unsafe |= d < P.d_safe;
+        }
+        acc = warp_sum_ff(acc);
+        const bool chi = __any_sync(full, unsafe);
+        if (lane == 0) finish_cost(V, r0 + s, acc, term[s], chi);
+    }
+}
+
+}  // namespace exact

@@ -22,11 +22,36 @@
 // The footprint constants are kernel parameters (compile-time edge count).
 // No K x T x N intermediate exists; scratch is per-sample J~ / weights,
 // per-block partial sums and per-step nominal data in the context arena.
+// Clouds of 1,024 points or more without a d_min output take another route
+// (mppi_grid.cu): a kernel that sorts the cloud into a cell grid (one block,
+// or one per step for a predicted cloud), a sample kernel whose blocks share
+// out the points near each sample's footprint, the same update, and a
+// validation of one block per step (cloud_grid.cuh).
 // The kernels live in mppi_kernels.cuh; this file instantiates them for
 // static clouds and mppi_predicted.cu for clouds with point velocities.
+#include <algorithm>
+
 #include "mppi_kernels.cuh"
 
 namespace exact {
+
+// One block builds the grid over the cloud (build_grid), or block h the grid
+// over a predicted cloud's positions at step h.
+template <bool MOVING>
+__global__ void __launch_bounds__(kGridThreads)
+cloud_grid_kernel(const float2 *pts, const float2 *vel, const uint8_t *mask, int N, float2 *opts, float2 *ovel,
+                  CloudGrid *grid) {
+    __shared__ GridSmem sm;
+    build_grid<MOVING>(pts, vel, mask, N, opts, ovel, grid, sm);
+}
+__global__ void __launch_bounds__(kGridThreads)
+step_grid_kernel(const float2 *pts, const float2 *vel, const uint8_t *mask, int N, float2 *opts, CloudGrid *grid,
+                 int stride, float dt, int state_offset) {
+    __shared__ GridSmem sm;
+    const int h = blockIdx.x;
+    build_grid<false, true>(pts, vel, mask, N, opts + (size_t)h * stride, nullptr, grid + h, sm,
+                            (float)(h + state_offset) * dt);
+}
 
 // Statistics of the cycle just run (one block, after the validation): the
 // normalised weights' effective sample size, J~ minimum and mean, and the
@@ -108,7 +133,9 @@ extern "C" int exact_ctx_reserve_cloud(exact_ctx *ctx, int max_poses, int max_K,
     if (!ctx || max_poses < 0 || max_K < 0 || max_T < 0 || max_points < 0) return EXACT_EINVAL;
     size_t need = sdf_scratch_bytes(max_poses);
     const size_t m = kArenaHeader + scene_scratch_bytes(max_K, max_T, parts_of(ctx, max_K, max_T)) +
-                     (max_points >= kPruneMin ? cloud_copy_bytes(max_points, true) : 0);
+                     (max_points < kPruneMin ? 0 :
+                      std::max(grid_copy_bytes(max_points, true),
+                               std::min(step_grid_bytes(max_points, max_T), kStepGridBytes)));   // static or predicted
     if (m > need) need = m;
     return ensure_scratch(ctx, need);
 }
@@ -126,11 +153,12 @@ int mppi_step_impl(exact_ctx *ctx, const float *state, const float *cloud, const
     if (rc != EXACT_OK) return rc;
     const MppiP P = to_device_params(params);
     const int parts = parts_of(ctx, P.K, P.T);
-    // without a d_min output the sample phase prunes; it pays when the cloud
-    // is in spatial order, so large clouds get a spatially ordered copy
-    const bool sort = !dmin && n_points >= kPruneMin;
+    // without a d_min output the costs only need the points near the
+    // footprint: clouds of kPruneMin points or more get a cell grid
+    const bool grid = !dmin && n_points >= kPruneMin && n_points <= kGridMaxPoints;
+    const bool steps = grid && velocity && step_grid_bytes(n_points, P.T) <= kStepGridBytes;
     const size_t scene_bytes = kArenaHeader + scene_scratch_bytes(P.K, P.T, parts);
-    rc = ensure_scratch(ctx, scene_bytes + (sort ? cloud_copy_bytes(n_points, velocity != nullptr) : 0));
+    rc = ensure_scratch(ctx, scene_bytes + (!grid ? 0 : steps ? step_grid_bytes(n_points, P.T) : grid_copy_bytes(n_points, velocity != nullptr)));
     if (rc != EXACT_OK) return rc;
     SceneView V;
     V.P = P;
@@ -150,7 +178,7 @@ int mppi_step_impl(exact_ctx *ctx, const float *state, const float *cloud, const
     carve_scene(V, static_cast<char *>(ctx->scratch) + kArenaHeader, P.K, P.T, parts);
     V.upd_chunk = upd_chunk_for(P.K, P.T, P.nu);
     V.upd_blocks = upd_blocks_for(P.K, P.T, P.nu);
-    V.val_chunks = val_chunks_for(n_points);
+    V.val_chunks = val_chunks_for(n_points, grid);
     cudaStream_t st = (cudaStream_t)stream;
     // the per-sample part tickets rearm themselves after each cycle; zero
     // them once whenever the arena layout changes
@@ -159,24 +187,34 @@ int mppi_step_impl(exact_ctx *ctx, const float *state, const float *cloud, const
         if (cudaMemsetAsync(V.tk, 0, (size_t)P.K * sizeof(unsigned), st) != cudaSuccess) return EXACT_ECUDA;
     }
     ctx->mppi_layout = layout;
-    const float4 *cc = nullptr;
-    if (sort) {
+    const int sms = ctx->sm_count > 0 ? ctx->sm_count : current_sm_count();
+    if (grid) {
         char *q = static_cast<char *>(ctx->scratch) + scene_bytes;
-        const size_t pbytes = align_up((size_t)n_points * sizeof(float2), 256);
-        float2 *copy = reinterpret_cast<float2 *>(q);
-        float2 *vcopy = velocity ? reinterpret_cast<float2 *>(q + pbytes) : nullptr;
-        float4 *circ = reinterpret_cast<float4 *>(q + pbytes * (velocity ? 2 : 1));
-        if (velocity)
-            cloud_sort_kernel<true><<<1, kSortThreads, 0, st>>>(V.pts, V.vel, mask, n_points, copy, vcopy, circ);
-        else
-            cloud_sort_kernel<false><<<1, kSortThreads, 0, st>>>(V.pts, nullptr, mask, n_points, copy, nullptr, circ);
+        CloudGrid *g = reinterpret_cast<CloudGrid *>(q);
+        GridStride gst{0, 0};
+        if (steps) {
+            gst = GridStride{1, (int)step_points(n_points)};
+            float2 *copy = reinterpret_cast<float2 *>(q + align_up((size_t)P.T * sizeof(CloudGrid), 256));
+            step_grid_kernel<<<P.T, kGridThreads, 0, st>>>(V.pts, V.vel, mask, n_points, copy, g, gst.points, P.dt,
+                                                           P.state_offset);
+            V.pts = copy;
+            V.vel = nullptr;
+        } else {
+            float2 *copy = reinterpret_cast<float2 *>(q + kGridBytes);
+            float2 *vcopy = velocity ? copy + align_up((size_t)n_points * sizeof(float2), 256) / sizeof(float2) : nullptr;
+            if (velocity)
+                cloud_grid_kernel<true><<<1, kGridThreads, 0, st>>>(V.pts, V.vel, mask, n_points, copy, vcopy, g);
+            else
+                cloud_grid_kernel<false><<<1, kGridThreads, 0, st>>>(V.pts, nullptr, mask, n_points, copy, nullptr, g);
+            V.pts = copy;
+            V.vel = vcopy;
+        }
         if (cudaGetLastError() != cudaSuccess) return EXACT_ECUDA;
-        V.pts = copy;
-        V.vel = vcopy;
         V.mask = nullptr;
-        cc = circ;
+        rc = launch_cycle_grid(V, fp, st, g, gst, sms);
+    } else {
+        rc = launch_cycle(V, fp, st, sms);
     }
-    rc = launch_cycle(V, fp, st, sort, cc, ctx->sm_count > 0 ? ctx->sm_count : current_sm_count());
     if (rc != EXACT_OK || !ctx->stats) return rc;
     cycle_stats_kernel<<<1, 256, 0, st>>>(V.Jt, V.wt, P.K, V.hdr, ctx->d_stats);
     return cuda_status(cudaGetLastError());
@@ -188,17 +226,16 @@ int mppi_step_impl(exact_ctx *ctx, const float *state, const float *cloud, const
 // leaves): those of mppi_points.cu when the cloud is pruned point by point,
 // those of mppi_dense.cu when the sample grid exceeds four blocks per SM;
 // else to the unbounded ones here.
-int launch_cycle(const SceneView &V, const exact_footprint *fp, cudaStream_t st, bool pdl, const float4 *circ,
-                 int sms) {
+int launch_cycle(const SceneView &V, const exact_footprint *fp, cudaStream_t st, int sms) {
     if (sms <= 0) sms = 148;
-    if (V.vel) return launch_cycle_moving(V, fp, st, pdl, circ, sms);
+    if (V.vel) return launch_cycle_moving(V, fp, st, sms);
     const bool small_fp = fp->kind == EXACT_FP_RECTS || fp->n_pad <= 16;
     // small clouds without a d_min output are pruned point by point: little
     // evaluation work is left, and the capped kernel's occupancy wins
     const bool queued = !V.dmin && V.N < kPruneMin;
-    if (small_fp && queued) return launch_cycle_points(V, fp, st, pdl, circ, sms);
-    if (small_fp && (long long)V.P.K * V.parts > 4LL * sms) return launch_cycle_dense(V, fp, st, pdl, circ, sms);
-    return launch_cycle_t<false, 0>(V, fp, st, pdl, circ, sms);
+    if (small_fp && queued) return launch_cycle_points(V, fp, st, sms);
+    if (small_fp && (long long)V.P.K * V.parts > 4LL * sms) return launch_cycle_dense(V, fp, st, sms);
+    return launch_cycle_t<false, 0>(V, fp, st, sms);
 }
 
 }  // namespace exact

@@ -3,11 +3,11 @@
 // and the batched persistent kernels (batched.cu):
 //   sample_body    one sample r: rollout, every (step, point) body-frame
 //                  signed distance, per-step minima, J~ (Sec. III-E, IV-C..E);
-//                  when no d_min output is wanted, points that cannot come
-//                  within d_safe of the footprint are skipped (sub-chunk
-//                  circles, then the footprint's bounding box per point or
-//                  per 16-point fine sub-chunk; per-point circles for small
-//                  clouds)
+//                  when no d_min output is wanted and the cloud has no cell
+//                  grid (cloud_grid.cuh), points that cannot come within
+//                  d_safe of the footprint are skipped (sub-chunk circles,
+//                  then the footprint's bounding box per point; per-point
+//                  circles for small clouds)
 //   update_body    one chunk of samples: weights and weighted clipped noise
 //                  into a partial slot (Alg. 1 step 3)
 //   validate_body  one (step, point chunk) of the nominal: adds the partial
@@ -21,6 +21,7 @@
 // distance), either with compile-time constants or from shared memory.
 #pragma once
 
+#include "grid_walk.cuh"
 #include "internal.h"
 #include "mppi_common.cuh"
 
@@ -102,7 +103,8 @@ cudaError_t launch_dependent(void (*kernel)(KArgs...), unsigned grid, unsigned b
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-inline int val_chunks_for(int N) {
+inline int val_chunks_for(int N, bool grid) {
+    if (grid) return 1;   // one block per step walks the rows near the footprint
     const int np = (N + 1) / 2;
     return np > kValChunkPairs ? (np + kValChunkPairs - 1) / kValChunkPairs : 1;
 }
@@ -305,6 +307,45 @@ struct SmemEval {
     }
 };
 
+// A footprint's terms as the slot table of SmemEval, with its bounds.
+constexpr int kFpSlots = poly_slot_count(EXACT_MAX_POLY_VERTICES);
+struct FpTable {
+    float4 c[kFpSlots];
+    float3 bc;    // bounding circle
+    float2 bh;    // half extents of the bounding box about the circle's centre
+    int kind, n;
+};
+inline FpTable make_table(const exact_footprint *fp) {
+    FpTable t;
+    memset(&t, 0, sizeof t);
+    t.kind = fp->kind;
+    t.n = fp->n_pad;
+    t.bc = make_float3(fp->bcx, fp->bcy, fp->brad);
+    t.bh = make_float2(fp->bhx, fp->bhy);
+    if (fp->kind == EXACT_FP_POLYGON) {
+        const int E = fp->n_pad;
+        float *eyn = reinterpret_cast<float *>(t.c + 3 * E + 1);
+        for (int e = 0; e < E; ++e) {
+            t.c[3 * e] = make_float4(-fp->vx[e], -fp->vx[e], -fp->vy[e], -fp->vy[e]);
+            t.c[3 * e + 1] = make_float4(fp->exn[e], fp->exn[e], -fp->kx[e], -fp->kx[e]);
+            t.c[3 * e + 2] = make_float4(-fp->ex[e], -fp->ex[e], -fp->ey[e], -fp->ey[e]);
+            eyn[e] = fp->eyn[e];
+        }
+        t.c[3 * E] = t.c[0];
+    } else {
+        for (int j = 0; j < fp->n_pad; ++j) t.c[j] = make_float4(fp->cx[j], fp->cy[j], fp->sx[j], fp->sy[j]);
+    }
+    return t;
+}
+// The block's copy of the slots in use; the caller synchronises.
+__device__ __forceinline__ void load_table(float4 *dst, const FpTable &t) {
+    const int n = t.kind == EXACT_FP_POLYGON ? poly_slot_count(t.n) : t.n;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = t.c[i];
+}
+__device__ __forceinline__ SmemEval table_eval(const FpTable &t, const float4 *slots) {
+    return SmemEval{slots, t.kind, t.n, t.bc, t.bh};
+}
+
 // ---------------------------------------------------------------- chunk bounds
 // The staged points are cut into sub-chunks of 64 * ppl consecutive points
 // (ppl pairs per lane of a warp).  For each, circ = (centre, radius, max
@@ -313,21 +354,11 @@ constexpr int kSub = 64;
 constexpr float kPruneSlack = 1e-3f;   // m: far above the float rounding of the distances
 constexpr int kPruneMin = 1024;        // points: smaller clouds are pruned point by point (see steps_min_keys)
 constexpr int kQueueAll = 1024;        // entries of the block's queues of kept (step, point) pairs
-constexpr int kFine = 16;              // points of a fine sub-chunk (a quarter of a sub-chunk)
 // Sample-phase code paths compiled into a kernel: every path (chosen per
 // call), or only the point-level pruning of small clouds (the caller passes
 // no d_min output and fewer than kPruneMin points) -- a smaller kernel whose
 // code each block fetches once per cycle.
 constexpr int kPathAny = 0, kPathPoints = 1;
-constexpr int kQueueFine = 640;        // entries of the block's queues of kept fine sub-chunks
-
-// An ordered cloud of N points carries the circles of its ceil(N / kSub)
-// sub-chunks and, after them (256-byte aligned), those of its ceil(N / kFine)
-// fine sub-chunks.
-__host__ __device__ constexpr int fine_circle_offset(int N) { return (((N + kSub - 1) / kSub) + 15) & ~15; }
-__host__ __device__ constexpr size_t circle_bytes(int N) {
-    return ((size_t)fine_circle_offset(N) + ((((size_t)N + kFine - 1) / kFine + 15) & ~(size_t)15)) * 16u;
-}
 
 template <bool MOVING>
 __device__ __forceinline__ void chunk_circles(const float2 *pts, int n, float4 *circ, int ppl) {
@@ -369,236 +400,7 @@ __device__ __forceinline__ void chunk_circles(const float2 *pts, int n, float4 *
     }
 }
 
-// ---------------------------------------------------------------- cloud order
-// Pruning pays only when 64 consecutive points lie close together.  Scans
-// deliver clouds in that order; for any other order one block rewrites the
-// cloud in Morton order of a 64 x 64 grid over its bounding box (a counting
-// sort: histogram, prefix sum, scatter).  Masked and non-finite points go
-// last, as NaN, so the copy needs no mask.  The order inside a grid cell
-// follows the scatter's atomics; nothing computed from the cloud depends on
-// it (minima over points are exact whatever the order).
-constexpr int kSortCells = 64 * 64;
-constexpr int kSortThreads = 1024;
-constexpr int kSortRegs = 4;   // points per thread kept in registers (clouds of up to 4,096)
-struct SortSmem {
-    int cnt[kSortCells + 1];
-    float red[4][kSortThreads / 32];
-    float box[4];
-    int part[kSortThreads / 32];
-};
-
-__device__ __forceinline__ unsigned morton6(unsigned x, unsigned y) {
-    unsigned r = 0u;
-#pragma unroll
-    for (int b = 0; b < 6; ++b) r |= (((x >> b) & 1u) << (2 * b)) | (((y >> b) & 1u) << (2 * b + 1));
-    return r;
-}
-
-template <bool MOVING>
-__device__ __forceinline__ void sort_cloud_block(const float2 *__restrict__ pts, const float2 *__restrict__ vel,
-                                                 const uint8_t *__restrict__ mask, int N, float2 *__restrict__ opts,
-                                                 float2 *__restrict__ ovel, SortSmem &sm) {
-    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
-    grid_dep_release();   // the sample kernel may start its rollouts meanwhile
-    auto valid = [&](int i, float2 &p) {
-        p = pts[i];
-        return (!mask || mask[i]) && isfinite(p.x) && isfinite(p.y);
-    };
-    // clouds of up to kSortRegs points per thread are read once and kept in
-    // registers (point tid + k nt in slot k); larger ones are re-read per pass
-    const bool inreg = N <= kSortRegs * nt;
-    float2 rp[kSortRegs];
-    bool rv[kSortRegs];
-    if (inreg) {
-#pragma unroll
-        for (int k = 0; k < kSortRegs; ++k) {
-            const int i = tid + k * nt;
-            rv[k] = i < N && valid(i, rp[k]);
-        }
-    }
-    float lx = finf(), ly = finf(), hx = -finf(), hy = -finf();
-    auto grow = [&](float2 p) { lx = fminf(lx, p.x); hx = fmaxf(hx, p.x); ly = fminf(ly, p.y); hy = fmaxf(hy, p.y); };
-    if (inreg) {
-#pragma unroll
-        for (int k = 0; k < kSortRegs; ++k)
-            if (rv[k]) grow(rp[k]);
-    } else {
-        for (int i = tid; i < N; i += nt) {
-            float2 p;
-            if (valid(i, p)) grow(p);
-        }
-    }
-    lx = warp_min_f(lx); ly = warp_min_f(ly); hx = -warp_min_f(-hx); hy = -warp_min_f(-hy);
-    if (lane == 0) { sm.red[0][warp] = lx; sm.red[1][warp] = ly; sm.red[2][warp] = hx; sm.red[3][warp] = hy; }
-    for (int c = tid; c <= kSortCells; c += nt) sm.cnt[c] = 0;
-    __syncthreads();
-    if (warp == 0) {   // the warps' boxes, reduced by one warp
-        const bool w = lane < nw;
-        lx = warp_min_f(w ? sm.red[0][lane] : finf());
-        ly = warp_min_f(w ? sm.red[1][lane] : finf());
-        hx = -warp_min_f(w ? -sm.red[2][lane] : finf());
-        hy = -warp_min_f(w ? -sm.red[3][lane] : finf());
-        if (lane == 0) { sm.box[0] = lx; sm.box[1] = ly; sm.box[2] = hx; sm.box[3] = hy; }
-    }
-    __syncthreads();
-    lx = sm.box[0]; ly = sm.box[1]; hx = sm.box[2]; hy = sm.box[3];
-    const float sx = 64.f / fmaxf(hx - lx, 1e-6f), sy = 64.f / fmaxf(hy - ly, 1e-6f);
-    auto cell_of = [&](bool ok, float2 p) -> int {
-        if (!ok) return kSortCells;
-        const int qx = min(63, max(0, (int)((p.x - lx) * sx))), qy = min(63, max(0, (int)((p.y - ly) * sy)));
-        return (int)morton6((unsigned)qx, (unsigned)qy);
-    };
-    int rc[kSortRegs];
-    if (inreg) {
-#pragma unroll
-        for (int k = 0; k < kSortRegs; ++k) {
-            rc[k] = cell_of(rv[k], rp[k]);
-            if (tid + k * nt < N) atomicAdd(&sm.cnt[rc[k]], 1);
-        }
-    } else {
-        for (int i = tid; i < N; i += nt) {
-            float2 p;
-            const bool ok = valid(i, p);
-            atomicAdd(&sm.cnt[cell_of(ok, p)], 1);
-        }
-    }
-    __syncthreads();
-    // exclusive prefix over the kSortCells + 1 counts: contiguous segments per thread
-    const int per = (kSortCells + 1 + nt - 1) / nt, c0 = tid * per, c1 = min(kSortCells + 1, c0 + per);
-    int s = 0;
-    for (int c = c0; c < c1; ++c) s += sm.cnt[c];
-    int inc = s;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += t;
-    }
-    if (lane == 31) sm.part[warp] = inc;
-    __syncthreads();
-    if (warp == 0) {   // exclusive prefix of the warps' totals, by one warp
-        const int v = lane < nw ? sm.part[lane] : 0;
-        int x = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += t;
-        }
-        __syncwarp();
-        if (lane < nw) sm.part[lane] = x - v;
-    }
-    __syncthreads();
-    const int base = sm.part[warp];
-    int run = base + inc - s;
-    for (int c = c0; c < c1; ++c) {
-        const int v = sm.cnt[c];
-        sm.cnt[c] = run;
-        run += v;
-    }
-    __syncthreads();
-    const float qnan = __int_as_float(0x7fffffff);
-    auto place = [&](int i, int c, float2 p) {
-        const int pos = atomicAdd(&sm.cnt[c], 1);
-        opts[pos] = c < kSortCells ? p : make_float2(qnan, qnan);
-        if (MOVING) ovel[pos] = c < kSortCells ? vel[i] : make_float2(0.f, 0.f);
-    };
-    if (inreg) {
-#pragma unroll
-        for (int k = 0; k < kSortRegs; ++k) {
-            const int i = tid + k * nt;
-            if (i < N) place(i, rc[k], rp[k]);
-        }
-    } else {
-        for (int i = tid; i < N; i += nt) {
-            float2 p;
-            const bool ok = valid(i, p);
-            place(i, cell_of(ok, p), p);
-        }
-    }
-}
-
-// Bounding circles (centre, radius, max speed) of the 64-point sub-chunks of
-// an ordered cloud in global memory, one warp per sub-chunk; the same values
-// chunk_circles computes for one staged pass, computed once per cycle.  The
-// circles of the 16-point fine sub-chunks (same construction over a half
-// warp's points) follow at circ + fine_circle_offset(N).
-template <bool MOVING>
-__device__ __forceinline__ void cloud_circles(const float2 *__restrict__ pts, const float2 *__restrict__ vel, int N,
-                                              float4 *__restrict__ circ) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const int nsub = (N + kSub - 1) / kSub;
-    for (int s = warp; s < nsub; s += nwarps) {
-        float x[2], y[2], v2 = 0.f;
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const int i = s * kSub + k * 32 + lane;
-            x[k] = y[k] = __int_as_float(0x7fffffff);
-            if (i < N) {
-                x[k] = pts[i].x; y[k] = pts[i].y;
-                if (MOVING && x[k] == x[k]) v2 = fmaxf(v2, fmaf(vel[i].x, vel[i].x, vel[i].y * vel[i].y));
-            }
-        }
-        float lx = warp_min_f(fminf(x[0], x[1])), ly = warp_min_f(fminf(y[0], y[1]));
-        float hx = -warp_min_f(-fmaxf(x[0], x[1])), hy = -warp_min_f(-fmaxf(y[0], y[1]));
-        const bool any = lx <= hx;
-        const float cx = 0.5f * (lx + hx), cy = 0.5f * (ly + hy);
-        float r2 = 0.f;
-#pragma unroll
-        for (int k = 0; k < 2; ++k)
-            if (x[k] == x[k]) r2 = fmaxf(r2, fmaf(x[k] - cx, x[k] - cx, (y[k] - cy) * (y[k] - cy)));
-        r2 = -warp_min_f(-r2);
-        if (MOVING) v2 = -warp_min_f(-v2);
-        if (lane == 0)
-            circ[s] = any ? make_float4(cx, cy, sqrtf(r2) * 1.000001f, MOVING ? sqrtf(v2) * 1.000001f : 0.f)
-                          : make_float4(0.f, 0.f, -1.f, 0.f);
-        // fine sub-chunk 2k + (lane >> 4): points k * 32 + lane of this sub-chunk
-        float4 *fine = circ + fine_circle_offset(N);
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            float flx = x[k], fly = y[k], fhx = x[k], fhy = y[k], fv2 = 0.f;
-            if (MOVING && x[k] == x[k]) {
-                const int i = s * kSub + k * 32 + lane;
-                fv2 = fmaf(vel[i].x, vel[i].x, vel[i].y * vel[i].y);
-            }
-#pragma unroll
-            for (int o = 8; o > 0; o >>= 1) {   // within each half warp; NaN (masked, absent) ignored
-                flx = fminf(flx, __shfl_xor_sync(0xffffffffu, flx, o));
-                fly = fminf(fly, __shfl_xor_sync(0xffffffffu, fly, o));
-                fhx = fmaxf(fhx, __shfl_xor_sync(0xffffffffu, fhx, o));
-                fhy = fmaxf(fhy, __shfl_xor_sync(0xffffffffu, fhy, o));
-                if (MOVING) fv2 = fmaxf(fv2, __shfl_xor_sync(0xffffffffu, fv2, o));
-            }
-            const bool fany = flx <= fhx;
-            const float fcx = 0.5f * (flx + fhx), fcy = 0.5f * (fly + fhy);
-            float fr2 = x[k] == x[k] ? fmaf(x[k] - fcx, x[k] - fcx, (y[k] - fcy) * (y[k] - fcy)) : 0.f;
-#pragma unroll
-            for (int o = 8; o > 0; o >>= 1) fr2 = fmaxf(fr2, __shfl_xor_sync(0xffffffffu, fr2, o));
-            const int f = s * (kSub / kFine) + 2 * k + (lane >> 4);
-            if ((lane & 15) == 0 && f * kFine < N)
-                fine[f] = fany ? make_float4(fcx, fcy, sqrtf(fr2) * 1.000001f, MOVING ? sqrtf(fv2) * 1.000001f : 0.f)
-                               : make_float4(0.f, 0.f, -1.f, 0.f);
-        }
-    }
-}
-
 // ---------------------------------------------------------------- sample phase
-// Position of the k-th (from 0) set bit of m; k < popc(m).
-__device__ __forceinline__ int nth_set_bit64(unsigned long long m, int k) {
-    int pos = 0;
-#pragma unroll
-    for (int w = 32; w > 0; w >>= 1) {
-        const unsigned long long low = m & ((1ull << w) - 1ull);
-        const int c = __popcll(low);
-        if (k >= c) {
-            k -= c;
-            m >>= w;
-            pos += w;
-        } else {
-            m = low;
-        }
-    }
-    return pos;
-}
-
 // Per-step minimum of the body-frame key over n staged points for the steps
 // [h0, h0 + nh) whose poses are in shared memory.  Masked points were staged
 // as NaN, which every evaluator turns into a +inf key (NaN terms are dropped
@@ -618,11 +420,8 @@ __device__ __forceinline__ int nth_set_bit64(unsigned long long m, int k) {
 //     sub-chunk) list; polygons and shared-memory footprints keep the points
 //     that lie within cap of the footprint's bounding box in that step's
 //     body frame and evaluate them through the warp's queue (queue:
-//     kQueueAll ints of shared memory); rectangle covers keep the 16-point
-//     fine sub-chunks whose circles (circf, from the ordered cloud) come
-//     within cap of that box and evaluate them through the queue qfine
-//     (kQueueFine ints), or, without fine circles, evaluate every point and
-//     fold each step's minimum into keyh[h] (one warp shuffle-min and one
+//     kQueueAll ints of shared memory); rectangle covers evaluate every point
+//     and fold each step's minimum into keyh[h] (one warp shuffle-min and one
 //     shared atomicMin per step run).
 // With queue_points (clouds below kPruneMin) the phases are replaced by a
 // point-level test against the footprint's bounding circle, feeding the
@@ -636,8 +435,7 @@ template <bool MOVING = false, int PATH = kPathAny, class EV>
 __device__ __forceinline__ void steps_min_keys(const EV &ev, const float2 *pts, int n, const float4 *pose,
                                                const float4 *cw, int h0, int nh, unsigned *keyh, int ppl,
                                                const float4 *circ, float cap, unsigned *msk, int *pre,
-                                               int *queue, bool queue_points, const float4 *circf, int *qfine,
-                                               int *err = nullptr) {
+                                               int *queue, bool queue_points, int *err = nullptr) {
     const int npairs = (n + 1) >> 1;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int nsub = (n + kSub * ppl - 1) / (kSub * ppl);
@@ -981,101 +779,6 @@ __device__ __forceinline__ void steps_min_keys(const EV &ev, const float2 *pts, 
                 if (!more && qn == 0) return;
             }
         }
-        if (circf) {
-            // Rectangle covers with the fine circles of an ordered cloud: the
-            // four 16-point fine sub-chunks of every kept (step, sub-chunk) entry
-            // are tested against the footprint's bounding box in the step's body
-            // frame (one lane per fine sub-chunk, eight entries per warp
-            // iteration, each lane decoding its own entry from pre and msk); the
-            // kept ones go through the warp's queue and are evaluated four at a
-            // time, eight lanes (one pair each) per fine sub-chunk, whose step
-            // minimum is folded over the eight lanes and into keyh[h] with one
-            // shared atomicMin.  Every point of a fine sub-chunk lies within its
-            // circle (radius grown by t_h times its largest speed when MOVING),
-            // sd_F >= sd_box for a footprint F inside the box, and sd_box is
-            // 1-Lipschitz, so a dropped fine sub-chunk holds no point within cap.
-            const float4 fb = ev.box();
-            const int capf = kQueueFine / nwarps;   // >= 40 for up to 16 warps: 3 left + 32 added fit
-            int *q = qfine + warp * capf;
-            int qn = 0;   // warp-uniform
-            const int nfine = (n + kFine - 1) / kFine;
-            for (int e = e0;; e += 8) {
-                const bool more = e < e1;
-                const int my = e + (lane >> 2);
-                bool keep = false;
-                int code = 0;
-                if (more && my < e1) {
-                    int lo = 0, hi = nh - 1;   // the step holding entry my: the last with pre <= my
-                    while (lo < hi) {
-                        const int mid = (lo + hi + 1) >> 1;
-                        if (pre[mid] <= my) lo = mid; else hi = mid - 1;
-                    }
-                    const unsigned long long mm = ((unsigned long long)msk[2 * lo + 1] << 32) | msk[2 * lo];
-                    const int fi = nth_set_bit64(mm, my - pre[lo]) * (kSub / kFine) + (lane & 3);
-                    if (fi < nfine) {
-                        const float4 c = circf[fi];
-                        if (c.z >= 0.f) {
-                            const float4 qp = pose[h0 + lo];
-                            float px, py;
-                            body_frame(c.x, c.y, qp.x, qp.y, qp.z, qp.w, px, py);
-                            float reach = c.z + 1e-5f * (fabsf(c.x) + fabsf(c.y) + fabsf(qp.x) + fabsf(qp.y));
-                            if (MOVING) reach = fmaf(cw[h0 + lo].z, c.w, reach);
-                            const float l = reach + lim;
-                            const float ax = fabsf(px - fb.x) - fb.z, ay = fabsf(py - fb.y) - fb.w;
-                            const float mx = fmaxf(ax, 0.f), my2 = fmaxf(ay, 0.f);
-                            keep = ax <= l && ay <= l && fmaf(mx, mx, my2 * my2) <= l * l;
-                        }
-                    }
-                    code = (lo << 12) | fi;
-                }
-                const unsigned b = __ballot_sync(0xffffffffu, keep);
-                if (keep) q[qn + __popc(b & ((1u << lane) - 1u))] = code;
-                qn += __popc(b);
-                while (qn >= 4 || (!more && qn > 0)) {
-                    // evaluate entries [0, f), f <= 4, and move the rest to the front
-                    const int f = min(qn, 4);
-                    __syncwarp();
-                    const int slot = lane >> 3, pr = lane & 7;
-                    float best = finf();
-                    int sh = 0;
-                    if (slot < f) {
-                        int ce = q[slot];
-                        if (!EXACT_DCHECK((ce >> 12) < nh && (ce & 4095) < nfine, err)) ce = 0;   // debug build: skip
-                        sh = ce >> 12;
-                        const int j = (ce & 4095) * (kFine / 2) + pr;   // pair j of the staged points
-                        if (j < npairs) {
-                            const int h = h0 + sh;
-                            const float4 qp = pose[h];
-                            float2 o0, o1;
-                            if constexpr (MOVING) {
-                                const float th = cw[h].z;
-                                const float4 *p4 = reinterpret_cast<const float4 *>(pts);
-                                const float4 a0 = p4[2 * j], a1 = p4[min(2 * j + 1, n - 1)];
-                                o0 = make_float2(fmaf(th, a0.z, a0.x), fmaf(th, a0.w, a0.y));
-                                o1 = make_float2(fmaf(th, a1.z, a1.x), fmaf(th, a1.w, a1.y));
-                            } else {
-                                o0 = pts[2 * j];
-                                o1 = pts[min(2 * j + 1, n - 1)];
-                            }
-                            float px0, py0, px1, py1;
-                            body_frame(o0.x, o0.y, qp.x, qp.y, qp.z, qp.w, px0, py0);
-                            body_frame(o1.x, o1.y, qp.x, qp.y, qp.z, qp.w, px1, py1);
-                            float k0, k1;
-                            ev.eval2(px0, py0, px1, py1, k0, k1);
-                            best = fminf(k0, k1);
-                        }
-                    }
-    #pragma unroll
-                    for (int o = 4; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
-                    if (slot < f && pr == 0 && best < finf()) atomicMin(keyh + h0 + sh, f2ord(best));
-                    __syncwarp();
-                    for (int i = lane; i < qn - f; i += 32) q[i] = q[f + i];
-                    __syncwarp();
-                    qn -= f;
-                }
-                if (!more) return;
-            }
-        }
         float best = finf();
         for (int e = e0; e < e1; ++e) {
             if (!EXACT_DCHECK(hh < nh, err)) break;
@@ -1238,15 +941,22 @@ __device__ __forceinline__ ff add_phi_obs(const MppiP &P, float d, ff acc) {
     return acc;
 }
 
+// J~ = J + w_inf I(chi) (Sec. IV-E) of sample r, summed as a float-float and
+// kept as a double; beta = min J~ is gathered with one 64-bit atomic per
+// sample into the scene's header (complemented key; 0 = empty).
+__device__ __forceinline__ void finish_cost(const SceneView &V, int r, ff acc, float term, bool chi) {
+    acc = ff_add(acc, term);
+    if (chi) acc = ff_add(acc, V.P.w_inf);
+    const double jt = ff_to_d(acc);
+    V.Jt[r] = jt;
+    atomicMax(&V.hdr->beta_enc, ~d2ord(jt));
+}
+
 struct SampleSmem {
     float4 circ[kStage / kSub];            // sub-chunk bounding circles
     unsigned msk[2 * EXACT_MAX_HORIZON];   // kept (step, sub-chunk) pairs, 64 bits per step
     int pre[EXACT_MAX_HORIZON + 1];        // exclusive prefix of their counts
-    union {
-        int queue[kQueueAll];              // per-warp queues of kept (step, point) entries
-        float4 circf[kStage / kFine];      // fine sub-chunk circles (rectangle covers)
-    };
-    int qfine[kQueueFine];                 // per-warp queues of kept (step, fine sub-chunk) entries
+    int queue[kQueueAll];                  // per-warp queues of kept (step, point) entries
     float4 cw[EXACT_MAX_HORIZON];      // footprint circle centre (world) and t_h per step
     float4 pose[EXACT_MAX_HORIZON];
     float stage[EXACT_MAX_HORIZON];
@@ -1276,9 +986,6 @@ __device__ __forceinline__ void sample_smem_init(SampleSmem &sm) {
 // order), so the split never changes a bit of the result.  Ends with a
 // __syncthreads.  MOVING: V.vel holds the points' velocities and every step
 // sees the predicted cloud (see steps_min_keys).
-// circ: bounding circles of the 64-point sub-chunks of an ordered cloud
-// (cloud_circles), or NULL.  (Kept out of SceneView: a larger SceneView
-// parameter block made the compiler spill in the large-footprint kernels.)
 // r2 >= 0: the block takes a second sample r2 of the same scene (parts == 1,
 // 2T <= EXACT_MAX_HORIZON, blockDim >= 96): warps 0 and 1 roll the two out
 // side by side, the per-step slots hold sample r's steps then r2's (slot
@@ -1287,8 +994,7 @@ __device__ __forceinline__ void sample_smem_init(SampleSmem &sm) {
 // one-sample path.
 template <bool MOVING = false, int PATH = kPathAny, class EV>
 __device__ __forceinline__ void sample_body(const SceneView &V, const EV &ev, int r, int p, SampleSmem &sm,
-                                            float2 *s_pts, bool staged, int pairs_per_lane,
-                                            const float4 *circ = nullptr, int r2 = -1) {
+                                            float2 *s_pts, bool staged, int pairs_per_lane, int r2 = -1) {
     const MppiP &P = V.P;
     const int T = P.T, nu = P.nu, N = V.N;
     constexpr int kS = stage_points_of<MOVING>();
@@ -1334,20 +1040,8 @@ __device__ __forceinline__ void sample_body(const SceneView &V, const EV &ev, in
     }
     __syncthreads();
     const bool prune = PATH == kPathAny && !V.dmin && N >= kPruneMin;
-    // sub-chunk circles: copied from the ordered cloud's (64-point sub-chunks),
-    // or computed from the staged points
-    const bool pre_circ = circ != nullptr && pairs_per_lane == 1;
-    // rectangle covers test the fine sub-chunks of the kept sub-chunks too
-    // (polygons test single points instead; see steps_min_keys)
-    const bool fine = pre_circ && !EV::kBoxTest;
-    const float4 *circ_f = fine ? circ + fine_circle_offset(N) : nullptr;
     if (!staged && prune) {
-        if (pre_circ)
-            for (int s = threadIdx.x; s < (n0 + kSub - 1) / kSub; s += blockDim.x) sm.circ[s] = circ[s];
-        else
-            chunk_circles<MOVING>(s_pts, n0, sm.circ, pairs_per_lane);
-        if (fine)
-            for (int s = threadIdx.x; s < (n0 + kFine - 1) / kFine; s += blockDim.x) sm.circf[s] = circ_f[s];
+        chunk_circles<MOVING>(s_pts, n0, sm.circ, pairs_per_lane);
         __syncthreads();
     }
     // without a d_min output the costs only need min(d_min, d_safe): far
@@ -1355,8 +1049,7 @@ __device__ __forceinline__ void sample_body(const SceneView &V, const EV &ev, in
     // clouds, one pass) are skipped
     const float cap = V.dmin ? -1.f : fmaxf(P.d_safe, 0.f);
     steps_min_keys<MOVING, PATH>(ev, s_pts, n0, sm.pose, sm.cw, k0, nk, sm.key, pairs_per_lane, sm.circ, cap, sm.msk,
-                                 sm.pre, sm.queue, !V.dmin && N < kPruneMin, fine ? sm.circf : nullptr, sm.qfine,
-                                 V.err);
+                                 sm.pre, sm.queue, !V.dmin && N < kPruneMin, V.err);
     if constexpr (PATH == kPathAny) for (int base = kS; base < N; base += kS) {   // clouds larger than the stage
         const int n = min(kS, N - base);
         __syncthreads();
@@ -1364,17 +1057,11 @@ __device__ __forceinline__ void sample_body(const SceneView &V, const EV &ev, in
                              V.err);
         __syncthreads();
         if (prune) {
-            if (pre_circ)
-                for (int s = threadIdx.x; s < (n + kSub - 1) / kSub; s += blockDim.x) sm.circ[s] = circ[base / kSub + s];
-            else
-                chunk_circles<MOVING>(s_pts, n, sm.circ, pairs_per_lane);
-            if (fine)
-                for (int s = threadIdx.x; s < (n + kFine - 1) / kFine; s += blockDim.x)
-                    sm.circf[s] = circ_f[base / kFine + s];
+            chunk_circles<MOVING>(s_pts, n, sm.circ, pairs_per_lane);
             __syncthreads();
         }
         steps_min_keys<MOVING>(ev, s_pts, n, sm.pose, sm.cw, k0, nk, sm.key, pairs_per_lane, sm.circ, cap, sm.msk,
-                               sm.pre, sm.queue, false, fine ? sm.circf : nullptr, sm.qfine, V.err);
+                               sm.pre, sm.queue, false, V.err);
     }
     grid_dep_release();
     __syncthreads();
@@ -1403,17 +1090,7 @@ __device__ __forceinline__ void sample_body(const SceneView &V, const EV &ev, in
         }
         acc = warp_sum_ff(acc);
         const bool chi = __any_sync(0xffffffffu, unsafe);
-        if (lane == 0) {
-            // J~ = J + w_inf I(chi) (Sec. IV-E), summed as a float-float and
-            // kept as a double; beta = min J~ is gathered with one 64-bit
-            // atomic per sample into the scene's header (complemented key;
-            // 0 = empty)
-            acc = ff_add(acc, sm.term[warp]);
-            if (chi) acc = ff_add(acc, P.w_inf);
-            const double jt = ff_to_d(acc);
-            V.Jt[rs] = jt;
-            atomicMax(&V.hdr->beta_enc, ~d2ord(jt));
-        }
+        if (lane == 0) finish_cost(V, rs, acc, sm.term[warp], chi);
     }
     __syncthreads();
 }
@@ -1521,7 +1198,7 @@ struct ValidateSmem {
 // J_m of Algorithm 2) and empties the step keys.
 template <bool MOVING = false, class EV>
 __device__ __forceinline__ void validate_body(const SceneView &V, const EV &ev, int h, int c, ValidateSmem &sm,
-                                              const float4 *circ = nullptr) {
+                                              const CloudGrid *grid = nullptr, int first = 0) {
     const MppiP &P = V.P;
     const int K = P.K, T = P.T, nu = P.nu, TN = T * nu, G = V.upd_blocks;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1588,30 +1265,15 @@ __device__ __forceinline__ void validate_body(const SceneView &V, const EV &ev, 
     }
     __syncthreads();
     const float4 qp = sm.pose;
-    const int N = V.N;
-    const int npairs = (N + 1) >> 1;
-    const int pend = min(npairs, (c + 1) * kValChunkPairs);
+    const int N = V.N, pend = min((N + 1) >> 1, (c + 1) * kValChunkPairs);
     const float th = (float)(h + P.state_offset) * P.dt;   // time of the scored state (MOVING)
-    // ordered clouds: skip 64-point sub-chunks farther than d_safe from the
-    // footprint (the validation and the nominal's cost only need min(d, d_safe))
-    const float3 bc = ev.bound();
-    const float cwx = fmaf(qp.z, bc.x, fmaf(-qp.w, bc.y, qp.x)), cwy = fmaf(qp.w, bc.x, fmaf(qp.z, bc.y, qp.y));
-    const float vlim = fmaxf(P.d_safe, 0.f) + kPruneSlack + 1e-5f * (fabsf(cwx) + fabsf(cwy));
     float best = finf();
-    for (int j = c * kValChunkPairs + tid; j < pend; j += kBlock) {
-        if (circ) {   // warp-uniform: the warp's 32 pairs are sub-chunk j / 32
-            const float4 cc = __ldg(circ + (j >> 5));
-            const float dx = cc.x - cwx, dy = cc.y - cwy;
-            float reach = cc.z + bc.z + 1e-5f * (fabsf(cc.x) + fabsf(cc.y));
-            if (MOVING) reach = fmaf(th, cc.w, reach);
-            const float far = reach + vlim;
-            if (cc.z < 0.f || fmaf(dx, dx, dy * dy) > far * far) continue;
-        }
-        const int i0 = 2 * j, i1 = min(2 * j + 1, N - 1);
-        float2 o0 = __ldg(V.pts + i0);
-        float2 o1 = __ldg(V.pts + i1);
+    // points 2j and 2j + 1 of the pair (i0, i1) folded into the minimum
+    auto take = [&](int i0, int i1) {
+        float2 o0 = __ldca(V.pts + i0);
+        float2 o1 = __ldca(V.pts + i1);
         if constexpr (MOVING) {
-            const float2 v0 = __ldg(V.vel + i0), v1 = __ldg(V.vel + i1);
+            const float2 v0 = __ldca(V.vel + i0), v1 = __ldca(V.vel + i1);
             o0 = make_float2(fmaf(th, v0.x, o0.x), fmaf(th, v0.y, o0.y));
             o1 = make_float2(fmaf(th, v1.x, o1.x), fmaf(th, v1.y, o1.y));
         }
@@ -1625,6 +1287,43 @@ __device__ __forceinline__ void validate_body(const SceneView &V, const EV &ev, 
             k1 = __ldg(V.mask + i1) ? k1 : finf();
         }
         best = fmin3(best, k0, k1);
+    };
+    // with a grid (one block per step) the block's warps share out the rows
+    // near the footprint: the validation and the nominal's cost only need
+    // min(d, d_safe); without one every point of the block's chunk is taken
+    int j = c * kValChunkPairs + tid, i = 0, iend = 0;
+    RowWalk w = {};
+    GridHead g = {};
+    float lim = 0.f;
+    int row = warp, rows = 0;
+    if (grid) {
+        g = load_head(grid);
+        lim = fmaxf(P.d_safe, 0.f) + kPruneSlack;
+        if (MOVING) lim = fmaf(th, g.vmax, lim);
+        w = row_walk(g, qp, ev.box(), lim);
+        rows = walk_rows(w);
+    }
+    for (;;) {   // one evaluator call site for both
+        int i0, i1;
+        if (grid) {
+            while (i >= iend && row < rows) {   // warp-uniform: the next row's run of points
+                row_run(g, grid->start, w, walk_row(w, row), lim, i, iend);
+                i += first;
+                iend += first;
+                row += kBlock / 32;
+            }
+            if (i >= iend) break;
+            i0 = i + 2 * lane;
+            i1 = min(i0 + 1, iend - 1);
+            i += 64;
+            if (i0 > i1) continue;
+        } else {
+            if (j >= pend) break;
+            i0 = 2 * j;
+            i1 = min(2 * j + 1, N - 1);
+            j += kBlock;
+        }
+        take(i0, i1);
     }
     best = warp_min_f(best);
     if (lane == 0) sm.mn[warp] = best;

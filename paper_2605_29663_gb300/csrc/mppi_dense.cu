@@ -6,9 +6,8 @@
 
 namespace exact {
 
-int launch_cycle_dense(const SceneView &V, const exact_footprint *fp, cudaStream_t st, bool pdl,
-                       const float4 *circ, int sms) {
-    return launch_cycle_t<false, 4>(V, fp, st, pdl, circ, sms);
+int launch_cycle_dense(const SceneView &V, const exact_footprint *fp, cudaStream_t st, int sms) {
+    return launch_cycle_t<false, 4>(V, fp, st, sms);
 }
 
 }  // namespace exact

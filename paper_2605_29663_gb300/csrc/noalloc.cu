@@ -15,8 +15,7 @@
 namespace exact {
 int check_params(const exact_mppi_params *p);
 MppiP to_device_params(const exact_mppi_params *p);
-int launch_cycle(const SceneView &V, const exact_footprint *fp, cudaStream_t st, bool pdl, const float4 *circ,
-                 int sms);
+int launch_cycle(const SceneView &V, const exact_footprint *fp, cudaStream_t st, int sms);
 }  // namespace exact
 
 using namespace exact;
@@ -87,11 +86,11 @@ extern "C" int mppi_step_noalloc(const float *state, const float *cloud, const u
     carve_scene(V, static_cast<char *>(arena) + kArenaHeader, P.K, P.T, parts);
     V.upd_chunk = upd_chunk_for(P.K, P.T, P.nu);
     V.upd_blocks = upd_blocks_for(P.K, P.T, P.nu);
-    V.val_chunks = val_chunks_for(n_points);
+    V.val_chunks = val_chunks_for(n_points, false);
     cudaStream_t st = (cudaStream_t)stream;
     // the array keeps the previous call's contents: zero the control words
     // and counters that must start at zero (no allocation involved)
     if (cudaMemsetAsync(arena, 0, kArenaHeader, st) != cudaSuccess) return EXACT_ECUDA;
     if (parts > 1 && cudaMemsetAsync(V.tk, 0, (size_t)P.K * sizeof(unsigned), st) != cudaSuccess) return EXACT_ECUDA;
-    return launch_cycle(V, fp, st, false, nullptr, sms);
+    return launch_cycle(V, fp, st, sms);
 }
