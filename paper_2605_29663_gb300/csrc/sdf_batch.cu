@@ -91,8 +91,11 @@ __device__ __forceinline__ void poly_rows(const float2 *__restrict__ pts, const 
             f0 = v0 && fmaf(cx0, cx0, cy0 * cy0) <= lim2;
             f1 = v1 && fmaf(cx1, cx1, cy1 * cy1) <= lim2;
             if (DIST) {
-                const float d0 = key_to_dist(fpc, k0);
-                const float d1 = key_to_dist(fpc, k1);
+                float d0 = key_to_dist(fpc, m0), d1 = key_to_dist(fpc, m1);   // before the mask: see below
+                if (MASKED) {
+                    d0 = v0 ? d0 : finf();
+                    d1 = v1 ? d1 : finf();
+                }
                 if (vec_store) {
                     __stcs(reinterpret_cast<float2 *>(drow) + j, make_float2(d0, d1));
                 } else {
@@ -161,15 +164,20 @@ sdf_batch_kernel(const float2 *__restrict__ pts, const uint8_t *__restrict__ mas
         float k0, k1;
         eval2(fpc, px0, py0, px1, py1, k0, k1);
         bool v0 = true, v1 = has1;
+        float d0 = 0.f, d1 = 0.f;
+        if (DIST) {   // before the mask: the root of +inf takes a slow branch
+            d0 = key_to_dist(fpc, k0);
+            d1 = key_to_dist(fpc, k1);
+        }
         if (MASKED) {
             v0 = __ldg(mask + i0) != 0;
             v1 = has1 && __ldg(mask + i1) != 0;
             k0 = v0 ? k0 : finf();
             k1 = v1 ? k1 : finf();
+            d0 = v0 ? d0 : finf();
+            d1 = v1 ? d1 : finf();
         }
         if (DIST) {
-            const float d0 = key_to_dist(fpc, k0);
-            const float d1 = key_to_dist(fpc, k1);
             if (vec_store) {
                 __stcs(reinterpret_cast<float2 *>(drow) + j, make_float2(d0, d1));
             } else {
