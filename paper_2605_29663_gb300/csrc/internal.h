@@ -39,6 +39,9 @@ namespace exact {
 
 // Grow the context arena to at least `bytes` (synchronous when it grows).
 int ensure_scratch(exact_ctx *ctx, size_t bytes);
+// Whether the arena holds `bytes`, or can be grown to them now (not while
+// the stream captures): for paths that have one needing less to fall back on.
+bool try_scratch(exact_ctx *ctx, size_t bytes, cudaStream_t st);
 int current_sm_count();
 // Arena bytes needed by exact_sdf_batch (n_poses) and mppi_step (K, T).
 size_t sdf_scratch_bytes(int n_poses);

@@ -32,6 +32,7 @@
 #include <algorithm>
 
 #include "mppi_kernels.cuh"
+#include "sdf_near.h"
 
 namespace exact {
 
@@ -131,7 +132,7 @@ extern "C" int exact_ctx_reserve(exact_ctx *ctx, int max_poses, int max_K, int m
 
 extern "C" int exact_ctx_reserve_cloud(exact_ctx *ctx, int max_poses, int max_K, int max_T, int max_points) {
     if (!ctx || max_poses < 0 || max_K < 0 || max_T < 0 || max_points < 0) return EXACT_EINVAL;
-    size_t need = sdf_scratch_bytes(max_poses);
+    size_t need = sdf_scratch_bytes(max_poses) + sdf_near_bytes(max_points);
     const size_t m = kArenaHeader + scene_scratch_bytes(max_K, max_T, parts_of(ctx, max_K, max_T)) +
                      (max_points < kPruneMin ? 0 :
                       std::max(grid_copy_bytes(max_points, true),
@@ -156,9 +157,12 @@ int mppi_step_impl(exact_ctx *ctx, const float *state, const float *cloud, const
     // without a d_min output the costs only need the points near the
     // footprint: clouds of kPruneMin points or more get a cell grid
     const bool grid = !dmin && n_points >= kPruneMin && n_points <= kGridMaxPoints;
-    const bool steps = grid && velocity && step_grid_bytes(n_points, P.T) <= kStepGridBytes;
     const size_t scene_bytes = kArenaHeader + scene_scratch_bytes(P.K, P.T, parts);
-    rc = ensure_scratch(ctx, scene_bytes + (!grid ? 0 : steps ? step_grid_bytes(n_points, P.T) : grid_copy_bytes(n_points, velocity != nullptr)));
+    const bool steps = grid && velocity && step_grid_bytes(n_points, P.T) <= kStepGridBytes &&
+                       try_scratch(ctx, scene_bytes + step_grid_bytes(n_points, P.T),
+                                   (cudaStream_t)stream);
+    rc = steps ? EXACT_OK
+               : ensure_scratch(ctx, scene_bytes + (grid ? grid_copy_bytes(n_points, velocity != nullptr) : 0));
     if (rc != EXACT_OK) return rc;
     SceneView V;
     V.P = P;

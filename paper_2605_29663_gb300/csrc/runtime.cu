@@ -220,6 +220,18 @@ int ensure_scratch(exact_ctx *ctx, size_t bytes) {
     return EXACT_OK;
 }
 
+bool try_scratch(exact_ctx *ctx, size_t bytes, cudaStream_t st) {
+    if (bytes <= ctx->scratch_bytes) return true;
+    if (bytes > ((size_t)1 << 30)) return false;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone ||
+        ensure_scratch(ctx, bytes) != EXACT_OK) {
+        cudaGetLastError();   // not this call's error: it takes the other path
+        return false;
+    }
+    return true;
+}
+
 }  // namespace exact
 
 extern "C" int exact_ctx_create(exact_ctx **out) {

@@ -10,6 +10,7 @@
 // words); when several blocks share a pose they meet in a 64-bit atomicMin
 // on a per-pose key in the context arena, finished by a small kernel.
 #include "internal.h"
+#include "sdf_near.h"
 
 namespace exact {
 
@@ -241,11 +242,32 @@ extern "C" int exact_sdf_batch(exact_ctx *ctx, const float *points, const uint8_
     if ((size_t)n_points * (size_t)n_poses >= ((size_t)1 << 62)) return EXACT_ECAPACITY;
     cudaStream_t st = (cudaStream_t)stream;
 
+    int sms = ctx ? ctx->sm_count : 0;
+    if (sms <= 0) sms = current_sm_count();
+    const float2 *p2 = reinterpret_cast<const float2 *>(points);
+    // many poses against one cloud: the pruned path (sdf_near.cu), where the
+    // context has (or can get) scratch for the sorted cloud
+    const size_t near_off = sdf_scratch_bytes(n_poses);
+    if (ctx && (dist || dmin || argmin) && sdf_near_fits(fp, n_points, n_poses, dist != nullptr) &&
+        try_scratch(ctx, near_off + sdf_near_bytes(n_points), st)) {
+        ctx->mppi_layout = -1;   // overlays the MPPI per-sample counters
+        unsigned long long *keys = nullptr;
+        if (dist && (dmin || argmin) && n_points > kSdfChunk) {
+            keys = reinterpret_cast<unsigned long long *>(static_cast<char *>(ctx->scratch) + kArenaHeader);
+            sdf_keys_init<<<(n_poses + 255) / 256, 256, 0, st>>>(keys, n_poses);
+        }
+        const int rc = sdf_near_launch(p2, mask, n_points, poses, n_poses, fp, dist, dmin, argmin, keys,
+                                       static_cast<char *>(ctx->scratch) + near_off, sms, ctx->d_err, st);
+        if (rc != EXACT_OK || !keys) return rc;
+        return with_footprint(fp, [&](auto fpc) -> int {
+            sdf_keys_finish<decltype(fpc)><<<(n_poses + 255) / 256, 256, 0, st>>>(keys, n_poses, fpc, dmin, argmin);
+            return cuda_status(cudaGetLastError());
+        });
+    }
+
     // one block per pose when there are enough poses to fill the GPU;
     // otherwise split each pose's points over several blocks
     const int npairs = (n_points + 1) / 2;
-    int sms = ctx ? ctx->sm_count : 0;
-    if (sms <= 0) sms = current_sm_count();
     const int target = sms * 8;
     int chunks = 1;
     if (n_poses < target && npairs > 256) {
@@ -266,7 +288,6 @@ extern "C" int exact_sdf_batch(exact_ctx *ctx, const float *points, const uint8_
         ctx->mppi_layout = -1;   // the keys overlay the MPPI per-sample counters
         sdf_keys_init<<<(n_poses + 255) / 256, 256, 0, st>>>(keys, n_poses);
     }
-    const float2 *p2 = reinterpret_cast<const float2 *>(points);
     const unsigned grid = (unsigned)(n_poses * chunks);
     return with_footprint(fp, [&](auto fpc) -> int {
         using FPC = decltype(fpc);
