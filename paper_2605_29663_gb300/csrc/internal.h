@@ -24,11 +24,19 @@ struct exact_footprint {
     float bhx, bhy;         // half extents of the bounding box about (bcx, bcy), rounded up
 };
 
+// Minimum of one pose of a split exact_sdf_batch (complemented packed key; 0
+// = empty) and its finished blocks; both zero between calls.
+struct SdfKey {
+    unsigned long long best;
+    unsigned ticket, pad;
+};
+
 struct exact_ctx {
     int device = 0;
     int sm_count = 0;
     void *scratch = nullptr;     // growable device arena
     size_t scratch_bytes = 0;
+    SdfKey *sdf_keys = nullptr;  // sdf_split_poses of them, apart from the arena: other calls leave them alone
     int *d_err = nullptr;        // device error word (exact_status)
     long long mppi_layout = -1;  // (K, T, parts) of the last mppi_step; -1 = arena reused otherwise
     bool stats = false;          // mppi_step also records cycle statistics
@@ -43,6 +51,9 @@ int ensure_scratch(exact_ctx *ctx, size_t bytes);
 // the stream captures): for paths that have one needing less to fall back on.
 bool try_scratch(exact_ctx *ctx, size_t bytes, cudaStream_t st);
 int current_sm_count();
+// exact_sdf_batch splits a pose's points over several blocks below this many
+// poses (about eight blocks per SM).
+inline int sdf_split_poses(int sms) { return (sms > 0 ? sms : 148) * 8; }
 // Arena bytes needed by exact_sdf_batch (n_poses) and mppi_step (K, T).
 size_t sdf_scratch_bytes(int n_poses);
 

@@ -242,15 +242,20 @@ extern "C" int exact_ctx_create(exact_ctx **out) {
     if (cudaGetDevice(&ctx->device) != cudaSuccess) { delete ctx; return EXACT_ECUDA; }
     ctx->sm_count = exact::current_sm_count();
     if (cudaMalloc(&ctx->d_err, sizeof(int)) != cudaSuccess) { delete ctx; return EXACT_ECUDA; }
-    if (cudaMalloc(&ctx->d_stats, sizeof(exact_cycle_stats)) != cudaSuccess) {
+    const size_t key_bytes = sizeof(SdfKey) * (size_t)exact::sdf_split_poses(ctx->sm_count);
+    if (cudaMalloc(&ctx->d_stats, sizeof(exact_cycle_stats)) != cudaSuccess ||
+        cudaMalloc(&ctx->sdf_keys, key_bytes) != cudaSuccess) {
         cudaFree(ctx->d_err);
+        cudaFree(ctx->d_stats);
         delete ctx;
         return EXACT_ECUDA;
     }
     if (cudaMemset(ctx->d_err, 0, sizeof(int)) != cudaSuccess ||
-        cudaMemset(ctx->d_stats, 0, sizeof(exact_cycle_stats)) != cudaSuccess) {
+        cudaMemset(ctx->d_stats, 0, sizeof(exact_cycle_stats)) != cudaSuccess ||
+        cudaMemset(ctx->sdf_keys, 0, key_bytes) != cudaSuccess) {
         cudaFree(ctx->d_err);
         cudaFree(ctx->d_stats);
+        cudaFree(ctx->sdf_keys);
         delete ctx;
         return EXACT_ECUDA;
     }
@@ -262,6 +267,7 @@ extern "C" void exact_ctx_destroy(exact_ctx *ctx) {
     if (!ctx) return;
     cudaDeviceSynchronize();
     if (ctx->scratch) cudaFree(ctx->scratch);
+    if (ctx->sdf_keys) cudaFree(ctx->sdf_keys);
     if (ctx->d_err) cudaFree(ctx->d_err);
     if (ctx->d_stats) cudaFree(ctx->d_stats);
     delete ctx;
