@@ -70,7 +70,7 @@ batched_sample_kernel(const SceneDev *__restrict__ scenes, const int2 *__restric
 
 // The scenes without a d_min output: persistent blocks take grid items from
 // the queue, a scene's footprint terms and distance field in shared memory.
-__global__ void __launch_bounds__(768)   // at most 512 are launched: 80 registers, three blocks of 256 per SM
+__global__ void __launch_bounds__(1024)   // at most 512 are launched: 64 registers, four blocks of 256 per SM
 batched_grid_sample_kernel(const SceneDev *__restrict__ scenes, const int2 *__restrict__ items, int n_items,
                            int group, unsigned *queue) {
     extern __shared__ float4 dyn[];
@@ -106,8 +106,10 @@ batched_cloud_grid_kernel(const SceneDev *__restrict__ scenes, const int *__rest
 __global__ void __launch_bounds__(kUpdBlock)
 batched_update_kernel(const SceneDev *__restrict__ scenes, const int2 *__restrict__ table) {
     __shared__ UpdateSmem sm;
+    __shared__ SceneView V;
     const int2 t = table[blockIdx.x];
-    update_body(scenes[t.x].V, t.y, sm);
+    stage_view(V, scenes[t.x].V);
+    update_body(V, t.y, sm);
 }
 
 __global__ void __launch_bounds__(kBlock)
@@ -115,11 +117,13 @@ batched_validate_kernel(const SceneDev *__restrict__ scenes, const int2 *__restr
     __shared__ float4 s_fp[kFpSlots];
     __shared__ ValidateSmem sm;
     const int2 t = table[blockIdx.x];
+    __shared__ SceneView V;
     const SceneDev &D = scenes[t.x];
     load_table(s_fp, D.fp);
-    __syncthreads();
+    const CloudGrid *grid = D.grid;
     const SmemEval ev = table_eval(D.fp, s_fp);
-    validate_body(D.V, ev, t.y / D.V.val_chunks, t.y % D.V.val_chunks, sm, D.grid);
+    stage_view(V, D.V);
+    validate_body(V, ev, t.y / V.val_chunks, t.y % V.val_chunks, sm, grid);
 }
 
 int check_params(const exact_mppi_params *p);
@@ -202,7 +206,7 @@ extern "C" int exact_batch_create(int n_scenes, const exact_scene *scenes, exact
         }
     }
     const int sms_now = current_sm_count();
-    const int group = grid_group(grid_k, sms_now);
+    const int group = grid_group(grid_k, grid_T, kBlock / 32, sms_now);
     for (int s : order) {
         const exact_mppi_params &p = scenes[s].params;
         if (uses_grid(scenes[s])) {
@@ -349,7 +353,8 @@ static int launch_sample(exact_batch *b, const SceneDev *table, cudaStream_t st)
     if (cudaGetLastError() != cudaSuccess) return EXACT_ECUDA;
     // the persistent warps start early (rollouts first; grid_sample waits
     // before it reads a grid)
-    return cuda_status(launch_dependent(batched_grid_sample_kernel, (unsigned)b->ggrid, (unsigned)b->threads,
+    // no more blocks than items: idle ones would crowd the busy ones on an SM
+    return cuda_status(launch_dependent(batched_grid_sample_kernel, (unsigned)std::min(b->ggrid, b->n_gitems), (unsigned)b->threads,
                                         grid_smem(b), st, table, (const int2 *)b->d_gitems, b->n_gitems, b->grid_group,
                                         b->d_queue + 1));
 }

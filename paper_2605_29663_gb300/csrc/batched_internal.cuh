@@ -17,6 +17,16 @@ struct SceneDev {
     FpTable fp;
 };
 
+// The scene's view in shared memory, read before the block waits for its
+// predecessor: its fields are otherwise fetched from the table one dependent
+// load after the other behind the wait.  Ends with a block barrier.
+__device__ __forceinline__ void stage_view(SceneView &dst, const SceneView &src) {
+    static_assert(sizeof(SceneView) % 4 == 0, "copied in words");
+    for (int i = threadIdx.x; i < (int)(sizeof(SceneView) / 4); i += blockDim.x)
+        reinterpret_cast<int *>(&dst)[i] = reinterpret_cast<const int *>(&src)[i];
+    __syncthreads();
+}
+
 // A sample item of a scene with a d_min output is (scene, r); bit 30 of r
 // marks an item that also takes sample r + 1 of the same scene (see
 // sample_body).  A grid item is (scene, r): grid_group consecutive samples

@@ -39,8 +39,10 @@ batched_validate_kernel_c(const SceneDev *__restrict__ scenes, const int2 *__res
                           const ConstEval<FPC> ev) {
     __shared__ ValidateSmem sm;
     const int2 t = table[blockIdx.x];
-    const SceneDev &D = scenes[t.x];
-    validate_body(D.V, ev, t.y / D.V.val_chunks, t.y % D.V.val_chunks, sm, D.grid);
+    __shared__ SceneView V;
+    const CloudGrid *grid = scenes[t.x].grid;
+    stage_view(V, scenes[t.x].V);
+    validate_body(V, ev, t.y / V.val_chunks, t.y % V.val_chunks, sm, grid);
 }
 
 template <class FPC>

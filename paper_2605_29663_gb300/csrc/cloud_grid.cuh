@@ -14,15 +14,18 @@
 // No output changes by a bit: a point in no walked cell is farther than
 // d_safe, and a point not evaluated is farther than one that is.
 //
-// What bounds it: instruction issue (41 to 68 % of the cycles issue) where
+// What bounds it: instruction issue (49 to 71 % of the cycles issue) where
 // many points lie inside the footprints, else the latency of one sample's
 // rollout, walk and evaluation.  Measured against sub-chunk circles over a
 // Morton-ordered copy (cycle times, the nominal driven to where the samples
-// touch obstacles): forklift K = 2,048, T = 40, N = 4,096 127 -> 87 us;
-// hybrid 3 x K = 1,024, N = 2,048 70 -> 43 us; 64 scenes of up to 20,000
-// points 6.29 -> 1.60 ms; predicted K = 1,024, N = 2,048 49 -> 29 us.  One warp
-// per sample was slower than a block's warps sharing eight samples (the
-// forklift's near points range from 0 to 4,700 per sample).
+// touch obstacles): forklift K = 2,048, T = 40, N = 4,096 124 -> 82 us; hybrid
+// 3 x K = 1,024, N = 2,048 73 -> 41 us; 64 scenes of up to 20,000 points 6.47 ->
+// 1.28 ms; predicted K = 1,024, N = 2,048 57 -> 27 us.  One warp per sample was
+// slower than a block's warps sharing its samples (the forklift's near points
+// range from 0 to 4,700 per sample).  Clouds below 1,024 points stay with
+// the point-level pruning of steps_min_keys, which needs no launch before the
+// samples (512 points, K = 256: 18 against 22 us; 100 points, K = 1,000: 24
+// against 34 us).
 #pragma once
 
 #include "mppi_cycle.cuh"
@@ -103,7 +106,8 @@ __device__ __forceinline__ void build_grid(const float2 *__restrict__ pts, const
     const bool any = lx <= hx;
     if (!any) lx = ly = hx = hy = 0.f;
     const float w = hx - lx, h = hy - ly, wide = fmaxf(w, h);
-    const float cell = fmaxf(fmaxf(sqrtf(w * (h / kCellTarget)), wide / (float)(kGridDim - 1)), 1e-6f);
+    const float target = fminf(kCellTarget, fmaxf(1000.f, 2.f * (float)N));
+    const float cell = fmaxf(fmaxf(sqrtf(w * (h / target)), wide / (float)(kGridDim - 1)), 1e-6f);
     const float inv = 1.f / cell;
     const int nx = min(kGridDim, (int)(w * inv) + 1), ny = min(kGridDim, (int)(h * inv) + 1);
     const int ncell = min(kCells, nx * ny);
@@ -181,21 +185,35 @@ __device__ __forceinline__ void build_grid(const float2 *__restrict__ pts, const
 // steps at a time from a shared counter (a sample that drives through a wall
 // has thousands of near points, its neighbour none), then one warp each forms
 // the J~.
-constexpr int kGroup = 8;
+constexpr int kGroup = 16;
 constexpr int kRuns = 64;     // a warp's queued runs: 32 are handled at a time, at most 31 stay
 constexpr int kEvals = 128;   // a warp's queued points: 64 are evaluated at a time, at most 63 stay
-constexpr int kLongRun = 40;  // points from which a run is taken by itself
 constexpr int kField = 32;    // cells of the footprint's distance field along one axis
 __host__ __device__ constexpr int grid_T_pad(int T) { return (T + 3) / 4 * 4; }
 __host__ __device__ constexpr size_t grid_smem_bytes(int T, int samples, int warps) {
     return kField * kField * 4 + (size_t)grid_T_pad(T) * 32 * samples + kGroup * 4 + (size_t)warps * (kRuns * 12 + kEvals * 8);
 }
 
-// Samples per block: as few as keep the blocks to the three per SM that are
-// resident at once, so that a small sample count still spreads over the GPU.
-inline int grid_group(long long samples, int sms) {
-    const long long slots = 3LL * (sms > 0 ? sms : 148), g = (samples + slots - 1) / slots;
-    return (int)(g < 1 ? 1 : g > kGroup ? kGroup : g);
+// Samples per block: as few as keep the blocks to three per SM, so that a small
+// sample count still spreads over the GPU, and up to 16 beyond, which is where
+// a block's three phases and their barriers cost least (64 scenes with 114,688
+// samples: groups of 4, 8, 16, 24 take 1.94, 1.55, 1.35, 1.41 ms; the forklift's
+// 2,048 samples: groups of 3, 5, 7 take 94, 87, 93 us).
+// A long horizon lowers it to what leaves three blocks their shared memory.
+inline int grid_group(long long samples, int T, int warps, int sms) {
+    const long long slots = 3LL * (sms > 0 ? sms : 148), want = (samples + slots - 1) / slots;
+    int g = (int)(want < 1 ? 1 : want > kGroup ? kGroup : want);
+    while (g > 1 && grid_smem_bytes(T, g, warps) > 70u * 1024u) --g;
+    return g;
+}
+
+// Minimum of floats of either sign (not NaN): their bits order as signed
+// integers when positive, the other way round when negative.
+__device__ __forceinline__ void atomic_min(float *a, float v) {
+    if (v >= 0.f)
+        atomicMin(reinterpret_cast<int *>(a), __float_as_int(v));
+    else
+        atomicMax(reinterpret_cast<unsigned *>(a), __float_as_uint(v));
 }
 
 // The footprint's signed distance at the centres of kField x kField cells over
@@ -242,8 +260,8 @@ __device__ __forceinline__ void grid_samples(const SceneView &V, const CloudGrid
     float *field = reinterpret_cast<float *>(mem);
     float4 *pose = reinterpret_cast<float4 *>(field + kField * kField);
     unsigned *key = reinterpret_cast<unsigned *>(pose + ns * Tp);   // minimum order key
-    unsigned *lim = key + ns * Tp;                                  // f2ord of the distance that still matters
-    float *stage = reinterpret_cast<float *>(lim + ns * Tp);                                   // stage cost without the obstacle term
+    float *lim = reinterpret_cast<float *>(key + ns * Tp);          // distance that still matters
+    float *stage = lim + ns * Tp;                                   // stage cost without the obstacle term
     float *time = stage + ns * Tp;                                  // time of the scored state
     float *term = time + ns * Tp;                                   // per sample: terminal cost
     // this warp's queues: points to evaluate (slot, point); runs of points (slot, first, count)
@@ -270,7 +288,7 @@ __device__ __forceinline__ void grid_samples(const SceneView &V, const CloudGrid
                 sincosf(R.th[e], &sn, &cs);
                 pose[off + h] = make_float4(R.x[e], R.y[e], cs, sn);
                 key[off + h] = f2ord(finf());
-                lim[off + h] = f2ord(cap);
+                lim[off + h] = cap;
                 time[off + h] = (float)(h + P.state_offset) * P.dt;
                 const float u2 = fmaf(R.u[e][0], R.u[e][0], fmaf(R.u[e][1], R.u[e][1], R.u[e][2] * R.u[e][2]));
                 stage[off + h] = fmaf(P.w_goal, guidance_dist(R.x[e], R.y[e], V.wp, V.W), P.w_ctrl * u2);
@@ -313,68 +331,39 @@ __device__ __forceinline__ void grid_samples(const SceneView &V, const CloudGrid
             }
             __syncwarp();
         };
-        // the points of queued runs [0, n), n <= 32, 64 at a time: those whose
-        // lower bound is below their slot's limit go to the evaluation queue.
-        // A long run is taken by itself, the short ones' points are dealt out
-        // (each lane searches its run in the prefix sums of their lengths)
+        // the points of queued runs [0, n), n <= 32, dealt 64 at a time: those
+        // whose lower bound is below their slot's limit go to the evaluation
+        // queue.  The run of a dealt point is found by counting the runs that
+        // start at or before it: a bit per start in the window's mask
         auto walk_runs = [&](int n) {
             __syncwarp();
-            int cnt = lane < n ? run_n[lane] : 0;
-            const int first = lane < n ? run_p[lane] : 0, rs = lane < n ? run_s[lane] : 0;
-            unsigned longs = __ballot_sync(full, cnt >= kLongRun);
-            const int len = cnt;
-            if (cnt >= kLongRun) cnt = 0;
+            const int cnt = lane < n ? run_n[lane] : 0, rs = lane < n ? run_s[lane] : 0;
             int incl = cnt;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const int t = __shfl_up_sync(full, incl, o);
                 if (lane >= o) incl += t;
             }
-            const int off = first - (incl - cnt);   // the run's first point as an offset from the dealt index
+            const int excl = incl - cnt, off = (lane < n ? run_p[lane] : 0) - excl;   // first point, from the dealt index
             const int total = __shfl_sync(full, incl, 31);
-            int b = 0, long_p = 0, long_n = 0, long_s = 0;   // dealt points; the long run being taken
-            for (;;) {
+            const unsigned upto = (2u << lane) - 1u;
+            for (int b = 0; b < total; b += 64) {
                 float lb[2], ub[2], now[2];   // bounds of the distance; the slot's limit
                 int i[2], sl[2];
-                bool in[2], lower = false;
-                if (long_n <= 0 && longs) {
-                    const int l = __ffs(longs) - 1;
-                    longs &= longs - 1u;
-                    long_p = __shfl_sync(full, first, l);
-                    long_n = __shfl_sync(full, len, l);
-                    long_s = __shfl_sync(full, rs, l);
-                }
-                if (long_n > 0) {
-#pragma unroll
-                    for (int q = 0; q < 2; ++q) {
-                        i[q] = long_p + 32 * q + lane;
-                        sl[q] = long_s;
-                        in[q] = 32 * q + lane < long_n;
-                    }
-                    long_p += 64;
-                    long_n -= 64;
-                } else if (b < total) {
-                    int k[2] = {0, 0};   // the number of runs that end at or before an index
-#pragma unroll
-                    for (int st = 16; st > 0; st >>= 1)
-#pragma unroll
-                        for (int q = 0; q < 2; ++q)
-                            if (__shfl_sync(full, incl, k[q] + st - 1) <= b + 32 * q + lane) k[q] += st;
-#pragma unroll
-                    for (int q = 0; q < 2; ++q) {
-                        i[q] = b + 32 * q + lane + __shfl_sync(full, off, k[q]);
-                        sl[q] = __shfl_sync(full, rs, k[q]);
-                        in[q] = b + 32 * q + lane < total;
-                    }
-                    b += 64;
-                } else {
-                    break;
-                }
+                bool lower = false;
+                const int rel = excl - b;
+                const unsigned lo = __reduce_or_sync(full, (unsigned)rel < 32u ? 1u << rel : 0u);
+                const unsigned hi = __reduce_or_sync(full, (unsigned)(rel - 32) < 32u ? 1u << (rel - 32) : 0u);
+                const int before = __popc(__ballot_sync(full, rel < 0)) - 1;
+                const int k[2] = {before + __popc(lo & upto), before + __popc(lo) + __popc(hi & upto)};
 #pragma unroll
                 for (int q = 0; q < 2; ++q) {
+                    const int t = b + 32 * q + lane;
+                    i[q] = t + __shfl_sync(full, off, k[q] & 31);
+                    sl[q] = __shfl_sync(full, rs, k[q] & 31);
                     lb[q] = ub[q] = finf();
-                    now[q] = ord2f(lim[sl[q]]);
-                    if (in[q]) {
+                    now[q] = lim[sl[q]];
+                    if (t < total) {
                         const float4 p = pose[sl[q]];
                         const float2 o = point_at(i[q], sl[q]);
                         float px, py;
@@ -392,10 +381,10 @@ __device__ __forceinline__ void grid_samples(const SceneView &V, const CloudGrid
                 if (__any_sync(full, lower)) {   // some point's distance is below the limit: it falls
 #pragma unroll
                     for (int q = 0; q < 2; ++q)
-                        if (ub[q] < now[q]) atomicMin(lim + sl[q], f2ord(ub[q]));
+                        if (ub[q] < now[q]) atomic_min(lim + sl[q], ub[q]);
                     __syncwarp();
 #pragma unroll
-                    for (int q = 0; q < 2; ++q) now[q] = ord2f(*(volatile unsigned *)(lim + sl[q]));
+                    for (int q = 0; q < 2; ++q) now[q] = *(volatile float *)(lim + sl[q]);
                 }
                 const bool keep[2] = {lb[0] <= now[0], lb[1] <= now[1]};
                 const unsigned b0 = __ballot_sync(full, keep[0]), b1 = __ballot_sync(full, keep[1]);
@@ -447,7 +436,7 @@ __device__ __forceinline__ void grid_samples(const SceneView &V, const CloudGrid
             }
             for (int k = phase; __any_sync(full, k < rows); k += lanes) {
                 int p0 = 0, p1 = 0;
-                if (k < rows) row_run(g, gh->start, w, walk_row(w, k), ord2f(lim[slot]) + reach, p0, p1);
+                if (k < rows) row_run(g, gh->start, w, walk_row(w, k), lim[slot] + reach, p0, p1);
                 const bool some = p1 > p0;
                 const unsigned b = __ballot_sync(full, some);
                 if (b) {

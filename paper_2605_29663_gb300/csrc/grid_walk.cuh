@@ -25,7 +25,7 @@ constexpr size_t kGridBytes = (sizeof(CloudGrid) + 255) / 256 * 256;
 // at that step, while those fit kStepGridBytes; else one grid whose cells are
 // searched as far as the fastest point can have moved.  (Measured with K =
 // 1,024, T = 20, 2,048 points on boxes and discs at 0.5 m/s: the cycle takes
-// 29 us with a grid per step, 45 to 52 us with one.)
+// 27 to 29 us with a grid per step, 45 to 52 us with one.)
 constexpr size_t kStepGridBytes = 64u << 20;
 // The grid of step h and the first of its points: grid + h * grids, point
 // h * points (both 0 for a static cloud).

@@ -1179,7 +1179,6 @@ struct ValidateSmem {
     float red[kRedSlices][EXACT_MAX_HORIZON * 3 + 1];
     float U[EXACT_MAX_HORIZON * 3];
     float4 pose;
-    float Z;
     float mn[32];
     bool last, ok;
 };
@@ -1207,6 +1206,7 @@ __device__ __forceinline__ void validate_body(const SceneView &V, const EV &ev, 
     // the nominal U and the start state stay unchanged until this kernel's
     // last block: read them while the update phase drains
     for (int e = tid; e < TN; e += kBlock) sm.U[e] = V.U[e];
+    const float x0 = V.state[0], y0 = V.state[1], th0 = V.state[2];
     grid_dep_wait();   // the partial slots come from the update phase
     grid_dep_release();   // a dependent launch (the hybrid selection) waits for this grid's end anyway
 
@@ -1229,13 +1229,9 @@ __device__ __forceinline__ void validate_body(const SceneView &V, const EV &ev, 
         sm.red[warp][e] = a;
     }
     __syncthreads();
-    if (tid == 0) {
-        float z = 0.f;
-        for (int w = 0; w < kRedSlices; ++w) z += sm.red[w][TN];
-        sm.Z = z;
-    }
-    __syncthreads();
-    const float invZ = 1.f / sm.Z;
+    float z = 0.f;   // every thread adds the slices itself
+    for (int w = 0; w < kRedSlices; ++w) z += sm.red[w][TN];
+    const float invZ = 1.f / z;
     for (int e = tid; e < TN; e += kBlock) {
         float a = 0.f;
         for (int w = 0; w < kRedSlices; ++w) a += sm.red[w][e];
@@ -1246,8 +1242,7 @@ __device__ __forceinline__ void validate_body(const SceneView &V, const EV &ev, 
     __syncthreads();
     if (warp == 0) {   // the nominal's rollout on warp 0, the other warps share out the outputs
         LaneRollout R;
-        warp_rollout(P, V.state[0], V.state[1], V.state[2], [&](int hh, int j) { return clamp_u(P, j, sm.U[hh * nu + j]); },
-                     R);
+        warp_rollout(P, x0, y0, th0, [&](int hh, int j) { return clamp_u(P, j, sm.U[hh * nu + j]); }, R);
 #pragma unroll
         for (int q = 0; q < kMaxPerLane; ++q) {
             if (q < R.per && lane * R.per + q == h) {
@@ -1358,8 +1353,7 @@ __device__ __forceinline__ void validate_body(const SceneView &V, const EV &ev, 
     }
     if (V.nom_cost && warp == 0) {
         LaneRollout R;
-        warp_rollout(P, V.state[0], V.state[1], V.state[2], [&](int hh, int j) { return clamp_u(P, j, sm.U[hh * nu + j]); },
-                     R);
+        warp_rollout(P, x0, y0, th0, [&](int hh, int j) { return clamp_u(P, j, sm.U[hh * nu + j]); }, R);
         ff acc{0.f, 0.f};
 #pragma unroll
         for (int e = 0; e < kMaxPerLane; ++e) {

@@ -111,8 +111,12 @@ int launch_cycle_t(const SceneView &V, const exact_footprint *fp, cudaStream_t s
 template <bool MOVING>
 int launch_grid_cycle_t(const SceneView &V, const exact_footprint *fp, cudaStream_t st, const CloudGrid *grid,
                         GridStride gst, int sms) {
-    const int group = grid_group(V.P.K, sms);
+    const int group = grid_group(V.P.K, V.P.T, kBlock / 32, sms);
     const size_t smem = grid_smem_bytes(V.P.T, group, kBlock / 32);
+    // beyond the default 48 KB with the footprint's slots
+    if (smem > 40u * 1024u && cudaFuncSetAttribute(mppi_grid_sample_kernel<MOVING>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)smem) != cudaSuccess)
+        return EXACT_ECUDA;
     const FpTable t = make_table(fp);
     if (launch_dependent(mppi_grid_sample_kernel<MOVING>, (V.P.K + group - 1) / group, kBlock, smem, st, V, t, grid,
                          gst, group) != cudaSuccess ||

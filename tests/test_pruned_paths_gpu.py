@@ -61,7 +61,8 @@ def _cycle(cloud, n, fp, K, T, model, seed, mask=False):
     ("uniform", 4096, "star64", 3651, 20, synth.DIFF, False), ("wall", 4097, "forklift", 459, 40, synth.DIFF, False),
     ("wall", 9000, "star64", 40, 128, synth.DIFF, True), ("point", 3000, "L", 130, 24, synth.OMNI, False),
     ("outlier", 2500, "far", 300, 20, synth.SPIN, False), ("invalid", 2048, "L", 912, 10, synth.DIFF, True),
-    ("uniform", 30000, "far", 16, 60, synth.DIFF, False)])
+    ("uniform", 30000, "far", 16, 60, synth.DIFF, False), ("uniform", 1500, "L", 7300, 128, synth.DIFF, False),
+    ("wall", 1100, "L", 4000, 70, synth.OMNI, False)])
 def test_grid_cycle_equals_unpruned_bitwise(ex, cloud, n, fp, K, T, model, mask):
     """Cell grid and distance field against the evaluation of every point (a
     d_min output switches them off): one sample, ragged sample groups, every
