@@ -214,7 +214,11 @@ int ensure_scratch(exact_ctx *ctx, size_t bytes) {
         return EXACT_ECUDA;
     }
     // counters and flags in the arena must start at zero
-    if (cudaMemset(ctx->scratch, 0, bytes) != cudaSuccess) return EXACT_ECUDA;
+    // the clear runs on the legacy stream, which a caller's non-blocking stream
+    // does not wait for: end it here, before the call's kernels write the arena
+    if (cudaMemset(ctx->scratch, 0, bytes) != cudaSuccess ||
+        cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess)
+        return EXACT_ECUDA;
     ctx->scratch_bytes = bytes;
     ctx->mppi_layout = -1;
     return EXACT_OK;
@@ -252,7 +256,8 @@ extern "C" int exact_ctx_create(exact_ctx **out) {
     }
     if (cudaMemset(ctx->d_err, 0, sizeof(int)) != cudaSuccess ||
         cudaMemset(ctx->d_stats, 0, sizeof(exact_cycle_stats)) != cudaSuccess ||
-        cudaMemset(ctx->sdf_keys, 0, key_bytes) != cudaSuccess) {
+        cudaMemset(ctx->sdf_keys, 0, key_bytes) != cudaSuccess ||
+        cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {   // as in ensure_scratch
         cudaFree(ctx->d_err);
         cudaFree(ctx->d_stats);
         cudaFree(ctx->sdf_keys);
