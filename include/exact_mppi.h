@@ -88,7 +88,9 @@ typedef struct exact_ctx exact_ctx;
 int exact_ctx_create(exact_ctx **out);
 void exact_ctx_destroy(exact_ctx *ctx);
 /* Make sure scratch for sdf batches of up to max_poses poses and MPPI steps
- * of up to max_K samples and max_T steps exists (synchronous). */
+ * of up to max_K samples and max_T steps exists (synchronous).  Scratch that a
+ * larger call outgrows stays allocated until the context is destroyed (together
+ * at most the size of the current one), so captured graphs stay valid. */
 int exact_ctx_reserve(exact_ctx *ctx, int max_poses, int max_K, int max_T);
 /* The same, also for clouds of up to max_points points: an MPPI step without
  * a d_min output sorts clouds of 1,024 points or more into a cell grid kept in

@@ -7,6 +7,8 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <vector>
+
 #include "common.cuh"
 #include "exact_mppi.h"
 
@@ -36,6 +38,7 @@ struct exact_ctx {
     int sm_count = 0;
     void *scratch = nullptr;     // growable device arena
     size_t scratch_bytes = 0;
+    std::vector<void *> retired; // outgrown arenas
     SdfKey *sdf_keys = nullptr;  // sdf_split_poses of them, apart from the arena: other calls leave them alone
     int *d_err = nullptr;        // device error word (exact_status)
     long long mppi_layout = -1;  // (K, T, parts) of the last mppi_step; -1 = arena reused otherwise

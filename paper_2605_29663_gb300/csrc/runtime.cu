@@ -4,6 +4,7 @@
 #include <stdlib.h>
 #include <string.h>
 
+#include <algorithm>
 #include <new>
 
 #include "internal.h"
@@ -199,27 +200,37 @@ int current_sm_count() {
     return sms;
 }
 
+// Outgrown arenas stay allocated until the context goes: a captured graph may
+// still replay with their addresses, whichever later call grew the scratch.
+// Doubling keeps them below the current arena's size in sum; they are given
+// back early only where the new arena would not fit otherwise.
 int ensure_scratch(exact_ctx *ctx, size_t bytes) {
     if (!ctx) return EXACT_EINVAL;
     if (bytes <= ctx->scratch_bytes) return EXACT_OK;
     bytes = align_up(bytes, (size_t)1 << 20);
-    if (ctx->scratch) {
+    size_t got = std::max(bytes, 2 * ctx->scratch_bytes);
+    void *p = nullptr;
+    if (cudaMalloc(&p, got) != cudaSuccess) {
+        cudaGetLastError();
         if (cudaDeviceSynchronize() != cudaSuccess) return EXACT_ECUDA;
-        cudaFree(ctx->scratch);
+        if (ctx->scratch) cudaFree(ctx->scratch);
+        for (void *q : ctx->retired) cudaFree(q);
+        ctx->retired.clear();
         ctx->scratch = nullptr;
         ctx->scratch_bytes = 0;
+        got = bytes;
+        if (cudaMalloc(&p, got) != cudaSuccess) return EXACT_ECUDA;
     }
-    if (cudaMalloc(&ctx->scratch, bytes) != cudaSuccess) {
-        ctx->scratch = nullptr;
+    // counters and flags in the arena must start at zero; the clear runs on the
+    // legacy stream, which a caller's non-blocking stream does not wait for: end
+    // it here, before the call's kernels write the arena
+    if (cudaMemset(p, 0, got) != cudaSuccess || cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {
+        cudaFree(p);
         return EXACT_ECUDA;
     }
-    // counters and flags in the arena must start at zero
-    // the clear runs on the legacy stream, which a caller's non-blocking stream
-    // does not wait for: end it here, before the call's kernels write the arena
-    if (cudaMemset(ctx->scratch, 0, bytes) != cudaSuccess ||
-        cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess)
-        return EXACT_ECUDA;
-    ctx->scratch_bytes = bytes;
+    if (ctx->scratch) ctx->retired.push_back(ctx->scratch);
+    ctx->scratch = p;
+    ctx->scratch_bytes = got;
     ctx->mppi_layout = -1;
     return EXACT_OK;
 }
@@ -272,6 +283,7 @@ extern "C" void exact_ctx_destroy(exact_ctx *ctx) {
     if (!ctx) return;
     cudaDeviceSynchronize();
     if (ctx->scratch) cudaFree(ctx->scratch);
+    for (void *q : ctx->retired) cudaFree(q);
     if (ctx->sdf_keys) cudaFree(ctx->sdf_keys);
     if (ctx->d_err) cudaFree(ctx->d_err);
     if (ctx->d_stats) cudaFree(ctx->d_stats);

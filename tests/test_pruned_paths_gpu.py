@@ -178,3 +178,39 @@ def test_sdf_under_capture_without_scratch_takes_the_general_path(ex):
     torch.cuda.synchronize()
     _, m, a = ex.sdf_batch(pts, poses, f, dist=False, ctx=ex.Context())
     assert bool((o["dmin"] == m).all()) and bool((o["argmin"] == a).all())
+
+
+def test_captured_cycle_survives_scratch_growth(ex):
+    """A graph keeps the scratch it was captured with: a later call of the same
+    context that needs more must not take it away."""
+    import torch
+    s = synth.plain_step(3, K=64, T=10, N=1500)
+    dev = torch.device("cuda")
+    t = {k: torch.from_numpy(s[k]).to(dev) for k in ("q0", "cloud", "waypoints", "U", "eps")}
+    fp = ex.Footprint(s["kind"], s["fp"])
+    ctx = ex.Context()
+    outs = {}
+    u0 = t["U"].clone()
+
+    def cycle(c, out):
+        t["U"].copy_(u0)
+        out.update(ex.mppi_step(c, t["q0"], t["cloud"], t["waypoints"], t["U"], t["eps"], fp, s["params"], out=out))
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        cycle(ctx, outs)
+    side.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side):
+        cycle(ctx, outs)
+    g = synth.rng(4)
+    pts = torch.from_numpy(g.uniform(-6, 6, (200_000, 2)).astype(np.float32)).to(dev)
+    poses = torch.from_numpy(g.uniform(-3, 3, (300, 3)).astype(np.float32)).to(dev)
+    _, grown, _ = ex.sdf_batch(pts, poses, fp, dist=False, ctx=ctx)
+    graph.replay()
+    torch.cuda.synchronize()
+    want = {}
+    cycle(ex.Context(), want)
+    torch.cuda.synchronize()
+    for k in want:
+        assert torch.equal(outs[k], want[k]), k
+    assert torch.equal(grown, ex.sdf_batch(pts, poses, fp, dist=False)[1])
