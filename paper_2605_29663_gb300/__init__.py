@@ -57,6 +57,8 @@ class CycleStats(ctypes.Structure):
 def load() -> ctypes.CDLL:
     """Load the CUDA library (raises if it has not been built)."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -179,13 +181,23 @@ def _check(rc: int, what: str) -> None:
         raise ExactError(rc, what)
 
 
+# A call of the smallest sizes costs more in this file than on the GPU (1 pose
+# x 1,000 points: 3.7 us of device time, 6.1 us a call, 12 to 14 us before), so
+# what every call does stays plain: one module lookup, addresses as plain
+# integers, and the current stream's handle without building a Stream object.
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
 
 
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _dev(t, name, dtype=None, shape=None):
@@ -202,9 +214,13 @@ def _dev(t, name, dtype=None, shape=None):
 
 
 def _stream(stream):
+    """The handle of `stream`, by default the current device's current stream."""
+    if stream is not None:
+        return stream.cuda_stream
     torch = _torch()
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    if not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 class Footprint:
