@@ -95,10 +95,10 @@ int exact_ctx_reserve(exact_ctx *ctx, int max_poses, int max_K, int max_T);
 /* The same, also for clouds of up to max_points points: an MPPI step without
  * a d_min output sorts clouds of 1,024 points or more into a cell grid kept in
  * the context (so that each sample looks only at the points near its
- * footprint, whatever the input order), and exact_sdf_batch keeps a spatially
- * sorted copy for many poses, so a call with a larger cloud than any before
- * may allocate -- reserve ahead of stream capture.  (A capturing
- * exact_sdf_batch without that scratch takes its general path.) */
+ * footprint, whatever the input order), so a step with a larger cloud than any
+ * before may allocate -- reserve ahead of stream capture.  (exact_sdf_batch of
+ * many poses takes the memory of a spatially sorted copy of the points from a
+ * pool of the context, stream-ordered, and its general path in a capture.) */
 int exact_ctx_reserve_cloud(exact_ctx *ctx, int max_poses, int max_K, int max_T, int max_points);
 /* Device-side error word of the context (an exact_status, 0 = none): the
  * first error a kernel launched with this context recorded.  Kernels record

@@ -279,7 +279,7 @@ class Context:
     def reserve(self, max_poses: int = 0, max_K: int = 0, max_T: int = 0, max_points: int = 0):
         """Allocate scratch ahead of time (before a CUDA graph capture): SDF
         batches of max_poses poses, MPPI steps of max_K x max_T, clouds of
-        max_points points (their cell grid or spatially sorted copy)."""
+        max_points points (their cell grid)."""
         _check(load().exact_ctx_reserve_cloud(self._h, max_poses, max_K, max_T, max_points),
                "exact_ctx_reserve_cloud")
 

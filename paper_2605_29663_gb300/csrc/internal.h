@@ -7,8 +7,6 @@
 #include <stdint.h>
 #include <string.h>
 
-#include <vector>
-
 #include "common.cuh"
 #include "exact_mppi.h"
 
@@ -26,6 +24,8 @@ struct exact_footprint {
     float bhx, bhy;         // half extents of the bounding box about (bcx, bcy), rounded up
 };
 
+namespace exact { constexpr int kRetired = 128; }   // two arenas, doubled from 1 MB on: at most 40 steps each
+
 // Minimum of one pose of a split exact_sdf_batch (complemented packed key; 0
 // = empty) and its finished blocks; both zero between calls.
 struct SdfKey {
@@ -38,7 +38,15 @@ struct exact_ctx {
     int sm_count = 0;
     void *scratch = nullptr;     // growable device arena
     size_t scratch_bytes = 0;
-    std::vector<void *> retired; // outgrown arenas
+    // a second arena, for the cell grids, which each call writes before it reads:
+    // apart from the first, whose counters outlive a call
+    void *work = nullptr, *work_alloc = nullptr;   // work_alloc: null while it is the piece behind sdf_keys
+    size_t work_bytes = 0;
+    // exact_sdf_batch of many poses takes its sorted cloud from here, stream
+    // ordered: such calls may overlap on several streams.  NULL: no pool to be had
+    cudaMemPool_t pool = nullptr;
+    void *retired[exact::kRetired];   // outgrown arenas
+    int n_retired = 0;
     SdfKey *sdf_keys = nullptr;  // sdf_split_poses of them, apart from the arena: other calls leave them alone
     int *d_err = nullptr;        // device error word (exact_status)
     long long mppi_layout = -1;  // (K, T, parts) of the last mppi_step; -1 = arena reused otherwise
@@ -50,9 +58,9 @@ namespace exact {
 
 // Grow the context arena to at least `bytes` (synchronous when it grows).
 int ensure_scratch(exact_ctx *ctx, size_t bytes);
-// Whether the arena holds `bytes`, or can be grown to them now (not while
-// the stream captures): for paths that have one needing less to fall back on.
-bool try_scratch(exact_ctx *ctx, size_t bytes, cudaStream_t st);
+// Whether the second arena holds `bytes`, or can be grown to them now (not
+// while the stream captures, and to 1 GB at most).
+bool try_work(exact_ctx *ctx, size_t bytes, cudaStream_t st);
 int current_sm_count();
 // exact_sdf_batch splits a pose's points over several blocks below this many
 // poses (about eight blocks per SM).

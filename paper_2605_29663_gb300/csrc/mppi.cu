@@ -32,7 +32,6 @@
 #include <algorithm>
 
 #include "mppi_kernels.cuh"
-#include "sdf_near.h"
 
 namespace exact {
 
@@ -132,13 +131,13 @@ extern "C" int exact_ctx_reserve(exact_ctx *ctx, int max_poses, int max_K, int m
 
 extern "C" int exact_ctx_reserve_cloud(exact_ctx *ctx, int max_poses, int max_K, int max_T, int max_points) {
     if (!ctx || max_poses < 0 || max_K < 0 || max_T < 0 || max_points < 0) return EXACT_EINVAL;
-    size_t need = sdf_scratch_bytes(max_poses) + sdf_near_bytes(max_points);
-    const size_t m = kArenaHeader + scene_scratch_bytes(max_K, max_T, parts_of(ctx, max_K, max_T)) +
-                     (max_points < kPruneMin ? 0 :
-                      std::max(grid_copy_bytes(max_points, true),
-                               std::min(step_grid_bytes(max_points, max_T), kStepGridBytes)));   // static or predicted
-    if (m > need) need = m;
-    return ensure_scratch(ctx, need);
+    const int rc = ensure_scratch(ctx, std::max(sdf_scratch_bytes(max_poses),
+                                                kArenaHeader + scene_scratch_bytes(max_K, max_T, parts_of(ctx, max_K, max_T))));
+    if (rc != EXACT_OK) return rc;
+    if (max_points < kPruneMin) return EXACT_OK;
+    const size_t work = std::max(grid_copy_bytes(std::min(max_points, kGridMaxPoints), true),   // static or predicted
+                                 std::min(step_grid_bytes(max_points, max_T), kStepGridBytes));
+    return try_work(ctx, work, nullptr) ? EXACT_OK : EXACT_ECUDA;
 }
 
 namespace exact {
@@ -158,12 +157,25 @@ int mppi_step_impl(exact_ctx *ctx, const float *state, const float *cloud, const
     // footprint: clouds of kPruneMin points or more get a cell grid
     const bool grid = !dmin && n_points >= kPruneMin && n_points <= kGridMaxPoints;
     const size_t scene_bytes = kArenaHeader + scene_scratch_bytes(P.K, P.T, parts);
-    const bool steps = grid && velocity && step_grid_bytes(n_points, P.T) <= kStepGridBytes &&
-                       try_scratch(ctx, scene_bytes + step_grid_bytes(n_points, P.T),
-                                   (cudaStream_t)stream);
-    rc = steps ? EXACT_OK
-               : ensure_scratch(ctx, scene_bytes + (grid ? grid_copy_bytes(n_points, velocity != nullptr) : 0));
+    rc = ensure_scratch(ctx, scene_bytes);
     if (rc != EXACT_OK) return rc;
+    // grids go to the second arena, or where that is too small (and may not
+    // grow: a capture) behind the scene's scratch
+    char *room = nullptr;
+    auto make_room = [&](size_t bytes) {
+        room = try_work(ctx, bytes, (cudaStream_t)stream)    ? static_cast<char *>(ctx->work)
+               : scene_bytes + bytes <= ctx->scratch_bytes ? static_cast<char *>(ctx->scratch) + scene_bytes
+                                                           : nullptr;
+        return room != nullptr;
+    };
+    const bool steps = grid && velocity && step_grid_bytes(n_points, P.T) <= kStepGridBytes &&
+                       make_room(step_grid_bytes(n_points, P.T));
+    const size_t copy_bytes = grid ? grid_copy_bytes(n_points, velocity != nullptr) : 0;
+    if (grid && !steps && !make_room(copy_bytes)) {
+        rc = ensure_scratch(ctx, scene_bytes + copy_bytes);
+        if (rc != EXACT_OK) return rc;
+        room = static_cast<char *>(ctx->scratch) + scene_bytes;
+    }
     SceneView V;
     V.P = P;
     V.state = state;
@@ -193,7 +205,7 @@ int mppi_step_impl(exact_ctx *ctx, const float *state, const float *cloud, const
     ctx->mppi_layout = layout;
     const int sms = ctx->sm_count > 0 ? ctx->sm_count : current_sm_count();
     if (grid) {
-        char *q = static_cast<char *>(ctx->scratch) + scene_bytes;
+        char *q = room;
         CloudGrid *g = reinterpret_cast<CloudGrid *>(q);
         GridStride gst{0, 0};
         if (steps) {

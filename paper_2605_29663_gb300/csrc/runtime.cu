@@ -200,6 +200,13 @@ int current_sm_count() {
     return sms;
 }
 
+static void free_retired(exact_ctx *ctx) {
+    while (ctx->n_retired > 0) cudaFree(ctx->retired[--ctx->n_retired]);
+}
+static void retire(exact_ctx *ctx, void *p) {
+    if (p && ctx->n_retired < kRetired) ctx->retired[ctx->n_retired++] = p;   // doubling never gets there
+}
+
 // Outgrown arenas stay allocated until the context goes: a captured graph may
 // still replay with their addresses, whichever later call grew the scratch.
 // Doubling keeps them below the current arena's size in sum; they are given
@@ -214,8 +221,7 @@ int ensure_scratch(exact_ctx *ctx, size_t bytes) {
         cudaGetLastError();
         if (cudaDeviceSynchronize() != cudaSuccess) return EXACT_ECUDA;
         if (ctx->scratch) cudaFree(ctx->scratch);
-        for (void *q : ctx->retired) cudaFree(q);
-        ctx->retired.clear();
+        free_retired(ctx);
         ctx->scratch = nullptr;
         ctx->scratch_bytes = 0;
         got = bytes;
@@ -228,22 +234,28 @@ int ensure_scratch(exact_ctx *ctx, size_t bytes) {
         cudaFree(p);
         return EXACT_ECUDA;
     }
-    if (ctx->scratch) ctx->retired.push_back(ctx->scratch);
+    retire(ctx, ctx->scratch);
     ctx->scratch = p;
     ctx->scratch_bytes = got;
     ctx->mppi_layout = -1;
     return EXACT_OK;
 }
 
-bool try_scratch(exact_ctx *ctx, size_t bytes, cudaStream_t st) {
-    if (bytes <= ctx->scratch_bytes) return true;
+bool try_work(exact_ctx *ctx, size_t bytes, cudaStream_t st) {
+    if (bytes <= ctx->work_bytes) return true;
     if (bytes > ((size_t)1 << 30)) return false;
+    bytes = align_up(bytes, (size_t)1 << 20);
+    const size_t got = std::max(bytes, 2 * ctx->work_bytes);
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    void *p = nullptr;
     if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone ||
-        ensure_scratch(ctx, bytes) != EXACT_OK) {
-        cudaGetLastError();   // not this call's error: it takes the other path
+        cudaMalloc(&p, got) != cudaSuccess) {
+        cudaGetLastError();   // not this call's error: it has another path
         return false;
     }
+    retire(ctx, ctx->work_alloc);
+    ctx->work = ctx->work_alloc = p;
+    ctx->work_bytes = got;
     return true;
 }
 
@@ -257,9 +269,12 @@ extern "C" int exact_ctx_create(exact_ctx **out) {
     if (cudaGetDevice(&ctx->device) != cudaSuccess) { delete ctx; return EXACT_ECUDA; }
     ctx->sm_count = exact::current_sm_count();
     if (cudaMalloc(&ctx->d_err, sizeof(int)) != cudaSuccess) { delete ctx; return EXACT_ECUDA; }
-    const size_t key_bytes = sizeof(SdfKey) * (size_t)exact::sdf_split_poses(ctx->sm_count);
+    // the second arena starts as 1 MB behind the keys, so that a cycle on a
+    // cloud of ordinary size can be captured without any call before it
+    const size_t key_bytes = exact::align_up(sizeof(SdfKey) * (size_t)exact::sdf_split_poses(ctx->sm_count), 256);
+    ctx->work_bytes = (size_t)1 << 20;
     if (cudaMalloc(&ctx->d_stats, sizeof(exact_cycle_stats)) != cudaSuccess ||
-        cudaMalloc(&ctx->sdf_keys, key_bytes) != cudaSuccess) {
+        cudaMalloc(&ctx->sdf_keys, key_bytes + ctx->work_bytes) != cudaSuccess) {
         cudaFree(ctx->d_err);
         cudaFree(ctx->d_stats);
         delete ctx;
@@ -275,6 +290,18 @@ extern "C" int exact_ctx_create(exact_ctx **out) {
         delete ctx;
         return EXACT_ECUDA;
     }
+    ctx->work = reinterpret_cast<char *>(ctx->sdf_keys) + key_bytes;
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = ctx->device;
+    unsigned long long keep = 64ull << 20;   // kept over a synchronisation: the sorted copy of 6 million points
+    if (cudaMemPoolCreate(&ctx->pool, &props) != cudaSuccess) {
+        ctx->pool = nullptr;
+        cudaGetLastError();
+    } else {
+        cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    }
     *out = ctx;
     return EXACT_OK;
 }
@@ -283,7 +310,9 @@ extern "C" void exact_ctx_destroy(exact_ctx *ctx) {
     if (!ctx) return;
     cudaDeviceSynchronize();
     if (ctx->scratch) cudaFree(ctx->scratch);
-    for (void *q : ctx->retired) cudaFree(q);
+    if (ctx->work_alloc) cudaFree(ctx->work_alloc);
+    if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
+    exact::free_retired(ctx);
     if (ctx->sdf_keys) cudaFree(ctx->sdf_keys);
     if (ctx->d_err) cudaFree(ctx->d_err);
     if (ctx->d_stats) cudaFree(ctx->d_stats);

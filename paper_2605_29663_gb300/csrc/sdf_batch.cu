@@ -255,24 +255,30 @@ extern "C" int exact_sdf_batch(exact_ctx *ctx, const float *points, const uint8_
     int sms = ctx ? ctx->sm_count : 0;
     if (sms <= 0) sms = current_sm_count();
     const float2 *p2 = reinterpret_cast<const float2 *>(points);
-    // many poses against one cloud: the pruned path (sdf_near.cu), where the
-    // context has (or can get) scratch for the sorted cloud
-    const size_t near_off = sdf_scratch_bytes(n_poses);
-    if (ctx && (dist || dmin || argmin) && sdf_near_fits(fp, n_points, n_poses, dist != nullptr) &&
-        try_scratch(ctx, near_off + sdf_near_bytes(n_points), st)) {
-        ctx->mppi_layout = -1;   // overlays the MPPI per-sample counters
-        unsigned long long *keys = nullptr;
-        if (dist && (dmin || argmin) && n_points > kSdfChunk) {
-            keys = reinterpret_cast<unsigned long long *>(static_cast<char *>(ctx->scratch) + kArenaHeader);
-            sdf_keys_init<<<(n_poses + 255) / 256, 256, 0, st>>>(keys, n_poses);
+    // many poses against one cloud: the pruned path (sdf_near.cu), where there
+    // is memory for the sorted cloud: stream-ordered, since calls of one context
+    // may overlap on several streams, and not in a capture, whose replays may
+    // overlap anything
+    if (ctx && ctx->pool && (dist || dmin || argmin) && sdf_near_fits(fp, n_points, n_poses, dist != nullptr)) {
+        const bool split = dist && (dmin || argmin) && n_points > kSdfChunk;
+        const size_t key_bytes = split ? align_up((size_t)n_poses * sizeof(unsigned long long), 256) : 0;
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        void *mem = nullptr;
+        if (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
+            key_bytes + sdf_near_bytes(n_points) <= ((size_t)1 << 30) &&
+            cudaMallocFromPoolAsync(&mem, key_bytes + sdf_near_bytes(n_points), ctx->pool, st) == cudaSuccess) {
+            unsigned long long *keys = split ? static_cast<unsigned long long *>(mem) : nullptr;
+            if (keys) sdf_keys_init<<<(n_poses + 255) / 256, 256, 0, st>>>(keys, n_poses);
+            int rc = sdf_near_launch(p2, mask, n_points, poses, n_poses, fp, dist, dmin, argmin, keys,
+                                     static_cast<char *>(mem) + key_bytes, sms, ctx->d_err, st);
+            if (rc == EXACT_OK && keys)
+                rc = with_footprint(fp, [&](auto fpc) -> int {
+                    sdf_keys_finish<decltype(fpc)><<<(n_poses + 255) / 256, 256, 0, st>>>(keys, n_poses, fpc, dmin, argmin);
+                    return cuda_status(cudaGetLastError());
+                });
+            return cudaFreeAsync(mem, st) == cudaSuccess ? rc : EXACT_ECUDA;
         }
-        const int rc = sdf_near_launch(p2, mask, n_points, poses, n_poses, fp, dist, dmin, argmin, keys,
-                                       static_cast<char *>(ctx->scratch) + near_off, sms, ctx->d_err, st);
-        if (rc != EXACT_OK || !keys) return rc;
-        return with_footprint(fp, [&](auto fpc) -> int {
-            sdf_keys_finish<decltype(fpc)><<<(n_poses + 255) / 256, 256, 0, st>>>(keys, n_poses, fpc, dmin, argmin);
-            return cuda_status(cudaGetLastError());
-        });
+        cudaGetLastError();   // not this call's error: the general kernel needs no such memory
     }
 
     // one block per pose when there are enough poses to fill the GPU;

@@ -180,11 +180,13 @@ def test_sdf_under_capture_without_scratch_takes_the_general_path(ex):
     assert bool((o["dmin"] == m).all()) and bool((o["argmin"] == a).all())
 
 
-def test_captured_cycle_survives_scratch_growth(ex):
-    """A graph keeps the scratch it was captured with: a later call of the same
-    context that needs more must not take it away."""
+@pytest.mark.parametrize("n_cloud,n_pts", [(1500, 200_000), (500, 20_000), (500, 200_000)])
+def test_captured_cycle_survives_scratch_growth(ex, n_cloud, n_pts):
+    """A graph keeps the scratch it was captured with, and its counters: a later
+    call of the same context, with or without a need for more scratch, must not
+    take either away."""
     import torch
-    s = synth.plain_step(3, K=64, T=10, N=1500)
+    s = synth.plain_step(3, K=64, T=10, N=n_cloud)
     dev = torch.device("cuda")
     t = {k: torch.from_numpy(s[k]).to(dev) for k in ("q0", "cloud", "waypoints", "U", "eps")}
     fp = ex.Footprint(s["kind"], s["fp"])
@@ -203,8 +205,8 @@ def test_captured_cycle_survives_scratch_growth(ex):
     with torch.cuda.graph(graph, stream=side):
         cycle(ctx, outs)
     g = synth.rng(4)
-    pts = torch.from_numpy(g.uniform(-6, 6, (200_000, 2)).astype(np.float32)).to(dev)
-    poses = torch.from_numpy(g.uniform(-3, 3, (300, 3)).astype(np.float32)).to(dev)
+    pts = torch.from_numpy(g.uniform(-6, 6, (n_pts, 2)).astype(np.float32)).to(dev)
+    poses = torch.from_numpy(g.uniform(-3, 3, (1000, 3)).astype(np.float32)).to(dev)
     _, grown, _ = ex.sdf_batch(pts, poses, fp, dist=False, ctx=ctx)
     graph.replay()
     torch.cuda.synchronize()
@@ -214,3 +216,26 @@ def test_captured_cycle_survives_scratch_growth(ex):
     for k in want:
         assert torch.equal(outs[k], want[k]), k
     assert torch.equal(grown, ex.sdf_batch(pts, poses, fp, dist=False)[1])
+
+
+def test_many_pose_calls_of_one_context_overlap(ex):
+    """Calls of many poses on two streams share nothing but the context."""
+    import torch
+    g = synth.rng(5)
+    fp = ex.Footprint(synth.POLYGON, synth.star_polygon(g, 20, 0.3, 1.0))
+    ctx = ex.Context()
+    sets = [(torch.from_numpy(g.uniform(-6, 6, (20_000, 2)).astype(np.float32)).cuda(),
+             torch.from_numpy(g.uniform(-3, 3, (700, 3)).astype(np.float32)).cuda()) for _ in range(2)]
+    streams = [torch.cuda.Stream() for _ in sets]
+    torch.cuda.synchronize()
+    got = []
+    for _ in range(4):
+        for (pts, poses), s in zip(sets, streams):
+            with torch.cuda.stream(s):
+                got.append(ex.sdf_batch(pts, poses, fp, dist=True, ctx=ctx))
+                got.append(ex.sdf_batch(pts, poses, fp, dist=False, ctx=ctx))
+    torch.cuda.synchronize()
+    for i, (d, m, a) in enumerate(got):
+        want = ex.sdf_batch(*sets[i // 2 % 2], fp)
+        assert torch.equal(m, want[1]) and torch.equal(a, want[2])
+        assert d is None or torch.equal(d, want[0])
