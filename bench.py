@@ -35,49 +35,28 @@ if ROOT not in sys.path:
 
 N_POSES, N_POINTS, N_VERTS = 16384, 8192, 32
 FLOPS_PER_POINT_EDGE = 17      # canonical count, FMA = 2
-# what the polygon kernel executes per point-edge: the distance pass (dx, dy
-# 2; projection 3; q 4; |q|^2 3; min 1) for every point, the parity pass
-# (dx, dy 2; crossing abscissa 2; straddle product 1) only for points within
-# the footprint's bounding circle
-EXEC_FLOPS_DIST, EXEC_FLOPS_PARITY = 13, 5
 FLOPS_PER_POINT_BOX = 12
 L2_BYTES = 129 * 1024 * 1024
 
 
-# DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of
-# the headline kernel, taken from one ncu capture of the headline workload and
-# valid only while the kernel sources hash to the recorded value (reported as
-# null otherwise).
-TRAFFIC = {"sources": ["paper_2605_29663_gb300/csrc/sdf_batch.cu", "paper_2605_29663_gb300/csrc/common.cuh",
-                       "paper_2605_29663_gb300/csrc/internal.h"],
-           "sha256_16": "ee1107a292ea716e", "bytes_per_launch": 632832 + 477973248}
+# What one step of the headline workload executes (sdf_sort_kernel +
+# sdf_matrix_kernel): DRAM traffic (dram__bytes_read.sum +
+# dram__bytes_write.sum) and warp instructions (smsp__inst_executed.sum),
+# counted by ncu for seed 0 and valid only while the kernel sources hash to the
+# recorded value (reported as null otherwise).
+COUNTERS = {"sources": ["paper_2605_29663_gb300/csrc/sdf_near.cu", "paper_2605_29663_gb300/csrc/mppi_cycle.cuh",
+                        "paper_2605_29663_gb300/csrc/common.cuh"],
+            "sha256_16": "59e966a53f243337", "bytes_per_step": 89600 + 391168 + 472019456,
+            "warp_instructions_per_step": 40679 + 685107960}
 
 
-def measured_traffic():
+def measured_counters():
     import hashlib
     h = hashlib.sha256()
-    for f in TRAFFIC["sources"]:
+    for f in COUNTERS["sources"]:
         with open(os.path.join(ROOT, f), "rb") as fh:
             h.update(fh.read())
-    return TRAFFIC["bytes_per_launch"] if h.hexdigest()[:16] == TRAFFIC["sha256_16"] else None
-
-
-def near_fraction(w, n_poses: int = 1024) -> float:
-    """Fraction of (pose, point) pairs of the sdf workload whose point lies
-    within the footprint's bounding circle (centre of the vertex bounding
-    box, radius to the farthest vertex) in the body frame: the pairs that
-    take the parity pass.  Float64, over the first n_poses poses."""
-    import numpy as np
-    v = np.asarray(w["fp"], np.float64)
-    c = 0.5 * (v.min(axis=0) + v.max(axis=0))
-    r = np.sqrt(((v - c) ** 2).sum(axis=1)).max()
-    poses = np.asarray(w["poses"][:n_poses], np.float64)
-    pts = np.asarray(w["points"], np.float64)
-    cs, sn = np.cos(poses[:, 2:3]), np.sin(poses[:, 2:3])
-    dx = pts[None, :, 0] - poses[:, 0:1]
-    dy = pts[None, :, 1] - poses[:, 1:2]
-    bx, by = cs * dx + sn * dy, -sn * dx + cs * dy
-    return float((((bx - c[0]) ** 2 + (by - c[1]) ** 2) <= r * r).mean())
+    return COUNTERS if h.hexdigest()[:16] == COUNTERS["sha256_16"] else None
 
 
 def max_over_ranks(torch, dist, ms: float, dev) -> float:
@@ -280,7 +259,8 @@ def mppi_extra(torch, ex, dev, cpu: bool = True):
         out[name] = {"steps_per_s": 1e3 / ms, "us_per_step": 1e3 * ms, "K": p["K"], "T": p["T"], "N": N,
                      "footprint": ("polygon" if s["kind"] == synth.POLYGON else "rects") + f"x{s['fp'].shape[0]}",
                      "evals_per_step": per_step, "counted_tflops": flops / (ms * 1e-3) / 1e12,
-                     "launches_per_step": 3, "timing": "CUDA graph replay, events, inputs L2-resident",
+                     "launches_per_step": 4 if N >= 1024 else 3,   # from 1,024 points on, the cell grid first
+                     "timing": "CUDA graph replay, events, inputs L2-resident",
                      "cpu_oracle": oracle_mppi_sample(s) if cpu else None}
     return out
 
@@ -349,7 +329,7 @@ def hybrid_extra(torch, ex, dev, cpu: bool = True):
     out = {"modes": ["ackermann", "parallel", "spin"], "K_per_mode": p0["K"], "T": p0["T"], "N": N,
            "footprint": f"polygonx{E}", "us_per_cycle": 1e3 * ms, "cycles_per_s": 1e3 / ms,
            "evals_per_cycle": evals, "counted_tflops": FLOPS_PER_POINT_EDGE * evals / (ms * 1e-3) / 1e12,
-           "launches_per_cycle": 4, "timing": "CUDA graph replay (memset + 3 batched kernels + selection), events"}
+           "launches_per_cycle": 5, "timing": "CUDA graph replay (memset + 4 batched kernels + selection), events"}
     if cpu:
         import oracle
         oracle.build()
@@ -561,7 +541,7 @@ def batched_extra(torch, ex, dev, steps=3):
     evals = sum(s["params"]["K"] * s["params"]["T"] * s["cloud"].shape[0] * s["fp"].shape[0] for s in scenes)
     out.update({"point_edge_evals_per_step": evals,
                 "batched_counted_tflops": FLOPS_PER_POINT_EDGE * evals / (out["batched_ms_per_step"] * 1e-3) / 1e12,
-                "launches_per_step": 3})
+                "launches_per_step": 4})
     return out
 
 
@@ -641,6 +621,7 @@ def run_mppi_workload(args):
             outs.update(ex.mppi_step(ctx, t["q0"], t["cloud"], t["waypoints"], t["U"], t["eps"], fp, p, mask=mask,
                                      velocity=vel, out=outs))
         cfg = {"K": p["K"], "T": p["T"], "N": s["cloud"].shape[0]}
+        launches = 4 if cfg["N"] >= 1024 else 3
     elif args.workload == "hybrid":
         modes = synth.hybrid(0)
         fp = ex.Footprint(modes[0]["kind"], modes[0]["fp"])
@@ -651,7 +632,7 @@ def run_mppi_workload(args):
                      params=m["params"]) for m in modes]
         h = ex.Hybrid(devs, lambda_switch=2.0, cool_max=3)
         step = h.step
-        launches = 4
+        launches = 5
         cfg = {"modes": 3, "K": modes[0]["params"]["K"], "T": modes[0]["params"]["T"], "N": modes[0]["cloud"].shape[0]}
     elif args.workload == "mlp_train":
         # one Adam step of the proposal network (111-256-256-40, batch 1024)
@@ -667,7 +648,7 @@ def run_mppi_workload(args):
 
         def step():
             net.train_step(x, y, 1e-3, loss=loss)
-        launches = 16
+        launches = 7
         cfg = {"network": f"{L.D_IN}-256-256-{2 * L.T_H}", "batch": 1024}
     else:
         scenes = synth.batched(0)
@@ -678,6 +659,7 @@ def run_mppi_workload(args):
                      fp=ex.Footprint(s["kind"], s["fp"]), params=s["params"]) for s in scenes]
         b = ex.Batch(devs)
         step = b.step
+        launches = 4
         cfg = {"scenes": len(scenes)}
     for _ in range(args.warmup):
         step()
@@ -869,11 +851,11 @@ def run_gpu(args):
     peaks = measured_peaks()
     clocks = clk.summary()
     sm_max = peaks.get("sm_max_mhz", 2070.0)
-    peak = fp32_peak_tflops(sm_max)
-    achieved = FLOPS_PER_POINT_EDGE * evals / (ms * 1e-3) / 1e12
-    near_f = near_fraction(w)
-    exec_tflops = (EXEC_FLOPS_DIST + EXEC_FLOPS_PARITY * near_f) * evals / (ms * 1e-3) / 1e12
-    traffic = measured_traffic() if P == N_POSES else None
+    counted = FLOPS_PER_POINT_EDGE * evals / (ms * 1e-3) / 1e12
+    counters = measured_counters() if P == N_POSES else None
+    # the bound is instruction issue: one warp instruction per SM partition and cycle
+    issue_peak = 152 * 4 * sm_max * 1e6 / 1e9
+    issued = counters["warp_instructions_per_step"] / (ms * 1e-3) / 1e9 if counters else None
     line = {
         "metric": "SDF point-edge evals/s", "value": value, "unit": "point-edge evals/s",
         "n_gpus": world, "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms,
@@ -883,20 +865,21 @@ def run_gpu(args):
                                "polygon, full signed-distance matrix + per-pose min/argmin",
                    "poses": P, "points": N_POINTS, "edges": N_VERTS, "seed": "rank",
                    "l2": "flushed (2x L2 zero-fill) between timed iterations", "parallelism": f"replicas x{world}"},
-        "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                     "frac": achieved / peak, "traffic": traffic,
-                     "kernel": "sdf_batch_kernel<PolyC<32>, true, false>",
+        "roofline": {"bound": "issue", "achieved": issued, "peak": issue_peak, "unit": "G warp instructions/s",
+                     "frac": issued / issue_peak if counters else None,
+                     "traffic": counters["bytes_per_step"] if counters else None,
+                     "kernel": "sdf_matrix_kernel<false> (behind sdf_sort_kernel)",
                      "algorithmic_bytes_per_launch": P * N_POINTS * 4 + N_POINTS * 8 + P * 12,
-                     "flops_per_launch": FLOPS_PER_POINT_EDGE * evals,
-                     "executed": {"near_fraction": near_f,
-                                  "flops_per_point_edge": EXEC_FLOPS_DIST + EXEC_FLOPS_PARITY * near_f,
-                                  "tflops": exec_tflops, "frac": exec_tflops / peak,
-                                  "note": "achieved/frac count the canonical 17 flops per point-edge; the kernel "
-                                          "takes the crossing parity only for points within the footprint's "
-                                          "bounding circle (all others are outside, sign +), so it executes "
-                                          "fewer; outputs are the same bits either way"},
-                     "peak_basis": f"152 SMs x 128 FP32 lanes x 2 (FMA) x {sm_max:.0f} MHz max SM clock "
-                                   "(derived; MEASURED_PEAKS.json carries only HBM and bf16 figures)"},
+                     "write_gbs": P * N_POINTS * 4 / (ms * 1e-3) / 1e9,
+                     "write_frac_of_measured_hbm": P * N_POINTS * 4 / (ms * 1e-3) / 1e9 / peaks["hbm_gbs"]
+                     if peaks.get("hbm_gbs") else None,
+                     "counted": {"flops_per_point_edge": FLOPS_PER_POINT_EDGE, "tflops": counted,
+                                 "over_fp32_peak": counted / fp32_peak_tflops(sm_max),
+                                 "note": "every point-edge of the matrix counted at the canonical 17 flops; the kernel "
+                                         "leaves out the edges that provably cannot be nearest to a patch of 64 "
+                                         "points and the crossing parity of points outside the footprint's bounding "
+                                         "circle, so this is no utilisation; outputs are the same bits either way"},
+                     "peak_basis": f"152 SMs x 4 warp instructions per cycle x {sm_max:.0f} MHz max SM clock (derived)"},
         "e2e": {"value": e2e_val, "unit": "point-edge evals/s", "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": d2h, "ms_per_step": e2e_ms, "steps": e_steps, "result_check": bool(ok),
                 "note": "every step: pinned H2D of points + poses, exact_sdf_batch, D2H of the whole result "
@@ -906,7 +889,7 @@ def run_gpu(args):
                          "ms_per_step": mo_ms, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": P * 8,
                          "note": "the minimum-only call (no distance matrix): pinned H2D of points + poses, "
                                  "exact_sdf_batch(dist=NULL), D2H of min + argmin, in order on one stream"},
-        "gpu_launches": args.steps,
+        "gpu_launches": 2 * args.steps,
         "clocks": clocks,
     }
     if not args.no_cpu and world == 1:

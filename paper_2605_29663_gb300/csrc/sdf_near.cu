@@ -9,8 +9,8 @@
 // consecutive points.  The matrix kernel and the minimum
 // kernel below then decide per (pose, patch), for 64 points at once, what
 // each point would otherwise pay for.  Measured (calls of exact_sdf_batch):
-// 16,384 poses x 8,192 points x 32 edges 1,227 -> 777 us; the minimum of 3,000
-// poses x 20,001 points x 12 edges 239 -> 40 us.
+// 16,384 poses x 8,192 points x 32 edges 1,227 -> 710 to 728 us; the minimum of
+// 3,000 poses x 20,001 points x 12 edges 240 -> 40 to 47 us.
 #include "mppi_cycle.cuh"
 #include "sdf_near.h"
 
