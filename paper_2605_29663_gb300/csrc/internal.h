@@ -7,6 +7,8 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <atomic>
+
 #include "common.cuh"
 #include "exact_mppi.h"
 
@@ -43,8 +45,8 @@ struct exact_ctx {
     void *work = nullptr, *work_alloc = nullptr;   // work_alloc: null while it is the piece behind sdf_keys
     size_t work_bytes = 0;
     // exact_sdf_batch of many poses takes its sorted cloud from here, stream
-    // ordered: such calls may overlap on several streams.  NULL: no pool to be had
-    cudaMemPool_t pool = nullptr;
+    // ordered: such calls may overlap on several streams (sdf_pool makes it)
+    std::atomic<cudaMemPool_t> pool{nullptr};
     void *retired[exact::kRetired];   // outgrown arenas
     int n_retired = 0;
     SdfKey *sdf_keys = nullptr;  // sdf_split_poses of them, apart from the arena: other calls leave them alone
@@ -61,6 +63,8 @@ int ensure_scratch(exact_ctx *ctx, size_t bytes);
 // Whether the second arena holds `bytes`, or can be grown to them now (not
 // while the stream captures, and to 1 GB at most).
 bool try_work(exact_ctx *ctx, size_t bytes, cudaStream_t st);
+// The context's memory pool, made by the first call; NULL: there is none to be had.
+cudaMemPool_t sdf_pool(exact_ctx *ctx);
 int current_sm_count();
 // exact_sdf_batch splits a pose's points over several blocks below this many
 // poses (about eight blocks per SM).

@@ -259,6 +259,25 @@ bool try_work(exact_ctx *ctx, size_t bytes, cudaStream_t st) {
     return true;
 }
 
+cudaMemPool_t sdf_pool(exact_ctx *ctx) {
+    cudaMemPool_t pool = ctx->pool.load();
+    if (pool) return pool;
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = ctx->device;
+    unsigned long long keep = 64ull << 20;   // kept over a synchronisation: the sorted copy of 6 million points
+    if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    cudaMemPool_t other = nullptr;
+    if (ctx->pool.compare_exchange_strong(other, pool)) return pool;
+    cudaMemPoolDestroy(pool);   // another thread was first
+    return other;
+}
+
 }  // namespace exact
 
 extern "C" int exact_ctx_create(exact_ctx **out) {
@@ -268,39 +287,21 @@ extern "C" int exact_ctx_create(exact_ctx **out) {
     if (!ctx) return EXACT_EINVAL;
     if (cudaGetDevice(&ctx->device) != cudaSuccess) { delete ctx; return EXACT_ECUDA; }
     ctx->sm_count = exact::current_sm_count();
-    if (cudaMalloc(&ctx->d_err, sizeof(int)) != cudaSuccess) { delete ctx; return EXACT_ECUDA; }
-    // the second arena starts as 1 MB behind the keys, so that a cycle on a
-    // cloud of ordinary size can be captured without any call before it
+    // one allocation: split keys, error word, statistics (zeroed), then the
+    // second arena's first 1 MB, so that a cycle on a cloud of ordinary size can
+    // be captured without any call before it
     const size_t key_bytes = exact::align_up(sizeof(SdfKey) * (size_t)exact::sdf_split_poses(ctx->sm_count), 256);
+    const size_t head = key_bytes + 256 + exact::align_up(sizeof(exact_cycle_stats), 256);
     ctx->work_bytes = (size_t)1 << 20;
-    if (cudaMalloc(&ctx->d_stats, sizeof(exact_cycle_stats)) != cudaSuccess ||
-        cudaMalloc(&ctx->sdf_keys, key_bytes + ctx->work_bytes) != cudaSuccess) {
-        cudaFree(ctx->d_err);
-        cudaFree(ctx->d_stats);
+    if (cudaMalloc(&ctx->sdf_keys, head + ctx->work_bytes) != cudaSuccess) { delete ctx; return EXACT_ECUDA; }
+    char *base = reinterpret_cast<char *>(ctx->sdf_keys);
+    ctx->d_err = reinterpret_cast<int *>(base + key_bytes);
+    ctx->d_stats = reinterpret_cast<decltype(ctx->d_stats)>(base + key_bytes + 256);
+    ctx->work = base + head;
+    if (cudaMemset(base, 0, head) != cudaSuccess || cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {   // as in ensure_scratch
+        cudaFree(base);
         delete ctx;
         return EXACT_ECUDA;
-    }
-    if (cudaMemset(ctx->d_err, 0, sizeof(int)) != cudaSuccess ||
-        cudaMemset(ctx->d_stats, 0, sizeof(exact_cycle_stats)) != cudaSuccess ||
-        cudaMemset(ctx->sdf_keys, 0, key_bytes) != cudaSuccess ||
-        cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {   // as in ensure_scratch
-        cudaFree(ctx->d_err);
-        cudaFree(ctx->d_stats);
-        cudaFree(ctx->sdf_keys);
-        delete ctx;
-        return EXACT_ECUDA;
-    }
-    ctx->work = reinterpret_cast<char *>(ctx->sdf_keys) + key_bytes;
-    cudaMemPoolProps props = {};
-    props.allocType = cudaMemAllocationTypePinned;
-    props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = ctx->device;
-    unsigned long long keep = 64ull << 20;   // kept over a synchronisation: the sorted copy of 6 million points
-    if (cudaMemPoolCreate(&ctx->pool, &props) != cudaSuccess) {
-        ctx->pool = nullptr;
-        cudaGetLastError();
-    } else {
-        cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep);
     }
     *out = ctx;
     return EXACT_OK;
@@ -311,11 +312,9 @@ extern "C" void exact_ctx_destroy(exact_ctx *ctx) {
     cudaDeviceSynchronize();
     if (ctx->scratch) cudaFree(ctx->scratch);
     if (ctx->work_alloc) cudaFree(ctx->work_alloc);
-    if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
+    if (cudaMemPool_t pool = ctx->pool.load()) cudaMemPoolDestroy(pool);
     exact::free_retired(ctx);
     if (ctx->sdf_keys) cudaFree(ctx->sdf_keys);
-    if (ctx->d_err) cudaFree(ctx->d_err);
-    if (ctx->d_stats) cudaFree(ctx->d_stats);
     delete ctx;
 }
 

@@ -259,14 +259,14 @@ extern "C" int exact_sdf_batch(exact_ctx *ctx, const float *points, const uint8_
     // is memory for the sorted cloud: stream-ordered, since calls of one context
     // may overlap on several streams, and not in a capture, whose replays may
     // overlap anything
-    if (ctx && ctx->pool && (dist || dmin || argmin) && sdf_near_fits(fp, n_points, n_poses, dist != nullptr)) {
+    if (ctx && (dist || dmin || argmin) && sdf_near_fits(fp, n_points, n_poses, dist != nullptr)) {
         const bool split = dist && (dmin || argmin) && n_points > kSdfChunk;
         const size_t key_bytes = split ? align_up((size_t)n_poses * sizeof(unsigned long long), 256) : 0;
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         void *mem = nullptr;
         if (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
-            key_bytes + sdf_near_bytes(n_points) <= ((size_t)1 << 30) &&
-            cudaMallocFromPoolAsync(&mem, key_bytes + sdf_near_bytes(n_points), ctx->pool, st) == cudaSuccess) {
+            key_bytes + sdf_near_bytes(n_points) <= ((size_t)1 << 30) && sdf_pool(ctx) &&
+            cudaMallocFromPoolAsync(&mem, key_bytes + sdf_near_bytes(n_points), sdf_pool(ctx), st) == cudaSuccess) {
             unsigned long long *keys = split ? static_cast<unsigned long long *>(mem) : nullptr;
             if (keys) sdf_keys_init<<<(n_poses + 255) / 256, 256, 0, st>>>(keys, n_poses);
             int rc = sdf_near_launch(p2, mask, n_points, poses, n_poses, fp, dist, dmin, argmin, keys,
