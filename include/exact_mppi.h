@@ -83,7 +83,14 @@ int exact_footprint_info(const exact_footprint *fp, int *kind, int *n);
  * exact_sdf_batch reduction, plus a device error word.  It is bound to the
  * device that is current at creation.  Scratch grows on demand (a call with
  * larger sizes than any before may allocate, which must not happen during
- * stream capture); exact_ctx_reserve allocates ahead of time. */
+ * stream capture); exact_ctx_reserve allocates ahead of time.
+ *
+ * Calls that share a context share its scratch: they, and replays of graphs
+ * that captured them, must not overlap on the GPU (use one context per
+ * stream).  Calls that overlap all the same spoil each other's results, and no
+ * later call's.  Excepted are exact_sdf_batch calls of at least one pose per SM,
+ * of at most 4,096 points, or without dmin and argmin: they keep nothing in the
+ * context that another call could meet, and may overlap with any call. */
 typedef struct exact_ctx exact_ctx;
 int exact_ctx_create(exact_ctx **out);
 void exact_ctx_destroy(exact_ctx *ctx);

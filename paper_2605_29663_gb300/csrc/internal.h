@@ -29,7 +29,7 @@ struct exact_footprint {
 namespace exact { constexpr int kRetired = 128; }   // two arenas, doubled from 1 MB on: at most 40 steps each
 
 // Minimum of one pose of a split exact_sdf_batch (complemented packed key; 0
-// = empty) and its finished blocks; both zero between calls.
+// = empty) and its finished blocks; each call clears its own first.
 struct SdfKey {
     unsigned long long best;
     unsigned ticket, pad;
@@ -49,7 +49,7 @@ struct exact_ctx {
     std::atomic<cudaMemPool_t> pool{nullptr};
     void *retired[exact::kRetired];   // outgrown arenas
     int n_retired = 0;
-    SdfKey *sdf_keys = nullptr;  // sdf_split_poses of them, apart from the arena: other calls leave them alone
+    SdfKey *sdf_keys = nullptr;  // sdf_split_poses of them, apart from the arena
     int *d_err = nullptr;        // device error word (exact_status)
     long long mppi_layout = -1;  // (K, T, parts) of the last mppi_step; -1 = arena reused otherwise
     bool stats = false;          // mppi_step also records cycle statistics

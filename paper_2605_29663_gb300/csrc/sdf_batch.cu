@@ -7,17 +7,36 @@
 // 256 contiguous bytes of the distance row with streaming stores.  The pose's
 // sincos is taken once per thread; the footprint sits in the constant bank.
 // Minima are reduced per block (warp shuffles over packed (key, index)
-// words); when several blocks share a pose they meet in a per-pose key of the
-// context, and the last of them (atomic ticket) writes the result and empties
-// the key: one launch (a call for 1 pose x 1,000 points: 11.6 to 13.7 us with
-// its host side, 14 to 17 us with an initialising and a finishing kernel).
-#include "internal.h"
+// words).  Up to eight blocks that share a pose are a cluster, whose first
+// block collects the others' words from their shared memory: one launch, and
+// nothing kept anywhere (a call for 1 pose x 1,000 points: 6.2 us with its host
+// side).  More blocks meet in a per-pose key of the context, and the last of
+// them (atomic ticket) writes the result; every such call clears its keys
+// first, in stream order, so that nothing one call leaves behind reaches
+// another (1 pose x 20,000 points: 7.3 us).  The clear is a launch of its own
+// that the kernel only waits for where it takes a ticket (programmatic
+// dependent launch).
+#include "mppi_cycle.cuh"
 #include "sdf_near.h"
 
 namespace exact {
 
 constexpr int kSdfBlock = 128;   // threads per block (measured 1% faster than 256 at the same occupancy)
 constexpr int kNearQ = 128;   // per-warp queue of near points (two batches)
+constexpr int kSdfCluster = 8;   // most blocks of a cluster (the portable size)
+
+// Barrier of the cluster's threads, with release and acquire.
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// *p as it stands in the shared memory of block `rank` of the cluster.
+__device__ __forceinline__ unsigned long long cluster_load(const unsigned long long *p, int rank) {
+    unsigned a;
+    unsigned long long v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_addr(p)), "r"(rank));
+    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
+    return v;
+}
 
 // Polygon rows: point pairs [pbeg, pend) of one pose.  The edge loop takes
 // the distances only.  The crossing parity can be odd only for a point within
@@ -200,25 +219,42 @@ sdf_batch_kernel(const float2 *__restrict__ pts, const uint8_t *__restrict__ mas
     unsigned long long best = bi < 0 ? kNoKey : pack_key(bk, (unsigned)bi);
     best = warp_min_u64(best);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = best;
-    __syncthreads();
-    if (threadIdx.x == 0) {
+    const bool cluster = chunks > 1 && !keys;   // a pose's blocks are one cluster
+    if (cluster) cluster_sync();
+    else __syncthreads();
+    if (threadIdx.x == 0 && !(cluster && chunk > 0)) {
         unsigned long long b = red[0];
 #pragma unroll
         for (int w = 1; w < kSdfBlock / 32; ++w) b = red[w] < b ? red[w] : b;
-        if (chunks > 1) {
+        if (cluster) {
+            for (int k = 1; k < chunks; ++k)
+#pragma unroll
+                for (int w = 0; w < kSdfBlock / 32; ++w) {
+                    const unsigned long long o = cluster_load(red + w, k);
+                    b = o < b ? o : b;
+                }
+        } else if (chunks > 1) {
             // the blocks of a pose meet in its key (complemented: 0 is empty);
-            // the last one (ticket) takes it and empties it for the next call
+            // the last one (ticket) takes it
+            grid_dep_wait();   // the keys are cleared
             SdfKey *key = keys + pose;
             if (b != kNoKey) atomicMax(&key->best, ~b);
             __threadfence();
             if (atomicAdd(&key->ticket, 1u) != (unsigned)chunks - 1) return;
             __threadfence();
-            b = ~atomicExch(&key->best, 0ull);
-            key->ticket = 0u;
+            b = ~atomicMax(&key->best, 0ull);
         }
         if (dmin) dmin[pose] = b == kNoKey ? finf() : key_to_dist(fpc, ord2f((unsigned)(b >> 32)));
         if (argmin) argmin[pose] = b == kNoKey ? -1 : (int)(unsigned)(b & 0xffffffffu);
     }
+    if (cluster) cluster_sync();   // the others' shared memory stays until it has been read
+}
+
+// The keys of a split call, empty.
+__global__ void sdf_keys_clear(SdfKey *keys, int P) {
+    grid_dep_release();
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p < P) keys[p] = SdfKey{0ull, 0u, 0u};
 }
 
 // Per-pose minima over the chunks of the pruned path's kernel (sdf_near.cu).
@@ -256,9 +292,9 @@ extern "C" int exact_sdf_batch(exact_ctx *ctx, const float *points, const uint8_
     if (sms <= 0) sms = current_sm_count();
     const float2 *p2 = reinterpret_cast<const float2 *>(points);
     // many poses against one cloud: the pruned path (sdf_near.cu), where there
-    // is memory for the sorted cloud: stream-ordered, since calls of one context
-    // may overlap on several streams, and not in a capture, whose replays may
-    // overlap anything
+    // is memory for the sorted cloud: each call's own, stream-ordered, since
+    // calls of a pose per SM or more may overlap on several streams, and not in
+    // a capture, whose replays may overlap anything
     if (ctx && (dist || dmin || argmin) && sdf_near_fits(fp, n_points, n_poses, dist != nullptr)) {
         const bool split = dist && (dmin || argmin) && n_points > kSdfChunk;
         const size_t key_bytes = split ? align_up((size_t)n_poses * sizeof(unsigned long long), 256) : 0;
@@ -291,17 +327,40 @@ extern "C" int exact_sdf_batch(exact_ctx *ctx, const float *points, const uint8_
         const int max_chunks = (npairs + 255) / 256;
         if (chunks > max_chunks) chunks = max_chunks;
     }
-    if (chunks > 1 && (dmin || argmin) && !ctx) chunks = 1;   // no arena for the cross-block minimum
+    if (chunks > 1 && (dmin || argmin) && !ctx) chunks = 1;   // the call without a context: one block per pose
     if ((long long)n_poses * chunks > 0x7fffffffLL) chunks = 1;
+    // (always so from one pose per SM on)
+    const bool cluster = chunks > 1 && chunks <= kSdfCluster && (dmin || argmin);
+    if (cluster) chunks = chunks > 4 ? 8 : chunks > 2 ? 4 : 2;
     const int chunk_pairs = (npairs + chunks - 1) / chunks;
     const int vec = dist && (n_points % 2 == 0) && (((uintptr_t)dist & 7u) == 0);
 
-    SdfKey *keys = chunks > 1 && (dmin || argmin) ? ctx->sdf_keys : nullptr;
+    SdfKey *keys = chunks > 1 && !cluster && (dmin || argmin) ? ctx->sdf_keys : nullptr;
     const unsigned grid = (unsigned)(n_poses * chunks);
     return with_footprint(fp, [&](auto fpc) -> int {
         using FPC = decltype(fpc);
         auto k = mask ? (dist ? sdf_batch_kernel<FPC, true, true> : sdf_batch_kernel<FPC, false, true>)
                       : (dist ? sdf_batch_kernel<FPC, true, false> : sdf_batch_kernel<FPC, false, false>);
+        if (cluster) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(grid);
+            cfg.blockDim = dim3(kSdfBlock);
+            cfg.stream = st;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = (unsigned)chunks;
+            attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            return cuda_status(cudaLaunchKernelEx(&cfg, k, p2, mask, n_points, poses, fpc, dist, vec, dmin, argmin, keys,
+                                                  chunks, chunk_pairs, ctx->d_err));
+        }
+        if (keys) {
+            sdf_keys_clear<<<(n_poses + 255) / 256, 256, 0, st>>>(keys, n_poses);
+            if (cudaGetLastError() != cudaSuccess) return EXACT_ECUDA;
+            return cuda_status(launch_dependent(k, grid, (unsigned)kSdfBlock, 0, st, p2, mask, n_points, poses, fpc, dist, vec,
+                                                dmin, argmin, keys, chunks, chunk_pairs, ctx->d_err));
+        }
         k<<<grid, kSdfBlock, 0, st>>>(p2, mask, n_points, poses, fpc, dist, vec, dmin, argmin, keys, chunks,
                                    chunk_pairs, ctx ? ctx->d_err : nullptr);
         return cuda_status(cudaGetLastError());
