@@ -51,7 +51,11 @@ struct exact_ctx {
     int n_retired = 0;
     SdfKey *sdf_keys = nullptr;  // sdf_split_poses of them, apart from the arena
     int *d_err = nullptr;        // device error word (exact_status)
-    long long mppi_layout = -1;  // (K, T, parts) of the last mppi_step; -1 = arena reused otherwise
+    // finished horizon parts per sample (ticket_count of them), zero between
+    // cycles: the update rearms them.  Apart from the arena, whose layout follows
+    // each cycle's sizes: a graph replayed after a cycle of other sizes finds
+    // its tickets as it left them
+    unsigned *part_tickets = nullptr;
     bool stats = false;          // mppi_step also records cycle statistics
     exact_cycle_stats *d_stats = nullptr;   // device record of those statistics
 };
@@ -69,6 +73,8 @@ int current_sm_count();
 // exact_sdf_batch splits a pose's points over several blocks below this many
 // poses (about eight blocks per SM).
 inline int sdf_split_poses(int sms) { return (sms > 0 ? sms : 148) * 8; }
+// A cycle splits its samples' horizons below this many samples (parts_for).
+inline int ticket_count(int sms) { return sms > 0 ? sms : 148; }
 // Arena bytes needed by exact_sdf_batch (n_poses) and mppi_step (K, T).
 size_t sdf_scratch_bytes(int n_poses);
 

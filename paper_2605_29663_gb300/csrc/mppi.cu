@@ -93,9 +93,7 @@ cycle_stats_kernel(const double *__restrict__ Jt, const float *__restrict__ wt, 
     }
 }
 
-static int parts_of(const exact_ctx *ctx, int K, int T) {
-    return parts_for(K, T, ctx->sm_count > 0 ? ctx->sm_count : 148);
-}
+static int parts_of(const exact_ctx *ctx, int K, int T) { return parts_for(K, T, ticket_count(ctx->sm_count)); }
 
 int check_params(const exact_mppi_params *p) {
     if (!p) return EXACT_EINVAL;
@@ -196,13 +194,8 @@ int mppi_step_impl(exact_ctx *ctx, const float *state, const float *cloud, const
     V.upd_blocks = upd_blocks_for(P.K, P.T, P.nu);
     V.val_chunks = val_chunks_for(n_points, grid);
     cudaStream_t st = (cudaStream_t)stream;
-    // the per-sample part tickets rearm themselves after each cycle; zero
-    // them once whenever the arena layout changes
-    const long long layout = ((long long)P.K << 24) ^ ((long long)P.T << 8) ^ V.parts;
-    if (V.parts > 1 && ctx->mppi_layout != layout) {
-        if (cudaMemsetAsync(V.tk, 0, (size_t)P.K * sizeof(unsigned), st) != cudaSuccess) return EXACT_ECUDA;
-    }
-    ctx->mppi_layout = layout;
+    // the samples' part tickets, apart from the arena (see exact_ctx)
+    if (V.parts > 1) V.tk = ctx->part_tickets;
     const int sms = ctx->sm_count > 0 ? ctx->sm_count : current_sm_count();
     if (grid) {
         char *q = room;

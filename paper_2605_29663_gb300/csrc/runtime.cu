@@ -237,7 +237,6 @@ int ensure_scratch(exact_ctx *ctx, size_t bytes) {
     retire(ctx, ctx->scratch);
     ctx->scratch = p;
     ctx->scratch_bytes = got;
-    ctx->mppi_layout = -1;
     return EXACT_OK;
 }
 
@@ -287,16 +286,19 @@ extern "C" int exact_ctx_create(exact_ctx **out) {
     if (!ctx) return EXACT_EINVAL;
     if (cudaGetDevice(&ctx->device) != cudaSuccess) { delete ctx; return EXACT_ECUDA; }
     ctx->sm_count = exact::current_sm_count();
-    // one allocation: split keys, error word, statistics (zeroed), then the
+    // one allocation: split keys, error word, statistics, part tickets (zeroed), then the
     // second arena's first 1 MB, so that a cycle on a cloud of ordinary size can
     // be captured without any call before it
     const size_t key_bytes = exact::align_up(sizeof(SdfKey) * (size_t)exact::sdf_split_poses(ctx->sm_count), 256);
-    const size_t head = key_bytes + 256 + exact::align_up(sizeof(exact_cycle_stats), 256);
+    const size_t stats_bytes = exact::align_up(sizeof(exact_cycle_stats), 256);
+    const size_t head = key_bytes + 256 + stats_bytes +
+                        exact::align_up(sizeof(unsigned) * (size_t)exact::ticket_count(ctx->sm_count), 256);
     ctx->work_bytes = (size_t)1 << 20;
     if (cudaMalloc(&ctx->sdf_keys, head + ctx->work_bytes) != cudaSuccess) { delete ctx; return EXACT_ECUDA; }
     char *base = reinterpret_cast<char *>(ctx->sdf_keys);
     ctx->d_err = reinterpret_cast<int *>(base + key_bytes);
     ctx->d_stats = reinterpret_cast<decltype(ctx->d_stats)>(base + key_bytes + 256);
+    ctx->part_tickets = reinterpret_cast<unsigned *>(base + key_bytes + 256 + stats_bytes);
     ctx->work = base + head;
     if (cudaMemset(base, 0, head) != cudaSuccess || cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {   // as in ensure_scratch
         cudaFree(base);

@@ -75,3 +75,61 @@ def test_clustered_blocks_of_a_pose_meet(ex, P, N):
     torch.cuda.synchronize()
     for k, r in enumerate(got):
         assert all(torch.equal(a, b) for a, b in zip(r, want[k // 3]))
+
+
+class _Cycle:
+    """A cycle on buffers of its own, from the same nominal every time."""
+
+    def __init__(self, ex, ctx, K, T, N, dmin, seed):
+        s = synth.plain_step(seed, K=K, T=T, N=N)
+        s["params"] = synth.mppi_params(K, T, synth.OMNI)
+        s["eps"], s["U"] = synth.noise(synth.rng(seed), K, T, (0.5, 0.5, 1.0)), np.full((T, 3), 0.2, np.float32)
+        self.ex, self.ctx, self.dmin, self.out = ex, ctx, dmin, {}
+        self.t = {k: _t(s[k]) for k in ("q0", "cloud", "waypoints", "U", "eps")}
+        self.u0, self.fp, self.params = self.t["U"].clone(), ex.Footprint(s["kind"], s["fp"]), s["params"]
+
+    def run(self, ctx=None, out=None):
+        t, out = self.t, self.out if out is None else out
+        t["U"].copy_(self.u0)
+        out.update(self.ex.mppi_step(ctx or self.ctx, t["q0"], t["cloud"], t["waypoints"], t["U"], t["eps"], self.fp,
+                                     self.params, dmin=self.dmin, out=out))
+
+    def check(self, what):
+        import torch
+        torch.cuda.synchronize()
+        got, want = {k: v.clone() for k, v in self.out.items()}, {}
+        for v in self.out.values():
+            v.zero_()
+        self.run(self.ex.Context(), want)
+        torch.cuda.synchronize()
+        for k in want:
+            assert torch.equal(got[k], want[k]), (what, k)
+
+
+@pytest.mark.parametrize("dmin,N", [(False, 300), (True, 2000)])
+@pytest.mark.parametrize("a,b", [((64, 10), (128, 20)), ((151, 5), (40, 128)), ((16, 64), (1000, 30)), ((100, 12), (60, 40))])
+def test_replays_and_eager_cycles_of_other_sizes_take_turns(ex, a, b, dmin, N):
+    """Horizons split over several blocks: a graph replayed between eager cycles
+    of other sizes on the same context, and eager cycles of one size with a
+    replay of another between them, each give what a fresh context gives."""
+    import torch
+    ctx = ex.Context()
+    ctx.reserve(0, 1000, 128, N)
+    A, B = _Cycle(ex, ctx, *a, N, dmin, 1), _Cycle(ex, ctx, *b, N, dmin, 2)
+    B.run()
+    A.run()   # the usual warm-up before a capture
+    torch.cuda.synchronize()
+    graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.graph(graph, stream=side):
+        A.run()
+    for k in range(3):
+        B.run()
+        B.check(f"eager {k}")
+        graph.replay()
+        A.check(f"replay {k}")
+        graph.replay()
+        B.run()
+        A.check(f"replay before eager {k}")
+        B.run()
+        B.check(f"eager after replay {k}")
