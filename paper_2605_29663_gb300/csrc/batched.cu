@@ -138,7 +138,7 @@ static int batch_grid(exact_batch *b) {
     int per_sm = 0;
     // the staged points and footprint slots (dynamic) plus the sample state
     // (static) exceed the default 48 KB per block
-    if (cudaFuncSetAttribute(batched_sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem) !=
+    if (cudaFuncSetAttribute(batched_sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSampleSmemMax) !=
         cudaSuccess)
         return EXACT_ECUDA;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batched_sample_kernel, b->threads, b->smem) !=
@@ -148,7 +148,7 @@ static int batch_grid(exact_batch *b) {
     b->grid = b->sms * per_sm;
     if (b->n_gitems == 0) return EXACT_OK;
     if (cudaFuncSetAttribute(batched_grid_sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)grid_smem(b)) != cudaSuccess ||
+                             (int)kGridSmemMax) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batched_grid_sample_kernel, b->threads, grid_smem(b)) !=
             cudaSuccess)
         return EXACT_ECUDA;

@@ -8,6 +8,9 @@
 namespace exact {
 
 constexpr size_t kHdrStride = 64;                            // bytes between scene headers
+// Most dynamic shared memory of the sample kernels: footprint slots and staged
+// points.  Every plan sets this limit (see kGridSmemMax).
+constexpr size_t kSampleSmemMax = kFpSlots * sizeof(float4) + kStage * sizeof(float2);
 
 struct SceneDev {
     SceneView V;

@@ -51,7 +51,7 @@ int launch_uniform_sample_t(exact_batch *b, const SceneDev *table, cudaStream_t 
     if (b->grid_c <= 0) {
         int per_sm = 0;
         // staged points (dynamic) and sample state (static) exceed the default 48 KB per block
-        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b->smem) != cudaSuccess ||
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSampleSmemMax) != cudaSuccess ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, b->threads, b->smem) != cudaSuccess ||
             per_sm < 1)
             return EXACT_ECUDA;

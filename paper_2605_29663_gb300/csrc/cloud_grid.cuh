@@ -193,6 +193,12 @@ __host__ __device__ constexpr int grid_T_pad(int T) { return (T + 3) / 4 * 4; }
 __host__ __device__ constexpr size_t grid_smem_bytes(int T, int samples, int warps) {
     return kField * kField * 4 + (size_t)grid_T_pad(T) * 32 * samples + kGroup * 4 + (size_t)warps * (kRuns * 12 + kEvals * 8);
 }
+// grid_group keeps a block of 256 threads to kGridSmem; the largest block has
+// 512.  The kernels' limit is always set to kGridSmemMax, whatever a call or a
+// plan needs itself: the limit belongs to the kernel, and a smaller one would
+// be another plan's or thread's too.
+constexpr size_t kGridSmem = 70 * 1024, kGridSmemMax = kGridSmem + (512 - kBlock) / 32 * (kRuns * 12 + kEvals * 8);
+static_assert(grid_smem_bytes(EXACT_MAX_HORIZON, 1, kBlock / 32) <= kGridSmem, "one sample of the longest horizon fits");
 
 // Samples per block: as few as keep the blocks to three per SM, so that a small
 // sample count still spreads over the GPU, and up to 16 beyond, which is where
@@ -203,7 +209,7 @@ __host__ __device__ constexpr size_t grid_smem_bytes(int T, int samples, int war
 inline int grid_group(long long samples, int T, int warps, int sms) {
     const long long slots = 3LL * (sms > 0 ? sms : 148), want = (samples + slots - 1) / slots;
     int g = (int)(want < 1 ? 1 : want > kGroup ? kGroup : want);
-    while (g > 1 && grid_smem_bytes(T, g, warps) > 70u * 1024u) --g;
+    while (g > 1 && grid_smem_bytes(T, g, warps) > kGridSmem) --g;
     return g;
 }
 

@@ -115,7 +115,7 @@ int launch_grid_cycle_t(const SceneView &V, const exact_footprint *fp, cudaStrea
     const size_t smem = grid_smem_bytes(V.P.T, group, kBlock / 32);
     // beyond the default 48 KB with the footprint's slots
     if (smem > 40u * 1024u && cudaFuncSetAttribute(mppi_grid_sample_kernel<MOVING>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)smem) != cudaSuccess)
+                                                   (int)kGridSmemMax) != cudaSuccess)
         return EXACT_ECUDA;
     const FpTable t = make_table(fp);
     if (launch_dependent(mppi_grid_sample_kernel<MOVING>, (V.P.K + group - 1) / group, kBlock, smem, st, V, t, grid,
