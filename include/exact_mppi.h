@@ -366,13 +366,14 @@ void exact_batch_destroy(exact_batch *batch);
  * graph).  Calls on one batch must not overlap on the GPU. */
 int mppi_step_batched(exact_batch *batch, void *stream);
 
-/* Tile autotuner: times the batch's sample phase (which writes only batch
- * scratch, never the scenes' U or outputs) for each candidate tile shape
- * (threads per block x point pairs per lane; the scenes without a d_min
- * output, which walk a cell grid, only use the threads), `iters` runs
- * each, keeps the fastest for later steps and, when json_out is non-NULL,
- * writes the timings as JSON text (at most json_cap bytes, NUL-terminated).
- * Synchronises `stream`. */
+/* Tile autotuner: times the batch's sample phase as a step runs it, but
+ * writing only scratch (a d_min goes to memory that the call allocates and
+ * frees), never the scenes' U or outputs, for each candidate block size, each
+ * `iters` runs; keeps the fastest for later steps and, when json_out is
+ * non-NULL, writes the timings as JSON text (at most json_cap bytes,
+ * NUL-terminated).  The other half of a tile shape, point pairs per lane, is
+ * only varied for a batch with a scene that uses it (clouds pruned without a
+ * cell grid); otherwise each block size is timed twice.  Synchronises `stream`. */
 int exact_batch_autotune(exact_batch *batch, int iters, char *json_out, int json_cap, void *stream);
 /* The batch's device error word (as exact_ctx_get_error: first error of
  * any of its kernels, read and cleared in the order of `stream`, which is

@@ -126,6 +126,12 @@ batched_validate_kernel(const SceneDev *__restrict__ scenes, const int2 *__restr
     validate_body(V, ev, t.y / V.val_chunks, t.y % V.val_chunks, sm, grid);
 }
 
+// The tuning views write their d_min to buf instead of the scenes' outputs.
+// They share it: nothing reads it.
+__global__ void tune_dmin_kernel(SceneDev *tune, const SceneDev *scenes, int n, float *buf) {
+    for (int s = threadIdx.x; s < n; s += blockDim.x) tune[s].V.dmin = scenes[s].V.dmin ? buf : nullptr;
+}
+
 int check_params(const exact_mppi_params *p);
 MppiP to_device_params(const exact_mppi_params *p);
 
@@ -168,6 +174,8 @@ extern "C" int exact_batch_create(int n_scenes, const exact_scene *scenes, exact
     std::vector<size_t> scratch_off(n_scenes);
     size_t scratch_total = 0;
     int max_stage = 0;
+    size_t dmin_len = 0;
+    bool pairs_matter = false;
     for (int s = 0; s < n_scenes; ++s) {
         const exact_scene &S = scenes[s];
         int rc = check_params(&S.params);
@@ -182,6 +190,8 @@ extern "C" int exact_batch_create(int n_scenes, const exact_scene *scenes, exact
             scratch_total += grid_copy_bytes(S.n_points, false);
         else
             max_stage = std::max(max_stage, std::min(S.n_points, kStage));
+        if (S.dmin) dmin_len = std::max(dmin_len, (size_t)S.params.K * S.params.T);
+        pairs_matter |= !S.dmin && !uses_grid(S);
     }
     std::vector<int> sort_list;
     for (int s = 0; s < n_scenes; ++s)
@@ -256,6 +266,8 @@ extern "C" int exact_batch_create(int n_scenes, const exact_scene *scenes, exact
     b->n_gitems = (int)gitems.size();
     b->grid_group = group;
     b->grid_T = grid_T;
+    b->dmin_len = dmin_len;
+    b->pairs_matter = pairs_matter;
     b->n_upd = (int)upd.size();
     b->n_val = (int)val.size();
     b->smem = kFpSlots * sizeof(float4) + (size_t)max_stage * sizeof(float2);
@@ -298,11 +310,9 @@ extern "C" int exact_batch_create(int n_scenes, const exact_scene *scenes, exact
         const exact_footprint *fp = S.fp;
         D.fp = make_table(fp);
     }
-    std::vector<SceneDev> tune = host;
-    for (auto &D : tune) D.V.dmin = nullptr;
     int rc = EXACT_OK;
     if (cudaMemcpy(b->d_scenes, host.data(), sizeof(SceneDev) * n_scenes, cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(b->d_tune, tune.data(), sizeof(SceneDev) * n_scenes, cudaMemcpyHostToDevice) != cudaSuccess ||
+        cudaMemcpy(b->d_tune, host.data(), sizeof(SceneDev) * n_scenes, cudaMemcpyHostToDevice) != cudaSuccess ||
         (b->n_items &&
          cudaMemcpy(b->d_items, items.data(), items.size() * sizeof(int2), cudaMemcpyHostToDevice) != cudaSuccess) ||
         (b->n_gitems && cudaMemcpy(b->d_gitems, gitems.data(), gitems.size() * sizeof(int2), cudaMemcpyHostToDevice) !=
@@ -415,33 +425,41 @@ extern "C" int exact_batch_autotune(exact_batch *b, int iters, char *json_out, i
     cudaStream_t st = (cudaStream_t)stream;
     static const int kThreads[] = {128, 256, 512};
     static const int kPairs[] = {1, 2, 4, 8};
+    const int now[] = {b->pairs, b->pairs};
+    // point pairs per lane only shape the sub-chunks of a cloud pruned without
+    // a grid; elsewhere each block size is timed twice instead
+    const int *pairs = b->pairs_matter ? kPairs : now;
+    const int n_pairs = b->pairs_matter ? 4 : 2;
+    float *dmin = nullptr;
     cudaEvent_t e0, e1;
-    if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) return EXACT_ECUDA;
+    if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess ||
+        (b->dmin_len && cudaMalloc(&dmin, b->dmin_len * sizeof(float)) != cudaSuccess))
+        return EXACT_ECUDA;
+    tune_dmin_kernel<<<1, 256, 0, st>>>(b->d_tune, b->d_scenes, b->n, dmin);
     float best_ms = 3.0e38f;
     int best_t = b->threads, best_p = b->pairs;
     std::string json = "{\"candidates\": [";
     bool first = true;
-    int rc = EXACT_OK;
-    for (int t : kThreads) {
-        for (int pl : kPairs) {
-            if (exact_batch_set_tiles(b, t, pl) != EXACT_OK) continue;
-            if ((rc = launch_sample(b, b->d_tune, st)) != EXACT_OK) break;   // warm-up
-            cudaEventRecord(e0, st);
-            for (int i = 0; i < iters && rc == EXACT_OK; ++i) rc = launch_sample(b, b->d_tune, st);
-            cudaEventRecord(e1, st);
-            if (rc != EXACT_OK || cudaEventSynchronize(e1) != cudaSuccess) { rc = EXACT_ECUDA; break; }
-            float ms = 0.f;
-            cudaEventElapsedTime(&ms, e0, e1);
-            ms /= iters;
-            char buf[128];
-            snprintf(buf, sizeof(buf), "%s{\"threads\": %d, \"pairs_per_lane\": %d, \"ms\": %.6f}", first ? "" : ", ", t,
-                     pl, ms);
-            json += buf;
-            first = false;
-            if (ms < best_ms) { best_ms = ms; best_t = t; best_p = pl; }
-        }
-        if (rc != EXACT_OK) break;
+    int rc = cuda_status(cudaGetLastError());
+    for (int c = 0; c < 3 * n_pairs && rc == EXACT_OK; ++c) {
+        const int t = kThreads[c % 3], pl = pairs[c / 3];
+        if (exact_batch_set_tiles(b, t, pl) != EXACT_OK) continue;
+        if ((rc = launch_sample(b, b->d_tune, st)) != EXACT_OK) break;   // warm-up
+        cudaEventRecord(e0, st);
+        for (int i = 0; i < iters && rc == EXACT_OK; ++i) rc = launch_sample(b, b->d_tune, st);
+        cudaEventRecord(e1, st);
+        if (rc != EXACT_OK || cudaEventSynchronize(e1) != cudaSuccess) { rc = EXACT_ECUDA; break; }
+        float ms = 0.f;
+        cudaEventElapsedTime(&ms, e0, e1);
+        ms /= iters;
+        char buf[128];
+        snprintf(buf, sizeof(buf), "%s{\"threads\": %d, \"pairs_per_lane\": %d, \"ms\": %.6f}", first ? "" : ", ", t, pl, ms);
+        json += buf;
+        first = false;
+        if (ms < best_ms) { best_ms = ms; best_t = t; best_p = pl; }
     }
+    cudaStreamSynchronize(st);
+    if (dmin) cudaFree(dmin);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     const int src = exact_batch_set_tiles(b, best_t, best_p);

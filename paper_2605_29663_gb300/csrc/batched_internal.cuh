@@ -44,10 +44,12 @@ struct exact_batch {
     int n = 0;
     void *dev = nullptr;
     exact::SceneDev *d_scenes = nullptr;      // for steps
-    exact::SceneDev *d_tune = nullptr;        // same, without the dmin outputs (autotuning)
+    exact::SceneDev *d_tune = nullptr;        // same, with another d_min output (autotuning)
     int2 *d_items = nullptr, *d_gitems = nullptr, *d_upd = nullptr, *d_val = nullptr;
     int n_items = 0, n_gitems = 0, n_upd = 0, n_val = 0;
     int grid_group = 1, grid_T = 1;      // samples per grid item, longest horizon of a grid scene
+    size_t dmin_len = 0;                 // most d_min values of a scene that outputs them
+    bool pairs_matter = false;           // some scene is pruned without a grid
     char *d_ctrl = nullptr;            // n headers (kHdrStride apart) + queue head
     size_t ctrl_bytes = 0;
     unsigned *d_queue = nullptr;       // queue heads: items, grid items

@@ -60,3 +60,36 @@ def test_an_older_plan_steps_after_a_newer_smaller_one(ex, dmin, shared, tune):
         b.step()
     a.step()
     _check(ex, old, dev, a, dmin)
+
+
+@pytest.mark.parametrize("shared", [False, True])
+def test_autotune_times_what_a_step_runs(ex, shared):
+    """A d_min output switches every pruning off: the tuner must time that, not
+    the pruned cycle.  Points a metre and more beyond d_safe, so that pruned the
+    sample phase would do next to nothing: its times are those of the step, of
+    which it is all but a few us (a third is left for noise).  The scenes' d_min
+    is not written, and block sizes are all that varies."""
+    import torch
+    scenes = _scenes([(1500, 20, 6000)] * 6, shared, 8)
+    g = synth.rng(2)
+    for s in scenes:
+        a = g.uniform(-np.pi, np.pi, 6000)
+        s["cloud"], s["mask"] = (np.stack([np.cos(a), np.sin(a)], 1) * g.uniform(8, 12, (6000, 1))).astype(np.float32), None
+        s["q0"], s["U"] = np.zeros(3, np.float32), s["U"] * 0
+    b = ex.Batch([_dev_scene(ex, s) for s in scenes], dmin=True)
+    for o in b.outputs:
+        o["dmin"].fill_(-7.0)
+    report = b.autotune(iters=3)
+    assert all(bool((o["dmin"] == -7.0).all()) for o in b.outputs)
+    assert {c["threads"] for c in report["candidates"]} == {128, 256, 512}
+    assert len({c["pairs_per_lane"] for c in report["candidates"]}) == 1
+    b.step()
+    e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+    e[0].record()
+    for _ in range(5):
+        b.step()
+    e[1].record()
+    torch.cuda.synchronize()
+    step = e[0].elapsed_time(e[1]) / 5
+    assert report["best"]["ms"] > step / 3, (report["best"], step)
+    assert all(bool((o["dmin"] > 0).all()) for o in b.outputs)
