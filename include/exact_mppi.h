@@ -38,9 +38,10 @@ typedef enum {
     EXACT_ENOTSIMPLE = 2,   /* polygon is not simple (self-intersection, repeated vertex, zero area) */
     EXACT_ECAPACITY = 3,    /* size beyond a documented maximum */
     EXACT_ECUDA = 4,        /* a CUDA runtime call failed */
-    EXACT_ETIMEOUT = 5      /* a bounded device-side wait gave up: the bulk copy that stages a
-                               block's obstacle points did not complete (no kernel of this library
-                               waits on another block; phases end with atomic tickets) */
+    EXACT_ETIMEOUT = 5      /* a bounded device-side wait gave up, on the bulk copy that stages a
+                               block's obstacle points or on the warps that share out the rows of
+                               a many-pose exact_sdf_batch (only the blocks of a cluster wait for
+                               one another, at a barrier; phases end with atomic tickets) */
 } exact_status;
 
 typedef enum { EXACT_FP_POLYGON = 0, EXACT_FP_RECTS = 1 } exact_fp_kind;
@@ -114,7 +115,8 @@ int exact_ctx_reserve_cloud(exact_ctx *ctx, int max_poses, int max_K, int max_T,
  *                   exact_sdf_batch (the call still runs; its results are
  *                   not meaningful);
  *   EXACT_ETIMEOUT  a staging copy that did not complete within its bounded
- *                   wait;
+ *                   wait, or a row of distances whose warps did not (it and
+ *                   the block's later rows are then not written);
  *   EXACT_ECAPACITY an index out of range, in the debug build only
  *                   (compiled with -DEXACT_DEBUG_CHECKS: every checked access
  *                   is skipped instead of made).

@@ -218,11 +218,15 @@ sdf_matrix_kernel(const SortedChunk *__restrict__ chunks, int N, int csize, int 
             mbar_init(empty + k, 1);
             red[k][nwarps] = kNoKey;
         }
-    auto wait = [&](unsigned long long *bar, unsigned parity) {   // bounded, as every wait here
-        if (!mbar_wait(bar, parity)) {
-            report_error(err, EXACT_ETIMEOUT);
-            mbar_wait(bar, parity);
-        }
+    // bounded, as every wait here, and the same for the whole warp: false (and
+    // an error recorded) when the phase has not come, upon which the warp leaves
+    // the kernel and stores nothing more; the others' waits then end the same
+    // way.  Two limits in a row: the first may have passed while the GPU ran
+    // another program.
+    auto wait = [&](unsigned long long *bar, unsigned parity) {
+        const bool ok = __any_sync(0xffffffffu, mbar_wait(bar, parity)) || __any_sync(0xffffffffu, mbar_wait(bar, parity));
+        if (!ok) report_error(err, EXACT_ETIMEOUT);
+        return ok;
     };
     auto arrive = [&](unsigned long long *bar) {
         asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
@@ -267,7 +271,10 @@ sdf_matrix_kernel(const SortedChunk *__restrict__ chunks, int N, int csize, int 
                 if (chunk == 0 && lane == 0 && !(isfinite(poses[3 * (size_t)pose]) && isfinite(poses[3 * (size_t)pose + 1]) &&
                                                  isfinite(poses[3 * (size_t)pose + 2])))
                     report_error(err, EXACT_EINVAL);
-                wait(full + k, (i / kRows) & 1);
+                if (!wait(full + k, (i / kRows) & 1)) {
+                    if (bulk && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // its copies in flight
+                    return;
+                }
                 const float *row = rows + k * kChunk;
                 float *out = dist + (size_t)pose * N + base;
                 if (bulk && lane == 0)
@@ -306,7 +313,7 @@ sdf_matrix_kernel(const SortedChunk *__restrict__ chunks, int N, int csize, int 
             sincosf(th, &sn, &cs);
             const float size0 = fabsf(tx) + fabsf(ty) + span;
             float *row = rows + k * kChunk;
-            if (i >= kRows) wait(empty + k, ((i / kRows) & 1) ^ 1);   // the last row in this buffer has left it
+            if (i >= kRows && !wait(empty + k, ((i / kRows) & 1) ^ 1)) return;   // until the last row in this buffer has left it
             float bk = finf();
             int bi = -1;
             for (; q < npatch; q += nwarps) {
