@@ -98,7 +98,11 @@ void exact_ctx_destroy(exact_ctx *ctx);
 /* Make sure scratch for sdf batches of up to max_poses poses and MPPI steps
  * of up to max_K samples and max_T steps exists (synchronous).  Scratch that a
  * larger call outgrows stays allocated until the context is destroyed (together
- * at most the size of the current one), so captured graphs stay valid. */
+ * at most the size of the current one), so captured graphs stay valid; except
+ * that a call whose scratch does not fit into device memory beside it waits
+ * for the device and gives it back: graphs captured before such a call must
+ * not be replayed again.  (A context reserved for its largest call never gets
+ * there.) */
 int exact_ctx_reserve(exact_ctx *ctx, int max_poses, int max_K, int max_T);
 /* The same, also for clouds of up to max_points points: an MPPI step without
  * a d_min output sorts clouds of 1,024 points or more into a cell grid kept in

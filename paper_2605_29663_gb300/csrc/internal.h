@@ -26,7 +26,7 @@ struct exact_footprint {
     float bhx, bhy;         // half extents of the bounding box about (bcx, bcy), rounded up
 };
 
-namespace exact { constexpr int kRetired = 128; }   // two arenas, doubled from 1 MB on: at most 40 steps each
+namespace exact { constexpr int kRetired = 128; }   // two arenas, doubled from 1 MB on while there is memory: at most 40 steps each
 
 // Minimum of one pose of a split exact_sdf_batch (complemented packed key; 0
 // = empty) and its finished blocks; each call clears its own first.

@@ -204,21 +204,28 @@ static void free_retired(exact_ctx *ctx) {
     while (ctx->n_retired > 0) cudaFree(ctx->retired[--ctx->n_retired]);
 }
 static void retire(exact_ctx *ctx, void *p) {
-    if (p && ctx->n_retired < kRetired) ctx->retired[ctx->n_retired++] = p;   // doubling never gets there
+    if (p) ctx->retired[ctx->n_retired++] = p;   // growth looks for room first
 }
 
 // Outgrown arenas stay allocated until the context goes: a captured graph may
 // still replay with their addresses, whichever later call grew the scratch.
-// Doubling keeps them below the current arena's size in sum; they are given
-// back early only where the new arena would not fit otherwise.
+// Doubling keeps them below the current arena's size in sum.  Where there is no
+// memory for twice the size, the size asked for is tried; only where that does
+// not fit beside them are they given back (before that the call would have
+// been refused).
 int ensure_scratch(exact_ctx *ctx, size_t bytes) {
     if (!ctx) return EXACT_EINVAL;
     if (bytes <= ctx->scratch_bytes) return EXACT_OK;
     bytes = align_up(bytes, (size_t)1 << 20);
-    size_t got = std::max(bytes, 2 * ctx->scratch_bytes);
+    const size_t twice = std::max(bytes, 2 * ctx->scratch_bytes);
+    size_t got = 0;
     void *p = nullptr;
-    if (cudaMalloc(&p, got) != cudaSuccess) {
-        cudaGetLastError();
+    for (size_t want : {twice, bytes})
+        if (!p && ctx->n_retired < kRetired) {
+            if (cudaMalloc(&p, want) == cudaSuccess) got = want;
+            else { cudaGetLastError(); p = nullptr; }
+        }
+    if (!p) {
         if (cudaDeviceSynchronize() != cudaSuccess) return EXACT_ECUDA;
         if (ctx->scratch) cudaFree(ctx->scratch);
         free_retired(ctx);
@@ -244,14 +251,16 @@ bool try_work(exact_ctx *ctx, size_t bytes, cudaStream_t st) {
     if (bytes <= ctx->work_bytes) return true;
     if (bytes > ((size_t)1 << 30)) return false;
     bytes = align_up(bytes, (size_t)1 << 20);
-    const size_t got = std::max(bytes, 2 * ctx->work_bytes);
+    size_t got = std::max(bytes, 2 * ctx->work_bytes);
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     void *p = nullptr;
     if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone ||
-        cudaMalloc(&p, got) != cudaSuccess) {
+        ctx->n_retired >= kRetired ||
+        (cudaMalloc(&p, got) != cudaSuccess && cudaMalloc(&p, got = bytes) != cudaSuccess)) {
         cudaGetLastError();   // not this call's error: it has another path
         return false;
     }
+    cudaGetLastError();
     retire(ctx, ctx->work_alloc);
     ctx->work = ctx->work_alloc = p;
     ctx->work_bytes = got;
