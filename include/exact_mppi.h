@@ -95,8 +95,8 @@ int exact_footprint_info(const exact_footprint *fp, int *kind, int *n);
 typedef struct exact_ctx exact_ctx;
 int exact_ctx_create(exact_ctx **out);
 void exact_ctx_destroy(exact_ctx *ctx);
-/* Make sure scratch for sdf batches of up to max_poses poses and MPPI steps
- * of up to max_K samples and max_T steps exists (synchronous).  Scratch that a
+/* Make sure scratch for MPPI steps of up to max_K samples and max_T steps
+ * exists (synchronous; sdf batches need none without max_points, below).  Scratch that a
  * larger call outgrows stays allocated until the context is destroyed (together
  * at most the size of the current one), so captured graphs stay valid; except
  * that a call whose scratch does not fit into device memory beside it waits
@@ -108,9 +108,11 @@ int exact_ctx_reserve(exact_ctx *ctx, int max_poses, int max_K, int max_T);
  * a d_min output sorts clouds of 1,024 points or more into a cell grid kept in
  * the context (so that each sample looks only at the points near its
  * footprint, whatever the input order), so a step with a larger cloud than any
- * before may allocate -- reserve ahead of stream capture.  (exact_sdf_batch of
+ * before may allocate -- reserve ahead of stream capture.  exact_sdf_batch of
  * many poses takes the memory of a spatially sorted copy of the points from a
- * pool of the context, stream-ordered, and its general path in a capture.) */
+ * pool that the contexts of a device share while they live, stream-ordered, and
+ * its general path in a capture: with max_poses and max_points the pool gets
+ * that memory here and keeps it, instead of in the first such call. */
 int exact_ctx_reserve_cloud(exact_ctx *ctx, int max_poses, int max_K, int max_T, int max_points);
 /* Device-side error word of the context (an exact_status, 0 = none): the
  * first error a kernel launched with this context recorded.  Kernels record

@@ -277,9 +277,9 @@ class Context:
         return self._h
 
     def reserve(self, max_poses: int = 0, max_K: int = 0, max_T: int = 0, max_points: int = 0):
-        """Allocate scratch ahead of time (before a CUDA graph capture): SDF
-        batches of max_poses poses, MPPI steps of max_K x max_T, clouds of
-        max_points points (their cell grid)."""
+        """Allocate scratch ahead of time (before a CUDA graph capture): MPPI
+        steps of max_K x max_T, clouds of max_points points (their cell grid),
+        SDF batches of max_poses poses against them (their sorted copy)."""
         _check(load().exact_ctx_reserve_cloud(self._h, max_poses, max_K, max_T, max_points),
                "exact_ctx_reserve_cloud")
 

@@ -38,14 +38,17 @@ struct SdfKey {
 struct exact_ctx {
     int device = 0;
     int sm_count = 0;
-    void *scratch = nullptr;     // growable device arena
+    // growable device arena; scratch_alloc (and work_alloc below): null while it
+    // is a piece of the first allocation, at sdf_keys
+    void *scratch = nullptr, *scratch_alloc = nullptr;
     size_t scratch_bytes = 0;
     // a second arena, for the cell grids, which each call writes before it reads:
     // apart from the first, whose counters outlive a call
-    void *work = nullptr, *work_alloc = nullptr;   // work_alloc: null while it is the piece behind sdf_keys
+    void *work = nullptr, *work_alloc = nullptr;
     size_t work_bytes = 0;
-    // exact_sdf_batch of many poses takes its sorted cloud from here, stream
-    // ordered: such calls may overlap on several streams (sdf_pool makes it)
+    // exact_sdf_batch of many poses takes its sorted cloud from the device's
+    // pool, stream ordered: such calls may overlap on several streams.  Null
+    // until the context first uses it (sdf_pool)
     std::atomic<cudaMemPool_t> pool{nullptr};
     void *retired[exact::kRetired];   // outgrown arenas
     int n_retired = 0;
@@ -67,16 +70,19 @@ int ensure_scratch(exact_ctx *ctx, size_t bytes);
 // Whether the second arena holds `bytes`, or can be grown to them now (not
 // while the stream captures, and to 1 GB at most).
 bool try_work(exact_ctx *ctx, size_t bytes, cudaStream_t st);
-// The context's memory pool, made by the first call; NULL: there is none to be had.
-cudaMemPool_t sdf_pool(exact_ctx *ctx);
+// The memory pool of the context's device; NULL: there is none to be had.  It
+// keeps up to `keep` bytes over a synchronisation (the largest asked for).
+constexpr unsigned long long kPoolKeep = 64ull << 20;   // the sorted copy of 6 million points
+cudaMemPool_t sdf_pool(exact_ctx *ctx, unsigned long long keep = kPoolKeep);
 int current_sm_count();
 // exact_sdf_batch splits a pose's points over several blocks below this many
 // poses (about eight blocks per SM).
 inline int sdf_split_poses(int sms) { return (sms > 0 ? sms : 148) * 8; }
 // A cycle splits its samples' horizons below this many samples (parts_for).
 inline int ticket_count(int sms) { return sms > 0 ? sms : 148; }
-// Arena bytes needed by exact_sdf_batch (n_poses) and mppi_step (K, T).
-size_t sdf_scratch_bytes(int n_poses);
+// The memory of exact_sdf_batch for clouds and pose counts of up to these
+// sizes, in the context's pool ahead of the first call.
+int sdf_reserve(exact_ctx *ctx, int max_points, int max_poses);
 
 inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 

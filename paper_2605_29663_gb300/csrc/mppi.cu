@@ -129,13 +129,14 @@ extern "C" int exact_ctx_reserve(exact_ctx *ctx, int max_poses, int max_K, int m
 
 extern "C" int exact_ctx_reserve_cloud(exact_ctx *ctx, int max_poses, int max_K, int max_T, int max_points) {
     if (!ctx || max_poses < 0 || max_K < 0 || max_T < 0 || max_points < 0) return EXACT_EINVAL;
-    const int rc = ensure_scratch(ctx, std::max(sdf_scratch_bytes(max_poses),
-                                                kArenaHeader + scene_scratch_bytes(max_K, max_T, parts_of(ctx, max_K, max_T))));
-    if (rc != EXACT_OK) return rc;
-    if (max_points < kPruneMin) return EXACT_OK;
-    const size_t work = std::max(grid_copy_bytes(std::min(max_points, kGridMaxPoints), true),   // static or predicted
-                                 std::min(step_grid_bytes(max_points, max_T), kStepGridBytes));
-    return try_work(ctx, work, nullptr) ? EXACT_OK : EXACT_ECUDA;
+    int rc = ensure_scratch(ctx, kArenaHeader + scene_scratch_bytes(max_K, max_T, parts_of(ctx, max_K, max_T)));
+    if (rc == EXACT_OK && max_points >= kPruneMin) {
+        const size_t work = std::max(grid_copy_bytes(std::min(max_points, kGridMaxPoints), true),   // static or predicted
+                                     std::min(step_grid_bytes(max_points, max_T), kStepGridBytes));
+        rc = try_work(ctx, work, nullptr) ? EXACT_OK : EXACT_ECUDA;
+    }
+    if (rc == EXACT_OK) rc = sdf_reserve(ctx, max_points, max_poses);
+    return rc;
 }
 
 namespace exact {

@@ -5,6 +5,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <mutex>
 #include <new>
 
 #include "internal.h"
@@ -227,9 +228,9 @@ int ensure_scratch(exact_ctx *ctx, size_t bytes) {
         }
     if (!p) {
         if (cudaDeviceSynchronize() != cudaSuccess) return EXACT_ECUDA;
-        if (ctx->scratch) cudaFree(ctx->scratch);
+        if (ctx->scratch_alloc) cudaFree(ctx->scratch_alloc);
         free_retired(ctx);
-        ctx->scratch = nullptr;
+        ctx->scratch = ctx->scratch_alloc = nullptr;
         ctx->scratch_bytes = 0;
         got = bytes;
         if (cudaMalloc(&p, got) != cudaSuccess) return EXACT_ECUDA;
@@ -241,8 +242,8 @@ int ensure_scratch(exact_ctx *ctx, size_t bytes) {
         cudaFree(p);
         return EXACT_ECUDA;
     }
-    retire(ctx, ctx->scratch);
-    ctx->scratch = p;
+    retire(ctx, ctx->scratch_alloc);
+    ctx->scratch = ctx->scratch_alloc = p;
     ctx->scratch_bytes = got;
     return EXACT_OK;
 }
@@ -267,23 +268,56 @@ bool try_work(exact_ctx *ctx, size_t bytes, cudaStream_t st) {
     return true;
 }
 
-cudaMemPool_t sdf_pool(exact_ctx *ctx) {
+// One pool per device, shared by the contexts that use it and destroyed with
+// the last of them: making a pool and mapping its first memory takes some 130
+// us, which a second context need not pay again.
+constexpr int kMaxDevices = 64;
+static struct SharedPool {
+    std::mutex lock;
+    cudaMemPool_t pool = nullptr;
+    int users = 0;
+} g_pools[kMaxDevices];
+
+cudaMemPool_t sdf_pool(exact_ctx *ctx, unsigned long long keep) {
     cudaMemPool_t pool = ctx->pool.load();
-    if (pool) return pool;
-    cudaMemPoolProps props = {};
-    props.allocType = cudaMemAllocationTypePinned;
-    props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = ctx->device;
-    unsigned long long keep = 64ull << 20;   // kept over a synchronisation: the sorted copy of 6 million points
-    if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
+    if (pool && keep <= kPoolKeep) return pool;
+    if (ctx->device < 0 || ctx->device >= kMaxDevices) return nullptr;
+    SharedPool &shared = g_pools[ctx->device];
+    std::lock_guard<std::mutex> guard(shared.lock);
+    if (!shared.pool) {
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = ctx->device;
+        if (cudaMemPoolCreate(&shared.pool, &props) != cudaSuccess) {
+            cudaGetLastError();
+            shared.pool = nullptr;
+            return nullptr;
+        }
+        unsigned long long least = kPoolKeep;
+        int no = 0;   // a stream does not wait for another's call to end to take its memory
+        cudaMemPoolSetAttribute(shared.pool, cudaMemPoolAttrReleaseThreshold, &least);
+        cudaMemPoolSetAttribute(shared.pool, cudaMemPoolReuseAllowInternalDependencies, &no);
     }
-    cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
-    cudaMemPool_t other = nullptr;
-    if (ctx->pool.compare_exchange_strong(other, pool)) return pool;
-    cudaMemPoolDestroy(pool);   // another thread was first
-    return other;
+    pool = shared.pool;
+    if (!ctx->pool.load()) {
+        ++shared.users;
+        ctx->pool = pool;
+    }
+    unsigned long long now = 0;
+    if (cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &now) == cudaSuccess && now < keep)
+        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    return pool;
+}
+
+static void release_pool(exact_ctx *ctx) {
+    if (!ctx->pool.load()) return;
+    SharedPool &shared = g_pools[ctx->device];
+    std::lock_guard<std::mutex> guard(shared.lock);
+    if (--shared.users == 0) {
+        cudaMemPoolDestroy(shared.pool);
+        shared.pool = nullptr;
+    }
 }
 
 }  // namespace exact
@@ -295,19 +329,21 @@ extern "C" int exact_ctx_create(exact_ctx **out) {
     if (!ctx) return EXACT_EINVAL;
     if (cudaGetDevice(&ctx->device) != cudaSuccess) { delete ctx; return EXACT_ECUDA; }
     ctx->sm_count = exact::current_sm_count();
-    // one allocation: split keys, error word, statistics, part tickets (zeroed), then the
-    // second arena's first 1 MB, so that a cycle on a cloud of ordinary size can
-    // be captured without any call before it
+    // one allocation: split keys, error word, statistics, part tickets, the
+    // arena's first 1 MB (all zeroed), then the second arena's, so that a cycle of
+    // ordinary size can be captured without any call before it
     const size_t key_bytes = exact::align_up(sizeof(SdfKey) * (size_t)exact::sdf_split_poses(ctx->sm_count), 256);
     const size_t stats_bytes = exact::align_up(sizeof(exact_cycle_stats), 256);
-    const size_t head = key_bytes + 256 + stats_bytes +
-                        exact::align_up(sizeof(unsigned) * (size_t)exact::ticket_count(ctx->sm_count), 256);
-    ctx->work_bytes = (size_t)1 << 20;
+    const size_t first = key_bytes + 256 + stats_bytes +
+                         exact::align_up(sizeof(unsigned) * (size_t)exact::ticket_count(ctx->sm_count), 256);
+    ctx->scratch_bytes = ctx->work_bytes = (size_t)1 << 20;
+    const size_t head = first + ctx->scratch_bytes;
     if (cudaMalloc(&ctx->sdf_keys, head + ctx->work_bytes) != cudaSuccess) { delete ctx; return EXACT_ECUDA; }
     char *base = reinterpret_cast<char *>(ctx->sdf_keys);
     ctx->d_err = reinterpret_cast<int *>(base + key_bytes);
     ctx->d_stats = reinterpret_cast<decltype(ctx->d_stats)>(base + key_bytes + 256);
     ctx->part_tickets = reinterpret_cast<unsigned *>(base + key_bytes + 256 + stats_bytes);
+    ctx->scratch = base + first;
     ctx->work = base + head;
     if (cudaMemset(base, 0, head) != cudaSuccess || cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) {   // as in ensure_scratch
         cudaFree(base);
@@ -321,9 +357,9 @@ extern "C" int exact_ctx_create(exact_ctx **out) {
 extern "C" void exact_ctx_destroy(exact_ctx *ctx) {
     if (!ctx) return;
     cudaDeviceSynchronize();
-    if (ctx->scratch) cudaFree(ctx->scratch);
+    if (ctx->scratch_alloc) cudaFree(ctx->scratch_alloc);
     if (ctx->work_alloc) cudaFree(ctx->work_alloc);
-    if (cudaMemPool_t pool = ctx->pool.load()) cudaMemPoolDestroy(pool);
+    exact::release_pool(ctx);
     exact::free_retired(ctx);
     if (ctx->sdf_keys) cudaFree(ctx->sdf_keys);
     delete ctx;

@@ -273,7 +273,22 @@ __global__ void sdf_keys_finish(const unsigned long long *__restrict__ keys, int
     if (argmin) argmin[p] = b == kNoKey ? -1 : (int)(unsigned)(b & 0xffffffffu);
 }
 
-size_t sdf_scratch_bytes(int n_poses) { return kArenaHeader + align_up((size_t)n_poses * sizeof(unsigned long long), 256); }
+// Stream-ordered memory of a pruned call: per-pose keys where chunks meet, the
+// sorted chunks.
+static size_t sdf_key_bytes(int n_poses) { return align_up((size_t)n_poses * sizeof(unsigned long long), 256); }
+constexpr size_t kSdfNearBytes = (size_t)1 << 30;   // the most a call takes
+
+int sdf_reserve(exact_ctx *ctx, int max_points, int max_poses) {
+    const size_t bytes = sdf_key_bytes(max_poses) + sdf_near_bytes(max_points);
+    if (!sdf_near_possible(max_points, max_poses) || bytes > kSdfNearBytes) return EXACT_OK;   // the general kernel needs none
+    void *mem = nullptr;
+    const cudaMemPool_t pool = sdf_pool(ctx, bytes > kPoolKeep ? bytes : kPoolKeep);
+    if (!pool || cudaMallocFromPoolAsync(&mem, bytes, pool, nullptr) != cudaSuccess) {
+        cudaGetLastError();
+        return EXACT_OK;   // as a call would: without it
+    }
+    return cuda_status(cudaFreeAsync(mem, nullptr)) == EXACT_OK ? cuda_status(cudaStreamSynchronize(cudaStreamLegacy)) : EXACT_ECUDA;
+}
 
 }  // namespace exact
 
@@ -297,11 +312,11 @@ extern "C" int exact_sdf_batch(exact_ctx *ctx, const float *points, const uint8_
     // a capture, whose replays may overlap anything
     if (ctx && (dist || dmin || argmin) && sdf_near_fits(fp, n_points, n_poses, dist != nullptr)) {
         const bool split = dist && (dmin || argmin) && n_points > kSdfChunk;
-        const size_t key_bytes = split ? align_up((size_t)n_poses * sizeof(unsigned long long), 256) : 0;
+        const size_t key_bytes = split ? sdf_key_bytes(n_poses) : 0;
         cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
         void *mem = nullptr;
         if (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
-            key_bytes + sdf_near_bytes(n_points) <= ((size_t)1 << 30) && sdf_pool(ctx) &&
+            key_bytes + sdf_near_bytes(n_points) <= kSdfNearBytes && sdf_pool(ctx) &&
             cudaMallocFromPoolAsync(&mem, key_bytes + sdf_near_bytes(n_points), sdf_pool(ctx), st) == cudaSuccess) {
             unsigned long long *keys = split ? static_cast<unsigned long long *>(mem) : nullptr;
             if (keys) sdf_keys_init<<<(n_poses + 255) / 256, 256, 0, st>>>(keys, n_poses);

@@ -531,11 +531,17 @@ sdf_min_kernel(const SortedChunk *__restrict__ chunks, int N, int csize, const f
 // edges 187 against 249, 64 edges 288 against 568), and patches of a few
 // thousand points are too wide to leave edges out (8,192 x 1,024 points, 32
 // edges: 132 against 92 us).  Minimum: general calls from about 45 us on.
+constexpr int kMinPoses = 256, kMinPoints = 2 * kPatch, kMatrixPoses = 64, kMatrixPoints = 4096;
 bool sdf_near_fits(const exact_footprint *fp, int n_points, int n_poses, bool dist) {
     const long long pairs = (long long)n_points * n_poses;
     const long long work = pairs * (fp->kind == EXACT_FP_POLYGON ? fp->n_pad : 2 * fp->n_pad);
-    if (!dist) return n_poses >= 256 && n_points >= 2 * kPatch && work >= (1ll << 27);
-    return fp->kind == EXACT_FP_POLYGON && fp->n_pad >= 16 && n_points >= 4096 && n_poses >= 64 && work >= (1ll << 28);
+    if (!dist) return n_poses >= kMinPoses && n_points >= kMinPoints && work >= (1ll << 27);
+    return fp->kind == EXACT_FP_POLYGON && fp->n_pad >= 16 && n_points >= kMatrixPoints && n_poses >= kMatrixPoses &&
+           work >= (1ll << 28);
+}
+bool sdf_near_possible(int n_points, int n_poses) {
+    if ((long long)n_points * n_poses < (1ll << 27) / EXACT_MAX_POLY_VERTICES) return false;
+    return (n_poses >= kMinPoses && n_points >= kMinPoints) || (n_poses >= kMatrixPoses && n_points >= kMatrixPoints);
 }
 
 int sdf_near_launch(const float2 *pts, const uint8_t *mask, int N, const float *poses, int P, const exact_footprint *fp,

@@ -7,6 +7,8 @@ namespace exact {
 
 // Whether the pruned path is the faster one for this call.
 bool sdf_near_fits(const exact_footprint *fp, int n_points, int n_poses, bool dist);
+// Whether it can be for any footprint, at these sizes or smaller ones.
+bool sdf_near_possible(int n_points, int n_poses);
 // Device scratch of a call with n_points points.
 size_t sdf_near_bytes(int n_points);
 // keys: initialised per-pose keys for the minimum over several chunks, or NULL

@@ -133,3 +133,61 @@ def test_replays_and_eager_cycles_of_other_sizes_take_turns(ex, a, b, dmin, N):
         A.check(f"replay before eager {k}")
         B.run()
         B.check(f"eager after replay {k}")
+
+
+@pytest.mark.parametrize("dist,P,N", [(False, 3000, 20_000), (True, 1000, 60_000)])
+def test_reserve_holds_what_many_pose_calls_take(ex, dist, P, N):
+    """A context reserved for its poses and points makes and maps its memory
+    then: the first call takes none from the device."""
+    import torch
+    g = synth.rng(P)
+    f = ex.Footprint.polygon(synth.star_polygon(g, 24, 0.3, 1.2))
+    pts, poses = _t(g.uniform(-6, 6, (N, 2))), _t(g.uniform(-3, 3, (P, 3)))
+    out = dict(zip(("dist", "dmin", "argmin"), ex.sdf_batch(pts, poses, f, dist=True, ctx=ex.Context())))
+    want = {k: v.clone() for k, v in out.items()}
+    first = ex.Context()
+    ex.sdf_batch(pts, poses, f, dist=dist, ctx=first, out=out)   # loads the kernels
+    torch.cuda.synchronize()
+    first.close()                                                # and gives its memory back
+    ctx = ex.Context()
+    ctx.reserve(P, 0, 0, N)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    ex.sdf_batch(pts, poses, f, dist=dist, ctx=ctx, out=out)
+    torch.cuda.synchronize()
+    assert torch.cuda.mem_get_info()[0] == free
+    assert all(torch.equal(out[k], want[k]) for k in want)
+
+
+def test_contexts_share_the_pool_and_the_last_gives_it_back(ex):
+    """Two contexts' many-pose calls on two streams, one context going while the
+    other works on; with the last the memory is the device's again."""
+    import gc
+    import torch
+    gc.collect()
+    g = synth.rng(3)
+    f = ex.Footprint.polygon(synth.star_polygon(g, 24, 0.3, 1.2))
+    N = 2_000_000   # 20 MB of sorted chunks per call
+    pts, poses = _t(g.uniform(-6, 6, (N, 2))), _t(g.uniform(-3, 3, (300, 3)))
+    want = ex.sdf_batch(pts, poses, f, dist=False)
+    ex.sdf_batch(pts, poses, f, dist=False, ctx=ex.Context())   # loads the kernels
+    torch.cuda.synchronize()
+    gc.collect()
+    outs = [dict(dmin=torch.empty(300, device="cuda"), argmin=torch.empty(300, dtype=torch.int32, device="cuda")) for _ in range(2)]
+    free = torch.cuda.mem_get_info()[0]
+    ctxs, streams = [ex.Context() for _ in outs], [torch.cuda.Stream() for _ in outs]
+    for turn in range(3):
+        for k in range(2):
+            if ctxs[k]:
+                with torch.cuda.stream(streams[k]):
+                    ex.sdf_batch(pts, poses, f, dist=False, ctx=ctxs[k], out=outs[k])
+        torch.cuda.synchronize()
+        for o in outs:
+            assert torch.equal(o["dmin"], want[1]) and torch.equal(o["argmin"], want[2])
+            o["dmin"].zero_() if turn == 0 else None
+        if turn == 1:
+            ctxs[0].close()
+            ctxs[0] = None
+    assert free - torch.cuda.mem_get_info()[0] >= 20 << 20
+    ctxs[1].close()
+    assert free - torch.cuda.mem_get_info()[0] < 4 << 20   # the contexts' own allocations may stay with the driver
