@@ -210,23 +210,31 @@ sdf_matrix_kernel(const SortedChunk *__restrict__ chunks, int N, int csize, int 
     constexpr int nwarps = kNearThreads / 32 - 1;            // computing warps
     __shared__ unsigned long long red[kRows][nwarps + 1];
     __shared__ unsigned long long full[kRows], empty[kRows];
+    __shared__ int gone;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int E = fp.n;
+    if (tid == 0) gone = 0;
     if (tid == 0)
         for (int k = 0; k < kRows; ++k) {
             mbar_init(full + k, nwarps);
             mbar_init(empty + k, 1);
             red[k][nwarps] = kNoKey;
         }
-    // bounded, as every wait here, and the same for the whole warp: false (and
-    // an error recorded) when the phase has not come, upon which the warp leaves
-    // the kernel and stores nothing more; the others' waits then end the same
-    // way.  Two limits in a row: the first may have passed while the GPU ran
-    // another program.
+    // Bounded, as every wait here: when the phase has not come the error is
+    // recorded and the thread leaves the kernel, its copies in flight completed;
+    // the storing warp then stores no further row, and the others' waits end the
+    // same way.  Two limits in a row: the first may have passed while the GPU ran
+    // another program.  (An exit that the compiler does not see: a return or a
+    // vote here cost registers, and the loop over the patches 5 % on clouds
+    // dense on the footprint.)
+    auto leave = []() { asm volatile("cp.async.bulk.wait_group 0;\n\texit;" ::: "memory"); };
     auto wait = [&](unsigned long long *bar, unsigned parity) {
-        const bool ok = __any_sync(0xffffffffu, mbar_wait(bar, parity)) || __any_sync(0xffffffffu, mbar_wait(bar, parity));
-        if (!ok) report_error(err, EXACT_ETIMEOUT);
-        return ok;
+        if (!mbar_wait(bar, parity) && !mbar_wait(bar, parity)) {
+            report_error(err, EXACT_ETIMEOUT);
+            *(volatile int *)&gone = 1;
+            __threadfence_block();
+            leave();
+        }
     };
     auto arrive = [&](unsigned long long *bar) {
         asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
@@ -271,10 +279,8 @@ sdf_matrix_kernel(const SortedChunk *__restrict__ chunks, int N, int csize, int 
                 if (chunk == 0 && lane == 0 && !(isfinite(poses[3 * (size_t)pose]) && isfinite(poses[3 * (size_t)pose + 1]) &&
                                                  isfinite(poses[3 * (size_t)pose + 2])))
                     report_error(err, EXACT_EINVAL);
-                if (!wait(full + k, (i / kRows) & 1)) {
-                    if (bulk && lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // its copies in flight
-                    return;
-                }
+                wait(full + k, (i / kRows) & 1);
+                if (*(volatile int *)&gone) leave();   // a row may lack the part of a thread that left
                 const float *row = rows + k * kChunk;
                 float *out = dist + (size_t)pose * N + base;
                 if (bulk && lane == 0)
@@ -313,7 +319,7 @@ sdf_matrix_kernel(const SortedChunk *__restrict__ chunks, int N, int csize, int 
             sincosf(th, &sn, &cs);
             const float size0 = fabsf(tx) + fabsf(ty) + span;
             float *row = rows + k * kChunk;
-            if (i >= kRows && !wait(empty + k, ((i / kRows) & 1) ^ 1)) return;   // until the last row in this buffer has left it
+            if (i >= kRows) wait(empty + k, ((i / kRows) & 1) ^ 1);   // the last row in this buffer has left it
             float bk = finf();
             int bi = -1;
             for (; q < npatch; q += nwarps) {
