@@ -38,7 +38,6 @@ constexpr int kGridRegs = 4;          // points per thread kept in registers (cl
 struct GridSmem {
     int cnt[kCells + 1];
     float red[5][kGridThreads / 32];
-    float box[5];
     int part[kGridThreads / 32];
 };
 
@@ -152,8 +151,7 @@ __device__ __forceinline__ void build_grid(const float2 *__restrict__ pts, const
         }
     }
     if (tid == 0) {
-        grid->head = GridHead{lx, ly, inv, cell, fmaxf(fmaxf(fabsf(lx), fabsf(hx)), fmaxf(fabsf(ly), fabsf(hy))),
-                              MOVING ? vm * 1.0001f : 0.f, nx, ny};
+        grid->head = GridHead{lx, ly, inv, cell, MOVING ? vm * 1.0001f : 0.f, 0, nx, ny};
     }
     __syncthreads();
     for (int c = tid; c <= ncell; c += nt) grid->start[c] = sm.cnt[c];

@@ -32,8 +32,7 @@ inline int chunk_points(int N) {
 
 // One sorted chunk: points (invalid ones last, as NaN, which every evaluation
 // turns into +inf), their indices in the chunk, and the patches' circles
-// (centre, radius or -1 for a patch without a valid point, and |x| + |y| + r,
-// the size that scales the rounding slack).
+// (centre, radius or -1 for a patch without a valid point).
 struct __align__(256) SortedChunk {
     float2 pts[kChunk];
     unsigned short idx[kChunk];
@@ -143,7 +142,7 @@ sdf_sort_kernel(const float2 *__restrict__ pts, const uint8_t *__restrict__ mask
         if (b.x == b.x) r2 = fmaxf(r2, fmaf(b.x - cx, b.x - cx, (b.y - cy) * (b.y - cy)));
         r2 = -warp_min_f(-r2);
         const float r = sqrtf(r2) * 1.000001f;
-        if (lane == 0) C.circ[q] = x0 <= x1 ? make_float4(cx, cy, r, fabsf(cx) + fabsf(cy) + r) : make_float4(0.f, 0.f, -1.f, 0.f);
+        if (lane == 0) C.circ[q] = x0 <= x1 ? make_float4(cx, cy, r, 0.f) : make_float4(0.f, 0.f, -1.f, 0.f);
     }
 }
 
@@ -155,9 +154,11 @@ sdf_sort_kernel(const float2 *__restrict__ pts, const uint8_t *__restrict__ mask
 //   |p - b|^2 - |p - a|^2 = |c - b|^2 - |c - a|^2 + 2 (p - c) . (a - b)
 //                        >= d_e(c)^2 - d_f(c)^2 - 2 r |a - b|,
 // so edge e is not needed where d_e(c)^2 > d_f(c)^2 + 2 r max_b |a - b| (b an
-// end of e).  A margin of 1e-5 of the squared coordinates, far above the
-// rounding of the squared distances, keeps every edge whose computed distance
-// could be the minimum: the minimum over the kept edges is the same bits.  One
+// end of e).  A margin of 1e-5 of the squared coordinates in the body frame,
+// far above the rounding of the squared distances (that of o - t is relative to
+// the difference, wherever both lie on the map), keeps every edge whose computed
+// distance could be the minimum: the minimum over the kept edges is the same
+// bits.  One
 // lane per edge, two ballots per patch; far from a 32-gon about 4 edges stay.
 struct EdgeLane {
     float vx, vy, ex, ey, exn, eyn;
@@ -251,7 +252,9 @@ sdf_matrix_kernel(const SortedChunk *__restrict__ chunks, int N, int csize, int 
     const int ne = min(E, n_edges + 1);
     const EdgeLane e0 = edge_lane(s_fp, E, ne, lane), e1 = WIDE ? edge_lane(s_fp, E, ne, 32 + lane) : EdgeLane{};
     const float lim = fmaf(fp.bc.z, 1e-5f, fp.bc.z) + 1e-5f, lim2 = lim * lim;   // as in poly_rows
-    const float span = fabsf(fp.bc.x) + fabsf(fp.bc.y) + fp.bc.z;
+    // 1e-5 (|cx| + |cy| + r + span)^2, span bounding the footprint's coordinates,
+    // is at most 6e-5 of the centre's squared distance + 1.8e-4 span^2 + 3e-5 r^2
+    const float span = fabsf(fp.bc.x) + fabsf(fp.bc.y) + fp.bc.z, k0 = 1.8e-4f * span * span;
     const ulonglong2 *T = reinterpret_cast<const ulonglong2 *>(s_edge);
     const ulonglong2 *S = reinterpret_cast<const ulonglong2 *>(s_fp);
     __syncthreads();
@@ -270,7 +273,12 @@ sdf_matrix_kernel(const SortedChunk *__restrict__ chunks, int N, int csize, int 
             for (int j = tid; j < kChunk / 2; j += kNearThreads) reinterpret_cast<float4 *>(pts)[j] = src[j];
             const uint4 *si = reinterpret_cast<const uint4 *>(C.idx);
             for (int j = tid; j < kChunk / 8; j += kNearThreads) reinterpret_cast<uint4 *>(idx)[j] = si[j];
-            for (int j = tid; j < kPatches; j += kNearThreads) circ[j] = C.circ[j];
+            for (int j = tid; j < kPatches; j += kNearThreads) {
+                float4 c = C.circ[j];
+                const float rz = fmaxf(c.z, 0.f);
+                c.w = fmaf(1e-5f, rz + span, rz);   // the radius, with the slack that does not depend on the pose
+                circ[j] = c;
+            }
         }
         __syncthreads();
         if (warp == nwarps) {   // the storing warp
@@ -317,7 +325,6 @@ sdf_matrix_kernel(const SortedChunk *__restrict__ chunks, int N, int csize, int 
             const float tx = poses[3 * pose], ty = poses[3 * pose + 1], th = poses[3 * pose + 2];
             float sn, cs;
             sincosf(th, &sn, &cs);
-            const float size0 = fabsf(tx) + fabsf(ty) + span;
             float *row = rows + k * kChunk;
             if (i >= kRows) wait(empty + k, ((i / kRows) & 1) ^ 1);   // the last row in this buffer has left it
             float bk = finf();
@@ -326,7 +333,7 @@ sdf_matrix_kernel(const SortedChunk *__restrict__ chunks, int N, int csize, int 
                 const float4 cc = circ[q];
                 float cx, cy;
                 body_frame(cc.x, cc.y, tx, ty, cs, sn, cx, cy);
-                const float size = cc.w + size0, r = fmaf(1e-5f, size, fmaxf(cc.z, 0.f));
+                const float r = fmaf(1e-5f, fabsf(cx) + fabsf(cy), cc.w);
                 // edges that can be nearest
                 const EdgeNear n0 = edge_near(e0, cx, cy), n1 = WIDE ? edge_near(e1, cx, cy) : EdgeNear{finf(), 0.f, 0.f, 0.f, 0.f};
                 const float own = WIDE ? fminf(n0.d2, n1.d2) : n0.d2;
@@ -335,7 +342,7 @@ sdf_matrix_kernel(const SortedChunk *__restrict__ chunks, int N, int csize, int 
                 const bool second = WIDE && n0.d2 != best;
                 const float ax = __shfl_sync(0xffffffffu, second ? n1.qx : n0.qx, who & 31);
                 const float ay = __shfl_sync(0xffffffffu, second ? n1.qy : n0.qy, who & 31);
-                const float thr = fmaf(1e-5f * size, size, best), r4 = 4.0001f * r * r;
+                const float r4 = 4.0001f * r * r, thr = fmaf(7.5e-6f, r4, fmaf(best, 1.00006f, k0));
                 auto needed = [&](const EdgeLane &l, const EdgeNear &m) {
                     const float ux = ax - m.dx, uy = ay - m.dy, wx = ux + l.ex, wy = uy + l.ey;   // the ends - a
                     const float s2 = fmaxf(fmaf(ux, ux, uy * uy), fmaf(wx, wx, wy * wy));
@@ -457,7 +464,7 @@ sdf_min_kernel(const SortedChunk *__restrict__ chunks, int N, int csize, const f
     sincosf(th, &sn, &cs);
     const SmemEval ev = table_eval(fp, s_fp);
     const float4 box = ev.box();
-    const float size0 = fabsf(tx) + fabsf(ty) + fabsf(box.x) + fabsf(box.y) + box.z + box.w;
+    const float span = fabsf(box.x) + fabsf(box.y) + box.z + box.w;
     const int npatch = (N + kPatch - 1) / kPatch, per = csize / kPatch;   // chunks are whole patches
     // box distance of patch q's centre, and its radius with a slack far above
     // every rounding (the square root's too)
@@ -465,7 +472,7 @@ sdf_min_kernel(const SortedChunk *__restrict__ chunks, int N, int csize, const f
         const float4 cc = __ldg(&chunks[q / per].circ[q % per]);
         float cx, cy;
         body_frame(cc.x, cc.y, tx, ty, cs, sn, cx, cy);
-        r = cc.z < 0.f ? -1.f : fmaf(1e-5f, cc.w + size0, cc.z) + 1e-5f;
+        r = cc.z < 0.f ? -1.f : fmaf(1e-5f, fabsf(cx) + fabsf(cy) + cc.z + span, cc.z) + 1e-5f;
         const float ax = fabsf(cx - box.x) - box.z, ay = fabsf(cy - box.y) - box.w;
         const float mx = fmaxf(ax, 0.f), my = fmaxf(ay, 0.f);
         return sqrt_approx(fmaf(mx, mx, my * my)) + fminf(fmaxf(ax, ay), 0.f);

@@ -1,0 +1,41 @@
+"""The pruned paths at the ends of their ranges: far from the map's origin, with
+points far from all others, with safety distances beyond the scene.  Bit for bit
+against the evaluation of every point."""
+import numpy as np
+import pytest
+
+import synth
+from test_mppi_gpu import run_gpu as run_cycle
+from test_pruned_paths_gpu import FOOTPRINTS, _both, _cycle, ex  # noqa: F401 (ex: the fixture)
+
+pytestmark = pytest.mark.gpu
+
+
+def _same_cycle(ex, s):  # noqa: F811
+    a, b = run_cycle(ex, ex.Context(), s, dmin=True), run_cycle(ex, ex.Context(), s, dmin=False)
+    for k in ("costs", "weights", "U_upd", "U", "u_star"):
+        np.testing.assert_array_equal(a[k], b[k], err_msg=k)
+    assert a["valid"] == b["valid"]
+
+
+@pytest.mark.parametrize("at", [(1e4, -1e4), (-1e5, 1e5), (5e5, 4.5e6), (3e7, 0.0)])
+@pytest.mark.parametrize("cloud,fp,theta", [("uniform", "forklift", 0.0), ("wall", "far", np.pi / 2), ("uniform", "star64", 0.7)])
+def test_grid_cycle_in_map_coordinates(ex, at, cloud, fp, theta):  # noqa: F811
+    """Where the coordinates' own spacing is 1 mm, 8 mm, 0.5 m and 2 m."""
+    s = _cycle(cloud, 3000, fp, 300, 25, synth.DIFF, 77)
+    s["cloud"] = (s["cloud"] + np.array(at)).astype(np.float32)
+    s["waypoints"] = (s["waypoints"] + np.array(at)).astype(np.float32)
+    s["q0"] = np.array([at[0], at[1], theta], np.float32)
+    _same_cycle(ex, s)
+
+
+@pytest.mark.parametrize("at", [(1e4, 1e4), (-2e5, 1e5), (3e7, 0.0)])
+@pytest.mark.parametrize("dist", [True, False])
+def test_sdf_pruned_in_map_coordinates(ex, at, dist):  # noqa: F811
+    g = synth.rng(31)
+    pts = (g.uniform(-6, 6, (9000, 2)) + np.array(at)).astype(np.float32)
+    poses = np.concatenate([g.uniform(-5, 5, (1500, 2)) + np.array(at), g.uniform(-3, 3, (1500, 1))], 1).astype(np.float32)
+    poses[0, 2] = 0.0
+    (d0, m0, a0), (d1, m1, a1) = _both(ex, pts, poses, synth.POLYGON, synth.star_polygon(g, 32, 0.3, 1.2), None, dist)
+    assert d0 is None or bool((d0 == d1).all())
+    assert bool((m0 == m1).all()) and bool((a0 == a1).all())
