@@ -147,7 +147,7 @@ static int batch_grid(exact_batch *b) {
     if (cudaFuncSetAttribute(batched_sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSampleSmemMax) !=
         cudaSuccess)
         return EXACT_ECUDA;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batched_sample_kernel, b->threads, b->smem) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batched_sample_kernel, sample_threads(b), b->smem) !=
         cudaSuccess)
         return EXACT_ECUDA;
     if (per_sm < 1) return EXACT_EINVAL;
@@ -263,6 +263,7 @@ extern "C" int exact_batch_create(int n_scenes, const exact_scene *scenes, exact
     b->d_queue = reinterpret_cast<unsigned *>(b->d_ctrl + kHdrStride * n_scenes);
     b->n = n_scenes;
     b->n_items = (int)items.size();
+    b->paired = std::any_of(items.begin(), items.end(), [](int2 it) { return (it.y & kItemPair) != 0; });
     b->n_gitems = (int)gitems.size();
     b->grid_group = group;
     b->grid_T = grid_T;
@@ -350,7 +351,7 @@ static int launch_sample(exact_batch *b, const SceneDev *table, cudaStream_t st)
     if (cudaMemsetAsync(b->d_ctrl, 0, b->ctrl_bytes, st) != cudaSuccess) return EXACT_ECUDA;
     if (b->n_items > 0) {   // scenes with a d_min output
         if (!b->uniform) {
-            batched_sample_kernel<<<b->grid, b->threads, b->smem, st>>>(table, b->d_items, b->n_items, b->d_queue,
+            batched_sample_kernel<<<b->grid, sample_threads(b), b->smem, st>>>(table, b->d_items, b->n_items, b->d_queue,
                                                                          b->pairs);
             if (cudaGetLastError() != cudaSuccess) return EXACT_ECUDA;
         } else {

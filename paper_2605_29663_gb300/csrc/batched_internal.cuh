@@ -49,6 +49,7 @@ struct exact_batch {
     int n_items = 0, n_gitems = 0, n_upd = 0, n_val = 0;
     int grid_group = 1, grid_T = 1;      // samples per grid item, longest horizon of a grid scene
     size_t dmin_len = 0;                 // most d_min values of a scene that outputs them
+    bool paired = false;                 // some items take two samples
     bool pairs_matter = false;           // some scene is pruned without a grid
     char *d_ctrl = nullptr;            // n headers (kHdrStride apart) + queue head
     size_t ctrl_bytes = 0;
@@ -72,5 +73,8 @@ enum BatchPhase { kPhaseSample, kPhaseValidate };
 int launch_uniform_small(exact_batch *b, const SceneDev *table, cudaStream_t st, BatchPhase phase);
 int launch_uniform_large(exact_batch *b, const SceneDev *table, cudaStream_t st, BatchPhase phase);
 
+// Threads of the sample kernel: the tile's, and a third warp where items take
+// two samples, for the first two roll these out while the others stage the points.
+inline int sample_threads(const exact_batch *b) { return b->paired && b->threads < 96 ? 96 : b->threads; }
 inline size_t grid_smem(const exact_batch *b) { return grid_smem_bytes(b->grid_T, b->grid_group, b->threads / 32); }
 }  // namespace exact

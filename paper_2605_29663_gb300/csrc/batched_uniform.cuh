@@ -52,12 +52,12 @@ int launch_uniform_sample_t(exact_batch *b, const SceneDev *table, cudaStream_t 
         int per_sm = 0;
         // staged points (dynamic) and sample state (static) exceed the default 48 KB per block
         if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSampleSmemMax) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, b->threads, b->smem) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, sample_threads(b), b->smem) != cudaSuccess ||
             per_sm < 1)
             return EXACT_ECUDA;
         b->grid_c = b->sms * per_sm;
     }
-    k<<<b->grid_c, b->threads, b->smem, st>>>(table, b->d_items, b->n_items, b->d_queue, b->pairs,
+    k<<<b->grid_c, sample_threads(b), b->smem, st>>>(table, b->d_items, b->n_items, b->d_queue, b->pairs,
                                               ConstEval<FPC>{fpc});
     return cuda_status(cudaGetLastError());
 }

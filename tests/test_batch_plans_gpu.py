@@ -93,3 +93,16 @@ def test_autotune_times_what_a_step_runs(ex, shared):
     step = e[0].elapsed_time(e[1]) / 5
     assert report["best"]["ms"] > step / 3, (report["best"], step)
     assert all(bool((o["dmin"] > 0).all()) for o in b.outputs)
+
+
+@pytest.mark.parametrize("shared", [False, True])
+@pytest.mark.parametrize("T", [33, 64, 65])
+def test_smallest_block_with_two_samples_per_item(ex, T, shared):
+    """64 threads, with enough samples for two per item (and, at T = 65, not):
+    the warps that roll the two out leave none to stage the points."""
+    scenes = _scenes([(700, T, 300), (101, 20, 1200)], shared, T)
+    dev = [_dev_scene(ex, s) for s in scenes]
+    b = ex.Batch(dev, dmin=True)
+    b.set_tiles(64, 1)
+    b.step()
+    _check(ex, scenes, dev, b, True)
