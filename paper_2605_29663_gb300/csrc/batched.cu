@@ -3,8 +3,8 @@
 //
 // Plan (exact_batch_create, host, once): a device scene table (parameters,
 // pointers, footprint constants, scratch addresses), the work-item list of
-// the sample phase -- per scene without a d_min output one item per group of
-// samples (cloud_grid.cuh); per other scene one per (scene, sample), or per
+// the sample phase -- per scene that walks a cell grid (GridRule) one item per
+// group of samples (cloud_grid.cuh); per other scene one per (scene, sample), or per
 // (scene, two consecutive samples) when the batch holds at least four samples
 // per SM and the scene's horizon fits two in a block's step slots; scenes ordered by
 // per-sample cost T * N * edges, heaviest first (longest-processing-time
@@ -16,8 +16,8 @@
 //                           one block per cloud sorts it into a cell grid;
 //                           persistent blocks take groups of samples
 //   batched_sample_kernel   persistent: SMs x resident blocks; each block
-//                           pulls items from an atomic queue and runs
-//                           (scenes with a d_min output) sample_body with the scene's footprint constants
+//                           pulls items from an atomic queue and runs (the
+//                           other scenes) sample_body with the scene's footprint constants
 //                           in shared memory (reloaded only when the scene
 //                           changes; so are the staged points when the cloud
 //                           fits the stage);
@@ -68,7 +68,7 @@ batched_sample_kernel(const SceneDev *__restrict__ scenes, const int2 *__restric
     }
 }
 
-// The scenes without a d_min output: persistent blocks take grid items from
+// The scenes that walk a grid: persistent blocks take grid items from
 // the queue, a scene's footprint terms and distance field in shared memory.
 __global__ void __launch_bounds__(1024)   // at most 512 are launched: 64 registers, four blocks of 256 per SM
 batched_grid_sample_kernel(const SceneDev *__restrict__ scenes, const int2 *__restrict__ items, int n_items,
@@ -95,7 +95,7 @@ batched_grid_sample_kernel(const SceneDev *__restrict__ scenes, const int2 *__re
     }
 }
 
-// Cell grids of the scenes without a d_min output (one block each).
+// The cell grids (one block each).
 __global__ void __launch_bounds__(kGridThreads)
 batched_cloud_grid_kernel(const SceneDev *__restrict__ scenes, const int *__restrict__ list) {
     __shared__ GridSmem sm;
@@ -163,13 +163,42 @@ static int batch_grid(exact_batch *b) {
     return EXACT_OK;
 }
 
-// Scenes without a d_min output walk a cell grid (cloud_grid.cuh).
-static bool uses_grid(const exact_scene &S) { return !S.dmin && S.n_points <= kGridMaxPoints; }
+// Which scenes walk a cell grid (cloud_grid.cuh): those without a d_min output
+// and with 1,024 points or more, and the smaller ones where grids are built
+// anyway or pay.  Else these are items of the other sample kernel, which prunes
+// them point by point and is launched for scenes with a d_min output anyway.
+// Grids pay from about 2,048 samples on, up to T = 32, and beyond for ten points
+// a step (us, items against grids, one footprint: 4 scenes of 256 samples, T = 20,
+// 300 points 22.7, 26.4; 16 such scenes 41.8, 37.8, with T = 60 61.9, 68.5, with
+// T = 60 and 1,000 points 73.4, 72.5; four footprints: 61.8, 47.7; 84.4, 86.6; 118,
+// 94).
+struct GridRule {
+    bool small = false;   // scenes below kPruneMin points too
+    GridRule(const exact_scene *scenes, int n) {
+        bool grids = false, items = false;   // launched for other scenes anyway
+        long long samples = 0, paying = 0;
+        for (int s = 0; s < n; ++s) {
+            const exact_scene &S = scenes[s];
+            if (S.dmin || S.n_points > kGridMaxPoints) items = true;
+            else if (S.n_points >= kPruneMin) grids = true;
+            else {
+                samples += S.params.K;
+                if (S.params.T <= 32 || S.n_points >= 10 * S.params.T) paying += S.params.K;
+            }
+        }
+        const bool pays = paying >= 2048 && 2 * paying >= samples;
+        small = items ? grids && pays : grids || pays;
+    }
+    bool operator()(const exact_scene &S) const {
+        return !S.dmin && S.n_points <= kGridMaxPoints && (small || S.n_points >= kPruneMin);
+    }
+};
 
 extern "C" int exact_batch_create(int n_scenes, const exact_scene *scenes, exact_batch **out) {
     if (!out || !scenes || n_scenes < 1) return EXACT_EINVAL;
     *out = nullptr;
     if (n_scenes > 4096) return EXACT_ECAPACITY;
+    const GridRule uses_grid(scenes, n_scenes);
     std::vector<SceneDev> host(n_scenes);
     std::vector<size_t> scratch_off(n_scenes);
     size_t scratch_total = 0;
@@ -185,13 +214,13 @@ extern "C" int exact_batch_create(int n_scenes, const exact_scene *scenes, exact
         if (S.n_points > 0 && (!S.cloud || ((uintptr_t)S.cloud & 7u) != 0)) return EXACT_EINVAL;
         scratch_off[s] = scratch_total;
         scratch_total += align_up(scene_scratch_bytes(S.params.K, S.params.T, 1), 256);
-        // scenes without a d_min output get a grid and a copy of their cloud in cell order
+        // a grid and a copy of the cloud in cell order
         if (uses_grid(S))
             scratch_total += grid_copy_bytes(S.n_points, false);
         else
             max_stage = std::max(max_stage, std::min(S.n_points, kStage));
         if (S.dmin) dmin_len = std::max(dmin_len, (size_t)S.params.K * S.params.T);
-        pairs_matter |= !S.dmin && !uses_grid(S);
+        pairs_matter |= !S.dmin && S.n_points >= kPruneMin && !uses_grid(S);
     }
     std::vector<int> sort_list;
     for (int s = 0; s < n_scenes; ++s)
@@ -349,7 +378,7 @@ static int launch_uniform(exact_batch *b, const SceneDev *table, cudaStream_t st
 
 static int launch_sample(exact_batch *b, const SceneDev *table, cudaStream_t st) {
     if (cudaMemsetAsync(b->d_ctrl, 0, b->ctrl_bytes, st) != cudaSuccess) return EXACT_ECUDA;
-    if (b->n_items > 0) {   // scenes with a d_min output
+    if (b->n_items > 0) {   // scenes that walk no grid
         if (!b->uniform) {
             batched_sample_kernel<<<b->grid, sample_threads(b), b->smem, st>>>(table, b->d_items, b->n_items, b->d_queue,
                                                                          b->pairs);

@@ -30,7 +30,7 @@ __device__ __forceinline__ void stage_view(SceneView &dst, const SceneView &src)
     __syncthreads();
 }
 
-// A sample item of a scene with a d_min output is (scene, r); bit 30 of r
+// A sample item of a scene that walks no grid is (scene, r); bit 30 of r
 // marks an item that also takes sample r + 1 of the same scene (see
 // sample_body).  A grid item is (scene, r): grid_group consecutive samples
 // from r on (see grid_samples).

@@ -30,14 +30,30 @@ def _scenes(sizes, shared, seed):
     return out
 
 
+def _mixed_batch(ex, scenes, dev, dmin):
+    """A batch whose scene i has a d_min output when dmin[i]."""
+    import ctypes
+    arr, outputs, keep = ex._scene_array(dev, True, True, True, True, False)
+    for i, want in enumerate(dmin):
+        if not want:
+            arr[i].dmin = None
+            outputs[i].pop("dmin")
+    h = ctypes.c_void_p()
+    ex._check(ex.load().exact_batch_create(len(dev), ctypes.cast(arr, ctypes.c_void_p), ctypes.byref(h)), "create")
+    b = ex.Batch.__new__(ex.Batch)
+    b._h, b.n, b.outputs, b._keep, b.class_key = h, len(dev), outputs, keep, ""
+    return b
+
+
 def _check(ex, scenes, dev, b, dmin):
     import torch
     torch.cuda.synchronize()
     assert b.get_error() == 0
     ctx = ex.Context()
+    dmin = dmin if isinstance(dmin, list) else [dmin] * len(scenes)
     for i, (s, d, o) in enumerate(zip(scenes, dev, b.outputs)):
-        want = _run_single(ex, ctx, s, dmin=dmin)
-        for k in ("costs", "weights", "U_upd", "u_star"):
+        want = _run_single(ex, ctx, s, dmin=dmin[i])
+        for k in ("costs", "weights", "U_upd", "u_star") + (("dmin",) if dmin[i] else ()):
             np.testing.assert_array_equal(o[k].cpu().numpy(), want[k], err_msg=f"scene {i} {k}")
         np.testing.assert_array_equal(d["U"].cpu().numpy(), want["U"], err_msg=f"scene {i} U")
 
@@ -93,6 +109,34 @@ def test_autotune_times_what_a_step_runs(ex, shared):
     step = e[0].elapsed_time(e[1]) / 5
     assert report["best"]["ms"] > step / 3, (report["best"], step)
     assert all(bool((o["dmin"] > 0).all()) for o in b.outputs)
+
+
+@pytest.mark.parametrize("shared", [False, True])
+@pytest.mark.parametrize("sizes,dmin", [
+    ([(100, 20, 300), (64, 12, 1023), (200, 33, 900)], [0, 0, 0]),                  # few samples: items
+    ([(1500, 32, 100), (700, 20, 1), (300, 60, 599)], [0, 0, 0]),                   # many: grids
+    ([(1500, 33, 100), (700, 60, 400), (300, 20, 600)], [0, 0, 0]),                 # many, most of them not paying: items
+    ([(100, 20, 300), (64, 12, 1024), (200, 33, 0)], [0, 0, 0]),                    # beside a grid
+    ([(100, 20, 300), (64, 12, 700), (3000, 20, 800)], [1, 0, 0]),                  # beside d_min scenes: items
+    ([(100, 20, 300), (64, 12, 3000), (3000, 20, 800), (50, 9, 5000)], [1, 0, 0, 1]),   # beside both, many: grids
+    ([(100, 20, 300), (64, 12, 3000), (30, 20, 800), (50, 9, 5000)], [1, 0, 0, 1])])    # beside both, few: items
+def test_scenes_of_every_route_in_one_batch(ex, sizes, dmin, shared):
+    """Small scenes as items or on grids, alone, beside scenes that walk one and
+    beside scenes with a d_min output: each gives its single-scene bits, twice in
+    a row, whatever the block size."""
+    import torch
+    scenes = _scenes(sizes, shared, len(sizes) + sum(dmin))
+    for tiles in (None, (64, 8), (512, 1)):
+        dev = [_dev_scene(ex, s) for s in scenes]
+        b = _mixed_batch(ex, scenes, dev, dmin)
+        if tiles:
+            b.set_tiles(*tiles)
+        b.step()
+        _check(ex, scenes, dev, b, [bool(d) for d in dmin])
+        for s, d in zip(scenes, dev):
+            d["U"].copy_(torch.from_numpy(s["U"]))
+        b.step()
+        _check(ex, scenes, dev, b, [bool(d) for d in dmin])
 
 
 @pytest.mark.parametrize("shared", [False, True])
