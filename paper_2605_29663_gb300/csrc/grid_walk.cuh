@@ -22,11 +22,13 @@ struct CloudGrid {
 };
 constexpr size_t kGridBytes = (sizeof(CloudGrid) + 255) / 256 * 256;
 // A predicted cloud gets one grid per horizon step over its points' positions
-// at that step, while those fit kStepGridBytes; else one grid whose cells are
-// searched as far as the fastest point can have moved.  (Measured with K =
-// 1,024, T = 20, 2,048 points on boxes and discs at 0.5 m/s: the cycle takes
-// 27 to 29 us with a grid per step, 45 to 52 us with one.)
-constexpr size_t kStepGridBytes = 64u << 20;
+// at that step, while those fit kStepGridBytes (8 bytes per point and step: the
+// most try_work gives); else one grid whose cells are searched as far as the
+// fastest point can have moved.  (Measured with K = 1,024, T = 20, 2,048 points
+// on boxes and discs at 0.5 m/s: the cycle takes 27 to 29 us with a grid per step,
+// 45 to 52 us with one; K = 256, T = 100, 100,000 points at 0.3 m/s 0.29 ms against
+// 9.2, at 30 m/s 0.19 against 17.3.)
+constexpr size_t kStepGridBytes = (size_t)1 << 30;
 // The grid of step h and the first of its points: grid + h * grids, point
 // h * points (both 0 for a static cloud).
 struct GridStride {

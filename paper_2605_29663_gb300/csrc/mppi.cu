@@ -131,9 +131,9 @@ extern "C" int exact_ctx_reserve_cloud(exact_ctx *ctx, int max_poses, int max_K,
     if (!ctx || max_poses < 0 || max_K < 0 || max_T < 0 || max_points < 0) return EXACT_EINVAL;
     int rc = ensure_scratch(ctx, kArenaHeader + scene_scratch_bytes(max_K, max_T, parts_of(ctx, max_K, max_T)));
     if (rc == EXACT_OK && max_points >= kPruneMin) {
-        const size_t work = std::max(grid_copy_bytes(std::min(max_points, kGridMaxPoints), true),   // static or predicted
-                                     std::min(step_grid_bytes(max_points, max_T), kStepGridBytes));
-        rc = try_work(ctx, work, nullptr) ? EXACT_OK : EXACT_ECUDA;
+        // static or predicted; a grid per step is a matter of speed, not needed
+        const size_t one = grid_copy_bytes(std::min(max_points, kGridMaxPoints), true), steps = step_grid_bytes(max_points, max_T);
+        if (!(steps <= kStepGridBytes && try_work(ctx, std::max(one, steps), nullptr)) && !try_work(ctx, one, nullptr)) rc = EXACT_ECUDA;
     }
     if (rc == EXACT_OK) rc = sdf_reserve(ctx, max_points, max_poses);
     return rc;

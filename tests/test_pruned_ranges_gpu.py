@@ -39,3 +39,22 @@ def test_sdf_pruned_in_map_coordinates(ex, at, dist):  # noqa: F811
     (d0, m0, a0), (d1, m1, a1) = _both(ex, pts, poses, synth.POLYGON, synth.star_polygon(g, 32, 0.3, 1.2), None, dist)
     assert d0 is None or bool((d0 == d1).all())
     assert bool((m0 == m1).all()) and bool((a0 == a1).all())
+
+
+@pytest.mark.parametrize("N,T,speed", [(120_000, 80, 0.3), (4000, 25, 30.0), (1_200_000, 128, 1.0)])
+def test_predicted_cycle_with_a_grid_per_step_or_one(ex, N, T, speed):  # noqa: F811
+    """Grids of all steps together below and above 64 MB, and beyond 1 GB (one
+    grid for all steps): the bits of the evaluation of every point."""
+    import torch
+    g = synth.rng(N)
+    s = synth.plain_step(4, K=8, T=T, N=8)
+    t = {k: torch.from_numpy(np.ascontiguousarray(s[k])).cuda() for k in ("q0", "waypoints", "eps")}
+    cloud = torch.from_numpy(g.uniform(-40, 40, (N, 2)).astype(np.float32)).cuda()
+    vel = torch.from_numpy(g.normal(0, speed, (N, 2)).astype(np.float32)).cuda()
+    fp, res = ex.Footprint(s["kind"], s["fp"]), []
+    for dmin in (True, False):
+        U = torch.from_numpy(s["U"]).cuda()
+        o = ex.mppi_step(ex.Context(), t["q0"], cloud, t["waypoints"], U, t["eps"], fp, s["params"], velocity=vel, dmin=dmin)
+        res.append(dict(o, U=U))
+    for k in ("costs", "weights", "U_upd", "u_star", "valid", "U"):
+        assert torch.equal(res[0][k], res[1][k]), k
