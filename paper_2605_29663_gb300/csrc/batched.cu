@@ -70,6 +70,8 @@ batched_sample_kernel(const SceneDev *__restrict__ scenes, const int2 *__restric
 
 // The scenes that walk a grid: persistent blocks take grid items from
 // the queue, a scene's footprint terms and distance field in shared memory.
+// FAR: some scene's field ends before its d_safe.
+template <bool FAR>
 __global__ void __launch_bounds__(1024)   // at most 512 are launched: 64 registers, four blocks of 256 per SM
 batched_grid_sample_kernel(const SceneDev *__restrict__ scenes, const int2 *__restrict__ items, int n_items,
                            int group, unsigned *queue) {
@@ -90,7 +92,7 @@ batched_grid_sample_kernel(const SceneDev *__restrict__ scenes, const int2 *__re
             __syncthreads();
             fp_scene = it.x;
         }
-        grid_samples<false>(D.V, D.grid, GridStride{0, 0}, table_eval(D.fp, s_fp), it.y, min(group, D.V.P.K - it.y),
+        grid_samples<false, FAR>(D.V, D.grid, GridStride{0, 0}, table_eval(D.fp, s_fp), it.y, min(group, D.V.P.K - it.y),
                             reinterpret_cast<char *>(dyn), fresh, &s_next);
     }
 }
@@ -153,9 +155,10 @@ static int batch_grid(exact_batch *b) {
     if (per_sm < 1) return EXACT_EINVAL;
     b->grid = b->sms * per_sm;
     if (b->n_gitems == 0) return EXACT_OK;
-    if (cudaFuncSetAttribute(batched_grid_sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const auto grid_kernel = b->far ? batched_grid_sample_kernel<true> : batched_grid_sample_kernel<false>;
+    if (cudaFuncSetAttribute(grid_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kGridSmemMax) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batched_grid_sample_kernel, b->threads, grid_smem(b)) !=
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, grid_kernel, b->threads, grid_smem(b)) !=
             cudaSuccess)
         return EXACT_ECUDA;
     if (per_sm < 1) return EXACT_EINVAL;
@@ -298,6 +301,7 @@ extern "C" int exact_batch_create(int n_scenes, const exact_scene *scenes, exact
     b->grid_T = grid_T;
     b->dmin_len = dmin_len;
     b->pairs_matter = pairs_matter;
+    for (int s : sort_list) b->far |= field_ends(scenes[s].params.d_safe, scenes[s].fp->bhx, scenes[s].fp->bhy);
     b->n_upd = (int)upd.size();
     b->n_val = (int)val.size();
     b->smem = kFpSlots * sizeof(float4) + (size_t)max_stage * sizeof(float2);
@@ -394,7 +398,7 @@ static int launch_sample(exact_batch *b, const SceneDev *table, cudaStream_t st)
     // the persistent warps start early (rollouts first; grid_sample waits
     // before it reads a grid)
     // no more blocks than items: idle ones would crowd the busy ones on an SM
-    return cuda_status(launch_dependent(batched_grid_sample_kernel, (unsigned)std::min(b->ggrid, b->n_gitems), (unsigned)b->threads,
+    return cuda_status(launch_dependent(b->far ? batched_grid_sample_kernel<true> : batched_grid_sample_kernel<false>, (unsigned)std::min(b->ggrid, b->n_gitems), (unsigned)b->threads,
                                         grid_smem(b), st, table, (const int2 *)b->d_gitems, b->n_gitems, b->grid_group,
                                         b->d_queue + 1));
 }

@@ -49,6 +49,7 @@ struct exact_batch {
     int n_items = 0, n_gitems = 0, n_upd = 0, n_val = 0;
     int grid_group = 1, grid_T = 1;      // samples per grid item, longest horizon of a grid scene
     size_t dmin_len = 0;                 // most d_min values of a scene that outputs them
+    bool far = false;                    // some grid scene's field ends before its d_safe
     bool paired = false;                 // some items take two samples
     bool pairs_matter = false;           // some scene is pruned without a grid
     char *d_ctrl = nullptr;            // n headers (kHdrStride apart) + queue head

@@ -228,13 +228,22 @@ __device__ __forceinline__ void atomic_min(float *a, float v) {
 // smallest upper bound of a step's points replaces d_safe as what still
 // matters, and only the points whose lower bound is below it are evaluated
 // (a few per step, whatever the number of points inside the footprint).
+// A safety distance far beyond the footprint's size would leave the cells too
+// coarse to tell its points apart: the field then ends at twice the box's half
+// extent, and beyond it the box bounds the distance (its own, and that of its
+// farthest corner).  (K = 1,024, T = 30, 4,000 points all within d_safe = 50 m:
+// 207 us against 923 with the field over all of it, forklift 142 against 654.)
 struct Field {
     float x0, y0, ix, iy, rd;
 };
+// Whether the field ends before d_safe (the kernels' FAR: as a branch at run time
+// it cost every cycle 1 to 2 %).
+__host__ __device__ inline bool field_ends(float d_safe, float hx, float hy) { return d_safe > 2.f * fmaxf(hx, hy); }
 template <class EV>
 __device__ __forceinline__ Field make_field(const EV &ev, float cap) {
     const float4 fb = ev.box();
-    const float hx = fb.z + cap + 2.f * kPruneSlack, hy = fb.w + cap + 2.f * kPruneSlack;
+    const float m = fminf(cap, 2.f * fmaxf(fb.z, fb.w));
+    const float hx = fb.z + m + 2.f * kPruneSlack, hy = fb.w + m + 2.f * kPruneSlack;
     const float cx = 2.f * hx / kField, cy = 2.f * hy / kField;
     return Field{fb.x - hx, fb.y - hy, 1.f / cx, 1.f / cy, fmaf(0.50001f, sqrtf(fmaf(cx, cx, cy * cy)), 0.1f * kPruneSlack)};
 }
@@ -253,7 +262,8 @@ __device__ __forceinline__ void fill_field(const EV &ev, const Field &f, float *
 // calls.  mem holds grid_smem_bytes(V.P.T, ns, warps) bytes, first the
 // footprint's distance field (filled here when fill is set), and next is a
 // shared counter.  The keys are the same bits whatever warp takes a slot.
-template <bool MOVING, class EV>
+// FAR: field_ends for the scene (and right, but slower, where it does not).
+template <bool MOVING, bool FAR, class EV>
 __device__ __forceinline__ void grid_samples(const SceneView &V, const CloudGrid *grid, GridStride gst, const EV &ev,
                                              int r0, int ns, char *mem, bool fill, int *next) {
     const MppiP &P = V.P;
@@ -272,7 +282,7 @@ __device__ __forceinline__ void grid_samples(const SceneView &V, const CloudGrid
     char *own = reinterpret_cast<char *>(term + kGroup) + warp * (kRuns * 12 + kEvals * 8);
     int2 *eval = reinterpret_cast<int2 *>(own);
     int *run_p = reinterpret_cast<int *>(eval + kEvals), *run_n = run_p + kRuns, *run_s = run_n + kRuns;
-    const float cap = fmaxf(P.d_safe, 0.f);
+    const float cap = fminf(fmaxf(P.d_safe, 0.f), kCapMax);
     const Field fd = make_field(ev, cap);
     if (fill) fill_field(ev, fd, field);
     for (int s = warp; s < ns; s += nwarps) {
@@ -372,12 +382,17 @@ __device__ __forceinline__ void grid_samples(const SceneView &V, const CloudGrid
                         const float2 o = point_at(i[q], sl[q]);
                         float px, py;
                         body_frame(o.x, o.y, p.x, p.y, p.z, p.w, px, py);
-                        // cell of the field; a point outside it is farther than d_safe
+                        // cell of the field; a point outside one that reaches as far is farther than d_safe
                         const float u = (px - fd.x0) * fd.ix, v = (py - fd.y0) * fd.iy;
                         if (u >= 0.f && u < (float)kField && v >= 0.f && v < (float)kField) {
                             const float f = field[(int)v * kField + (int)u];
                             lb[q] = f - fd.rd;
                             ub[q] = f + fd.rd;
+                        } else if constexpr (FAR) {
+                            const float ax = fabsf(px - fb.x), ay = fabsf(py - fb.y);
+                            const float e = fmaf(1e-5f, ax + ay, 0.1f * kPruneSlack);
+                            lb[q] = fmaxf(ax - fb.z, ay - fb.w) - e;
+                            ub[q] = (ax + fb.z) + (ay + fb.w) + e;
                         }
                     }
                     lower |= ub[q] < now[q];

@@ -11,6 +11,9 @@ constexpr int kCells = 8192;          // cell-start table size (nx * ny <= kCell
 constexpr float kCellTarget = 7600.f; // nx * ny aimed at: (a + 1)(b + 1) <= kCells for a b <= 7600, a, b < 256
 constexpr int kGridDim = 256;         // most cells along one axis
 
+// Most that a safety distance counts for: beyond, squares would overflow.
+constexpr float kCapMax = 1e15f;
+
 struct __align__(16) GridHead {
     float lx, ly, inv, cell;   // lower corner, 1 / cell size, cell size
     float vmax;                // largest point speed (predicted clouds)

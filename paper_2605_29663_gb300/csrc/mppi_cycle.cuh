@@ -1293,7 +1293,7 @@ __device__ __forceinline__ void validate_body(const SceneView &V, const EV &ev, 
     int row = warp, rows = 0;
     if (grid) {
         g = load_head(grid);
-        lim = fmaxf(P.d_safe, 0.f) + kPruneSlack;
+        lim = fminf(fmaxf(P.d_safe, 0.f), kCapMax) + kPruneSlack;
         if (MOVING) lim = fmaf(th, g.vmax, lim);
         w = row_walk(g, qp, ev.box(), lim);
         rows = walk_rows(w);

@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(kBlock) mppi_validate_kernel(const SceneView V
 // its kernels take the footprint as a slot table in the kernel parameters,
 // copied to shared memory: one kernel for every footprint, small enough to be
 // fetched quickly.  Sample phase: block b takes samples b group ...
-template <bool MOVING>
+template <bool MOVING, bool FAR>
 __global__ void __launch_bounds__(kBlock, 3)
 mppi_grid_sample_kernel(const SceneView V, const __grid_constant__ FpTable fp, const CloudGrid *grid, GridStride gst,
                         int group) {
@@ -68,7 +68,7 @@ mppi_grid_sample_kernel(const SceneView V, const __grid_constant__ FpTable fp, c
     load_table(s_fp, fp);
     __syncthreads();
     const int r0 = (int)blockIdx.x * group;
-    grid_samples<MOVING>(V, grid, gst, table_eval(fp, s_fp), r0, min(group, V.P.K - r0), reinterpret_cast<char *>(s_mem),
+    grid_samples<MOVING, FAR>(V, grid, gst, table_eval(fp, s_fp), r0, min(group, V.P.K - r0), reinterpret_cast<char *>(s_mem),
                          true, &s_next);
 }
 template <bool MOVING>
@@ -113,12 +113,14 @@ int launch_grid_cycle_t(const SceneView &V, const exact_footprint *fp, cudaStrea
                         GridStride gst, int sms) {
     const int group = grid_group(V.P.K, V.P.T, kBlock / 32, sms);
     const size_t smem = grid_smem_bytes(V.P.T, group, kBlock / 32);
+    auto sample = field_ends(V.P.d_safe, fp->bhx, fp->bhy) ? mppi_grid_sample_kernel<MOVING, true>
+                                                            : mppi_grid_sample_kernel<MOVING, false>;
     // beyond the default 48 KB with the footprint's slots
-    if (smem > 40u * 1024u && cudaFuncSetAttribute(mppi_grid_sample_kernel<MOVING>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)kGridSmemMax) != cudaSuccess)
+    if (smem > 40u * 1024u &&
+        cudaFuncSetAttribute(sample, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGridSmemMax) != cudaSuccess)
         return EXACT_ECUDA;
     const FpTable t = make_table(fp);
-    if (launch_dependent(mppi_grid_sample_kernel<MOVING>, (V.P.K + group - 1) / group, kBlock, smem, st, V, t, grid,
+    if (launch_dependent(sample, (V.P.K + group - 1) / group, kBlock, smem, st, V, t, grid,
                          gst, group) != cudaSuccess ||
         launch_dependent(mppi_update_kernel<MOVING>, V.upd_blocks, kUpdBlock, 0, st, V) != cudaSuccess)
         return EXACT_ECUDA;

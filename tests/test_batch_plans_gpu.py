@@ -53,7 +53,7 @@ def _check(ex, scenes, dev, b, dmin):
     dmin = dmin if isinstance(dmin, list) else [dmin] * len(scenes)
     for i, (s, d, o) in enumerate(zip(scenes, dev, b.outputs)):
         want = _run_single(ex, ctx, s, dmin=dmin[i])
-        for k in ("costs", "weights", "U_upd", "u_star") + (("dmin",) if dmin[i] else ()):
+        for k in ("costs", "weights", "U_upd", "u_star") + (("dmin",) if "dmin" in o else ()):
             np.testing.assert_array_equal(o[k].cpu().numpy(), want[k], err_msg=f"scene {i} {k}")
         np.testing.assert_array_equal(d["U"].cpu().numpy(), want["U"], err_msg=f"scene {i} U")
 
@@ -148,5 +148,16 @@ def test_smallest_block_with_two_samples_per_item(ex, T, shared):
     dev = [_dev_scene(ex, s) for s in scenes]
     b = ex.Batch(dev, dmin=True)
     b.set_tiles(64, 1)
+    b.step()
+    _check(ex, scenes, dev, b, True)
+
+
+def test_batch_with_a_safety_distance_beyond_the_field(ex):
+    """One scene whose distance field ends before its d_safe beside one whose
+    does not."""
+    scenes = _scenes([(300, 20, 2000), (300, 20, 1500)], False, 12)
+    scenes[1]["params"]["d_safe"] = 7.0
+    dev = [_dev_scene(ex, s) for s in scenes]
+    b = ex.Batch(dev, dmin=False)
     b.step()
     _check(ex, scenes, dev, b, True)

@@ -58,3 +58,16 @@ def test_predicted_cycle_with_a_grid_per_step_or_one(ex, N, T, speed):  # noqa: 
         res.append(dict(o, U=U))
     for k in ("costs", "weights", "U_upd", "u_star", "valid", "U"):
         assert torch.equal(res[0][k], res[1][k]), k
+
+
+@pytest.mark.parametrize("d_safe", [0.0, -1.0, 2.0, 50.0, 3e4, 1e12, 1e25, np.inf])
+@pytest.mark.parametrize("cloud,fp,mask", [("uniform", "forklift", True), ("wall", "far", False), ("uniform", "star64", False)])
+def test_grid_cycle_at_any_safety_distance(ex, d_safe, cloud, fp, mask):  # noqa: F811
+    """The field that ends before d_safe, points inside it, beyond it and none of
+    them; distances whose squares overflow (costs that are not numbers, the same
+    ones), none and negative ones."""
+    s = _cycle(cloud, 2500, fp, 200, 25, synth.DIFF, 3, mask)
+    s["params"]["d_safe"] = d_safe
+    if d_safe == 50.0:
+        s["cloud"] += np.float32(30.0)
+    _same_cycle(ex, s)
