@@ -28,6 +28,7 @@
 // against 34 us).
 #pragma once
 
+#include "cell_window.cuh"
 #include "mppi_cycle.cuh"
 
 namespace exact {
@@ -39,12 +40,18 @@ struct GridSmem {
     int cnt[kCells + 1];
     float red[5][kGridThreads / 32];
     int part[kGridThreads / 32];
+    WindowSmem<kGridDim, kGridDim> window;
 };
 
 // One block sorts the cloud's valid points (unmasked, finite position and
 // velocity) into cells: opts / ovel in cell order, grid header and cell
 // starts.  The order inside a cell follows the scatter's atomics; nothing
 // computed from the cloud depends on it (minima are exact in any order).
+// Where a cell holds more than 1/64 of the points and most of them lie in a small
+// window, the cells are laid over that window again, and what lies outside goes
+// to its border cells (GridHead::open): a cloud of 8,000 points on 12 m x 12 m and
+// one point 10 km away, K = 2,048, T = 30, 80 us against 1,835 with cells over all of
+// it.
 // PREDICT: the points are taken where they are at time th.
 template <bool MOVING, bool PREDICT = false>
 __device__ __forceinline__ void build_grid(const float2 *__restrict__ pts, const float2 *__restrict__ vel,
@@ -64,69 +71,97 @@ __device__ __forceinline__ void build_grid(const float2 *__restrict__ pts, const
     const bool inreg = N <= kGridRegs * nt;
     float2 rp[kGridRegs], rv[kGridRegs];
     bool ok[kGridRegs];
-    float lx = finf(), ly = finf(), hx = -finf(), hy = -finf(), vm = 0.f;
-    auto grow = [&](float2 p, float2 v) {
-        lx = fminf(lx, p.x); hx = fmaxf(hx, p.x); ly = fminf(ly, p.y); hy = fmaxf(hy, p.y);
-        if (MOVING) vm = fmaxf(vm, fabsf(v.x) + fabsf(v.y));
-    };
     if (inreg) {
 #pragma unroll
         for (int k = 0; k < kGridRegs; ++k) {
             const int i = tid + k * nt;
             ok[k] = i < N && fetch(i, rp[k], rv[k]);
         }
-#pragma unroll
-        for (int k = 0; k < kGridRegs; ++k)
-            if (ok[k]) grow(rp[k], rv[k]);
-    } else {
-#pragma unroll 4
-        for (int i = tid; i < N; i += nt) {
-            float2 p, v;
-            if (fetch(i, p, v)) grow(p, v);
-        }
     }
-    for (int c = tid; c <= kCells; c += nt) sm.cnt[c] = 0;
-    lx = warp_min_f(lx); ly = warp_min_f(ly); hx = -warp_min_f(-hx); hy = -warp_min_f(-hy);
-    if (MOVING) vm = -warp_min_f(-vm);
-    if (lane == 0) {
-        sm.red[0][warp] = lx; sm.red[1][warp] = ly; sm.red[2][warp] = hx; sm.red[3][warp] = hy;
-        sm.red[4][warp] = vm;
-    }
-    __syncthreads();
-    {   // every warp reduces the warps' boxes itself: one barrier less
-        const bool w = lane < nw;
-        lx = warp_min_f(w ? sm.red[0][lane] : finf());
-        ly = warp_min_f(w ? sm.red[1][lane] : finf());
-        hx = -warp_min_f(w ? -sm.red[2][lane] : finf());
-        hy = -warp_min_f(w ? -sm.red[3][lane] : finf());
-        if (MOVING) vm = -warp_min_f(w ? -sm.red[4][lane] : 0.f);
-    }
-    // square cells over the box; a cloud without a valid point gets one cell
-    const bool any = lx <= hx;
-    if (!any) lx = ly = hx = hy = 0.f;
-    const float w = hx - lx, h = hy - ly, wide = fmaxf(w, h);
-    const float target = fminf(kCellTarget, fmaxf(1000.f, 2.f * (float)N));
-    const float cell = fmaxf(fmaxf(sqrtf(w * (h / target)), wide / (float)(kGridDim - 1)), 1e-6f);
-    const float inv = 1.f / cell;
-    const int nx = min(kGridDim, (int)(w * inv) + 1), ny = min(kGridDim, (int)(h * inv) + 1);
-    const int ncell = min(kCells, nx * ny);
+    float lx, ly, hx, hy, vm = 0.f;
+    float wx0 = 0.f, wy0 = 0.f, wx1 = 0.f, wy1 = 0.f;   // the window
+    float cell, inv;
+    int nx, ny, ncell, rc[kGridRegs], rank[kGridRegs];   // cell, place among its points
     auto cell_of = [&](float2 p) { return cell_axis(p.y, ly, inv, ny) * nx + cell_axis(p.x, lx, inv, nx); };
-    int rc[kGridRegs], rank[kGridRegs];   // cell, place among its points
-    if (inreg) {
+    // cells over the points (those in the window) and the counts of all; whether
+    // some cell holds more than 1/64 of them
+    auto lay = [&](auto windowed) {
+        constexpr bool W = decltype(windowed)::value;
+        lx = ly = finf();
+        hx = hy = -finf();
+        auto grow = [&](float2 p, float2 v) {
+            if (W && (p.x < wx0 || p.x > wx1 || p.y < wy0 || p.y > wy1)) return;
+            lx = fminf(lx, p.x); hx = fmaxf(hx, p.x); ly = fminf(ly, p.y); hy = fmaxf(hy, p.y);
+            if (MOVING && !W) vm = fmaxf(vm, fabsf(v.x) + fabsf(v.y));
+        };
+        if (inreg) {
 #pragma unroll
-        for (int k = 0; k < kGridRegs; ++k)
-            if (ok[k]) {
-                rc[k] = min(ncell - 1, cell_of(rp[k]));
-                rank[k] = atomicAdd(&sm.cnt[rc[k]], 1);
-            }
-    } else {
+            for (int k = 0; k < kGridRegs; ++k)
+                if (ok[k]) grow(rp[k], rv[k]);
+        } else {
 #pragma unroll 4
-        for (int i = tid; i < N; i += nt) {
-            float2 p, v;
-            if (fetch(i, p, v)) atomicAdd(&sm.cnt[min(ncell - 1, cell_of(p))], 1);
+            for (int i = tid; i < N; i += nt) {
+                float2 p, v;
+                if (fetch(i, p, v)) grow(p, v);
+            }
         }
-    }
-    __syncthreads();
+        for (int c = tid; c <= kCells; c += nt) sm.cnt[c] = 0;
+        lx = warp_min_f(lx); ly = warp_min_f(ly); hx = -warp_min_f(-hx); hy = -warp_min_f(-hy);
+        if (MOVING && !W) vm = -warp_min_f(-vm);
+        if (lane == 0) {
+            sm.red[0][warp] = lx; sm.red[1][warp] = ly; sm.red[2][warp] = hx; sm.red[3][warp] = hy;
+            if (!W) sm.red[4][warp] = vm;
+        }
+        __syncthreads();
+        {   // every warp reduces the warps' boxes itself: one barrier less
+            const bool w = lane < nw;
+            lx = warp_min_f(w ? sm.red[0][lane] : finf());
+            ly = warp_min_f(w ? sm.red[1][lane] : finf());
+            hx = -warp_min_f(w ? -sm.red[2][lane] : finf());
+            hy = -warp_min_f(w ? -sm.red[3][lane] : finf());
+            if (MOVING && !W) vm = -warp_min_f(w ? -sm.red[4][lane] : 0.f);
+        }
+        // square cells over the box; a cloud without a valid point gets one cell
+        const bool any = lx <= hx;
+        if (!any) lx = ly = hx = hy = 0.f;
+        const float w = hx - lx, h = hy - ly, wide = fmaxf(w, h);
+        const float target = fminf(kCellTarget, fmaxf(1000.f, 2.f * (float)N));
+        cell = fmaxf(fmaxf(sqrtf(w * (h / target)), wide / (float)(kGridDim - 1)), 1e-6f);
+        inv = 1.f / cell;
+        nx = min(kGridDim, (int)(w * inv) + 1);
+        ny = min(kGridDim, (int)(h * inv) + 1);
+        ncell = min(kCells, nx * ny);
+        bool crowded = false;
+        if (inreg) {
+#pragma unroll
+            for (int k = 0; k < kGridRegs; ++k)
+                if (ok[k]) {
+                    rc[k] = min(ncell - 1, cell_of(rp[k]));
+                    rank[k] = atomicAdd(&sm.cnt[rc[k]], 1);
+                    crowded |= rank[k] >= N / 64;
+                }
+        } else {
+#pragma unroll 4
+            for (int i = tid; i < N; i += nt) {
+                float2 p, v;
+                if (fetch(i, p, v)) atomicAdd(&sm.cnt[min(ncell - 1, cell_of(p))], 1);
+            }
+            __syncthreads();
+            for (int c = tid; c < ncell; c += nt) crowded |= sm.cnt[c] > N / 64;
+        }
+        return __syncthreads_or(crowded) != 0;
+    };
+    int open = 0;
+    if (lay(std::false_type{}))
+        for (int zoom = 0; zoom < kZooms; ++zoom) {
+            cell_window<false>(sm.cnt, ny, nx, sm.window);
+            wx0 = lx; wx1 = hx; wy0 = ly; wy1 = hy;
+            const bool cx = cut_axis(nx, cell, sm.window.lo[1], sm.window.hi[1], wx0, wx1);
+            const bool cy = cut_axis(ny, cell, sm.window.lo[0], sm.window.hi[0], wy0, wy1);
+            if (!cx && !cy) break;
+            open = 1;
+            if (!lay(std::true_type{})) break;
+        }
     // exclusive prefix over the counts: contiguous segments per thread
     const int per = ((ncell + nt) / nt) | 1, c0 = tid * per, c1 = min(ncell + 1, c0 + per);   // odd: no bank conflicts
     int s = 0;
@@ -151,7 +186,7 @@ __device__ __forceinline__ void build_grid(const float2 *__restrict__ pts, const
         }
     }
     if (tid == 0) {
-        grid->head = GridHead{lx, ly, inv, cell, MOVING ? vm * 1.0001f : 0.f, 0, nx, ny};
+        grid->head = GridHead{lx, ly, inv, cell, MOVING ? vm * 1.0001f : 0.f, open, nx, ny};
     }
     __syncthreads();
     for (int c = tid; c <= ncell; c += nt) grid->start[c] = sm.cnt[c];

@@ -17,7 +17,8 @@ constexpr float kCapMax = 1e15f;
 struct __align__(16) GridHead {
     float lx, ly, inv, cell;   // lower corner, 1 / cell size, cell size
     float vmax;                // largest point speed (predicted clouds)
-    int pad, nx, ny;
+    int open;                  // points outside lie in the border cells
+    int nx, ny;
 };
 struct CloudGrid {
     GridHead head;
@@ -106,11 +107,18 @@ __device__ __forceinline__ RowWalk row_walk(const GridHead &g, float4 pose, floa
     const float rx = fmaf(r.ac, ex, r.as * ey), ry = fmaf(r.as, ex, r.ac * ey);
     const float a = (r.cwy - ry - g.ly) * g.inv, b = (r.cwy + ry - g.ly) * g.inv;
     const float u = (r.cwx - rx - g.lx) * g.inv, v = (r.cwx + rx - g.lx) * g.inv;
-    // points lie in [0, ny] x [0, nx] of these coordinates: a box beyond holds none
-    const bool meets = !(a > (float)g.ny || b < 0.f || u > (float)g.nx || v < 0.f);
+    // points lie in [0, ny] x [0, nx] of these coordinates: a box beyond holds
+    // none, unless the border cells hold the points beyond
+    const bool meets = g.open || !(a > (float)g.ny || b < 0.f || u > (float)g.nx || v < 0.f);
     r.j0 = max(0, min(g.ny - 1, (int)a));
     r.j1 = meets ? min(g.ny - 1, max(0, (int)b)) : -1;
     r.jc = max(r.j0, min(r.j1, (int)((r.cwy - g.ly) * g.inv)));
+    if (g.open && (r.j0 == 0 || r.j1 == g.ny - 1)) {   // a border row has no outer edge: the whole width of the box
+        r.k1 = r.k2 = 0.f;
+        r.i1 = r.i2 = 1e6f;
+        r.y0 = -finf();
+        r.dy = finf();
+    }
     return r;
 }
 // Rows from the centre outwards: the k-th (k = 0, 1, ...) is jc, jc + 1,
@@ -134,7 +142,6 @@ __device__ __forceinline__ void row_run(const GridHead &g, const int *start, con
     // a box shrunk to nothing, a row beyond it, or a non-finite pose
     if (!(ex >= 0.f && ey >= 0.f && a <= b && lo <= hi)) return;
     const float fa = (r.cwx + lo - g.lx) * g.inv, fb = (r.cwx + hi - g.lx) * g.inv;
-    if (fb < 0.f || fa > (float)g.nx) return;
     const int i0 = max(0, min(g.nx - 1, (int)fa)), i1 = min(g.nx - 1, max(0, (int)fb));
     p0 = __ldca(start + j * g.nx + i0);
     p1 = __ldca(start + j * g.nx + i1 + 1);
