@@ -346,7 +346,7 @@ extern "C" int exact_sdf_batch(exact_ctx *ctx, const float *points, const uint8_
     if ((long long)n_poses * chunks > 0x7fffffffLL) chunks = 1;
     // (always so from one pose per SM on)
     const bool cluster = chunks > 1 && chunks <= kSdfCluster && (dmin || argmin);
-    if (cluster) chunks = chunks > 4 ? 8 : chunks > 2 ? 4 : 2;
+    if (cluster) chunks = chunks > 5 ? 8 : chunks > 2 ? 4 : 2;   // the nearest power of two
     const int chunk_pairs = (npairs + chunks - 1) / chunks;
     const int vec = dist && (n_points % 2 == 0) && (((uintptr_t)dist & 7u) == 0);
 

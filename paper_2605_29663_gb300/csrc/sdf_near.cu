@@ -573,18 +573,25 @@ sdf_min_kernel(const SortedChunk *__restrict__ chunks, int N, int csize, const f
 // ---------------------------------------------------------------- launches
 // Where the sort (a launch of about 12 us) pays.  Matrix: a patch costs the
 // pruned kernel a search, the transform, the root and the store whatever the
-// number of edges, about what 14 edges cost the general one (4,096 poses x
-// 8,192 points: 12 edges 166 against 157 us, 16 edges 173 against 179, 24
-// edges 187 against 249, 64 edges 288 against 568), and patches of a few
-// thousand points are too wide to leave edges out (8,192 x 1,024 points, 32
-// edges: 132 against 92 us).  Minimum: general calls from about 45 us on.
-constexpr int kMinPoses = 256, kMinPoints = 2 * kPatch, kMatrixPoses = 64, kMatrixPoints = 4096;
+// number of edges, about what 14 edges cost the general one, and patches of few
+// points are too wide to leave edges out: from 16 edges and 8,192 points, or 32
+// and 4,096, on (4,096 poses x 8,192 points: 12 edges 166 us against 157 with the
+// general kernel, 16 edges 171 against 178, 24 edges 187 against 252, 64 edges 288
+// against 568; 16 edges x 4,096 points 112 against 94).  A cloud dense on the
+// footprint keeps most edges and still gains (within 0.3 m of the origin: 16
+// edges 279 against 284, 32 edges 392 against 478).  Minimum: general calls from
+// about 45 us on, of 1,024 points (200,000 poses x 128 points lost up to 17 %); a
+// cover's general evaluation is so cheap that it takes 768 poses (256 poses x
+// 300,000 points, 3 boxes: 179 against 125 us).  It loses where nearly every patch
+// can hold the minimum: points all at one place 2.3x, on a circle about every
+// pose 1.5x, all inside the footprint 1.2x.
+constexpr int kMinPoses = 256, kMinPoints = 1024, kMatrixPoses = 64, kMatrixPoints = 4096;
 bool sdf_near_fits(const exact_footprint *fp, int n_points, int n_poses, bool dist) {
-    const long long pairs = (long long)n_points * n_poses;
-    const long long work = pairs * (fp->kind == EXACT_FP_POLYGON ? fp->n_pad : 2 * fp->n_pad);
-    if (!dist) return n_poses >= kMinPoses && n_points >= kMinPoints && work >= (1ll << 27);
-    return fp->kind == EXACT_FP_POLYGON && fp->n_pad >= 16 && n_points >= kMatrixPoints && n_poses >= kMatrixPoses &&
-           work >= (1ll << 28);
+    const bool polygon = fp->kind == EXACT_FP_POLYGON;
+    const long long pairs = (long long)n_points * n_poses, work = pairs * (polygon ? fp->n_pad : 2 * fp->n_pad);
+    if (!dist) return n_poses >= (polygon ? kMinPoses : 3 * kMinPoses) && n_points >= kMinPoints && work >= (1ll << 27);
+    return polygon && fp->n_pad >= 16 && n_points >= kMatrixPoints && (long long)n_points * fp->n_pad >= 16 * 8192 &&
+           n_poses >= kMatrixPoses && work >= (1ll << 28);
 }
 bool sdf_near_possible(int n_points, int n_poses) {
     if ((long long)n_points * n_poses < (1ll << 27) / EXACT_MAX_POLY_VERTICES) return false;

@@ -126,3 +126,17 @@ def test_sdf_pruned_with_points_far_away(ex, at, share, N, dist):  # noqa: F811
     (d0, m0, a0), (d1, m1, a1) = _both(ex, pts, poses, synth.POLYGON, synth.star_polygon(g, 32, 0.3, 1.2), None, dist)
     assert d0 is None or bool((d0 == d1).all())
     assert bool((m0 == m1).all()) and bool((a0 == a1).all())
+
+
+@pytest.mark.parametrize("E,N,P,dist", [(16, 8191, 2100, True), (16, 8192, 2100, True), (24, 5461, 2200, True), (24, 5462, 2200, True),
+                                        (32, 4095, 2200, True), (32, 4096, 2200, True), (12, 1023, 11_000, False),
+                                        (12, 1024, 11_000, False), (0, 70_000, 767, False), (0, 70_000, 768, False)])
+def test_sdf_on_both_sides_of_the_pruned_paths_lines(ex, E, N, P, dist):  # noqa: F811
+    """E = 0: the rectangle cover."""
+    g = synth.rng(N + P)
+    pts = g.uniform(-6, 6, (N, 2)).astype(np.float32)
+    poses = np.concatenate([g.uniform(-5, 5, (P, 2)), g.uniform(-3, 3, (P, 1))], 1).astype(np.float32)
+    kind, fp = (synth.POLYGON, synth.star_polygon(g, E, 0.3, 1.2)) if E else FOOTPRINTS["forklift"]
+    (d0, m0, a0), (d1, m1, a1) = _both(ex, pts, poses, kind, fp, None, dist)
+    assert d0 is None or bool((d0 == d1).all())
+    assert bool((m0 == m1).all()) and bool((a0 == a1).all())
