@@ -18,7 +18,7 @@
 // many points lie inside the footprints, else the latency of one sample's
 // rollout, walk and evaluation.  Measured against sub-chunk circles over a
 // Morton-ordered copy (cycle times, the nominal driven to where the samples
-// touch obstacles): forklift K = 2,048, T = 40, N = 4,096 124 -> 82 us; hybrid
+// touch obstacles): forklift K = 2,048, T = 40, N = 4,096 120 to 135 -> 82 to 94 us; hybrid
 // 3 x K = 1,024, N = 2,048 73 -> 41 us; 64 scenes of up to 20,000 points 6.47 ->
 // 1.28 ms; predicted K = 1,024, N = 2,048 57 -> 27 us.  One warp per sample was
 // slower than a block's warps sharing its samples (the forklift's near points

@@ -1031,9 +1031,7 @@ __device__ __forceinline__ void sample_body(const SceneView &V, const EV &ev, in
             }
         }
         if (lane == 0) sm.term[warp] = P.w_term * guidance_dist(R.qTx, R.qTy, V.wp, V.W);
-        grid_dep_wait();   // launched early behind a cloud-ordering kernel: the cloud is ready now
     } else {
-        grid_dep_wait();
         if (!staged)
             stage_points<MOVING>(s_pts, V.pts, V.vel, V.mask, 0, n0, threadIdx.x - 32 * ns, blockDim.x - 32 * ns, &sm.bar,
                                  &sm.bar_uses, V.err);
