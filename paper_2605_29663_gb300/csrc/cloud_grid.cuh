@@ -83,8 +83,10 @@ __device__ __forceinline__ void build_grid(const float2 *__restrict__ pts, const
     float cell, inv;
     int nx, ny, ncell, rc[kGridRegs], rank[kGridRegs];   // cell, place among its points
     auto cell_of = [&](float2 p) { return cell_axis(p.y, ly, inv, ny) * nx + cell_axis(p.x, lx, inv, nx); };
-    // cells over the points (those in the window) and the counts of all; whether
-    // some cell holds more than 1/64 of them
+    int c0, c1, s, inc;   // this thread's cells, their points, the warp's prefix
+    // cells over the points (those in the window), the counts of all and the start
+    // of their prefix; whether some cell holds more than 1/64 of them (from the
+    // counts: a look at what the atomics return would wait for them)
     auto lay = [&](auto windowed) {
         constexpr bool W = decltype(windowed)::value;
         lx = ly = finf();
@@ -131,14 +133,12 @@ __device__ __forceinline__ void build_grid(const float2 *__restrict__ pts, const
         nx = min(kGridDim, (int)(w * inv) + 1);
         ny = min(kGridDim, (int)(h * inv) + 1);
         ncell = min(kCells, nx * ny);
-        bool crowded = false;
         if (inreg) {
 #pragma unroll
             for (int k = 0; k < kGridRegs; ++k)
                 if (ok[k]) {
                     rc[k] = min(ncell - 1, cell_of(rp[k]));
                     rank[k] = atomicAdd(&sm.cnt[rc[k]], 1);
-                    crowded |= rank[k] >= N / 64;
                 }
         } else {
 #pragma unroll 4
@@ -146,9 +146,26 @@ __device__ __forceinline__ void build_grid(const float2 *__restrict__ pts, const
                 float2 p, v;
                 if (fetch(i, p, v)) atomicAdd(&sm.cnt[min(ncell - 1, cell_of(p))], 1);
             }
-            __syncthreads();
-            for (int c = tid; c < ncell; c += nt) crowded |= sm.cnt[c] > N / 64;
         }
+        __syncthreads();
+        // exclusive prefix over the counts: contiguous segments per thread
+        const int per = ((ncell + nt) / nt) | 1;   // odd: no bank conflicts
+        c0 = tid * per;
+        c1 = min(ncell + 1, c0 + per);
+        bool crowded = false;
+        s = 0;
+        for (int c = c0; c < c1; ++c) {
+            const int n = sm.cnt[c];
+            s += n;
+            crowded |= n > N / 64;
+        }
+        inc = s;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += t;
+        }
+        if (lane == 31) sm.part[warp] = inc;
         return __syncthreads_or(crowded) != 0;
     };
     int open = 0;
@@ -162,18 +179,6 @@ __device__ __forceinline__ void build_grid(const float2 *__restrict__ pts, const
             open = 1;
             if (!lay(std::true_type{})) break;
         }
-    // exclusive prefix over the counts: contiguous segments per thread
-    const int per = ((ncell + nt) / nt) | 1, c0 = tid * per, c1 = min(ncell + 1, c0 + per);   // odd: no bank conflicts
-    int s = 0;
-    for (int c = c0; c < c1; ++c) s += sm.cnt[c];
-    int inc = s;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += t;
-    }
-    if (lane == 31) sm.part[warp] = inc;
-    __syncthreads();
     {   // the totals of the warps below, again by every warp itself
         int v = lane < warp ? sm.part[lane] : 0;
 #pragma unroll
